@@ -11,6 +11,7 @@
 // associative, so the diagonal is bit-for-bit independent of scheduling.
 #include "internal.h"
 
+#include <algorithm>
 #include <mutex>
 
 namespace hpmxp {
@@ -61,27 +62,64 @@ __device__ inline double u128_to_f64(unsigned long long hi, unsigned long long l
   return d * __longlong_as_double((long long)(1023 + 64 - sh) << 52);
 }
 
-constexpr int kRows = 128;      // rows per CTA (one per thread)
-constexpr int kChunk = 512;     // columns per CTA; 512 * 2^52 < 2^64
+// |q| from a state: q = t - 2^52 with t = (s >> 11) | 1 (53 bits), so a set
+// top bit of s means q = t without that bit, and a clear one q = -(2^52 - t),
+// whose magnitude is t's low 52 bits inverted with the last bit (1) kept.
+__device__ inline uint64_t state_absq(uint64_t s) {
+  const uint64_t flip = (uint64_t)(~((int64_t)s >> 63));
+  return (((s ^ flip) & 0x7fffffffffffffffull) >> 11) | 1ull;
+}
+// The bit pattern of q 2^-53 from |q| and the state: the 52-bit integer is
+// normalised by its leading one (bit 52 - L) and lands in the fraction field
+// with its leading one added to the exponent 1021 - L.  Integer operations
+// only: the fp64 unit does 2 operations per clock and SM, so the conversion
+// and the scaling there took longer than writing the matrix.
+__device__ inline double absq_value(uint64_t m, uint64_t s) {
+  const uint32_t hi = (uint32_t)(m >> 32);   // 20 bits
+  if (hi == 0) return (int64_t)s < 0 ? (double)m * 0x1p-53 : (double)m * -0x1p-53;   // 1 draw in 2^20
+  const int L = __clz((int)hi) - 11;         // leading one at bit 52 - L of m, L >= 1
+  const uint64_t f = (m << L) + ((uint64_t)(1021 - L) << 52);
+  return __longlong_as_double((long long)(f | (~s & 0x8000000000000000ull)));
+}
 
-// Phase 1: values of A for a 128-row x 512-column tile, per-row partial sums
-// of the off-diagonal |q| into the 128-bit accumulators sums[2i], sums[2i+1].
+constexpr int kRows = 128;      // rows per CTA (one per thread)
+constexpr int kChunk = 512;     // most columns per CTA; 512 * 2^52 < 2^64
+
+// Columns per CTA.  A long chunk amortises the skip-ahead of its first state
+// (about 30 doublings); a small matrix takes shorter ones, down to 32 columns,
+// until there are about 8 CTAs per SM, since a chunk is one serial chain of
+// LCG steps (n = 1024: 45 us of chain at 512 columns).
+int gen_chunk(int64_t n) {
+  const int64_t rb = cdiv<int64_t>(n, kRows);
+  int64_t c = kChunk;
+  while (c > 32 && rb * cdiv<int64_t>(n, c) < 8 * 152) c /= 2;
+  return (int)c;
+}
+
+// Phase 1: values of A for a 128-row x `chunk`-column tile, per-row partial
+// sums of the off-diagonal |q| into the 128-bit accumulators sums[2i],
+// sums[2i+1].  About 25 integer instructions and 8 written bytes per entry (a
+// warp's 256 bytes of one column per store); n = 16384: 449 us per call, 4.8
+// TB/s written, against 973 us with (double)q * 2^-53 on the fp64 unit.
 __global__ void __launch_bounds__(kRows) gen_matrix_kernel(int64_t n, uint64_t seed, double* A,
                                                            int64_t lda, unsigned long long* sums,
-                                                           Affine stride_n) {
+                                                           Affine stride_n, int chunk) {
   const int64_t i = (int64_t)blockIdx.x * kRows + threadIdx.x;
-  const int64_t j0 = (int64_t)blockIdx.y * kChunk;
+  const int64_t j0 = (int64_t)blockIdx.y * chunk;
   if (i >= n) return;
-  const int64_t j1 = min(j0 + (int64_t)kChunk, n);
+  const int64_t j1 = min(j0 + (int64_t)chunk, n);
   const Affine start = lcg_power((uint64_t)(i + j0 * n) + 1);
   uint64_t s = start.a * seed + start.c;
   unsigned long long part = 0;
   double* col = A + i + j0 * lda;
-  for (int64_t j = j0; j < j1; ++j) {
-    const int64_t q = state_q(s);
-    *col = q_value(q);
+  const int cnt = (int)(j1 - j0);
+  const int jd = i >= j0 && i < j1 ? (int)(i - j0) : -1;   // this row's diagonal entry within the chunk
+#pragma unroll 4
+  for (int jj = 0; jj < cnt; ++jj) {
+    const uint64_t m = state_absq(s);
+    *col = absq_value(m, s);
     col += lda;
-    if (j != i) part += (unsigned long long)(q < 0 ? -q : q);
+    if (jj != jd) part += m;
     s = stride_n.a * s + stride_n.c;
   }
   if (part) atomic_add_u128(sums + 2 * i, part);
@@ -135,8 +173,9 @@ cudaError_t launch_generate(int64_t n, uint64_t seed, double margin, int mode, d
   cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * 2 * (size_t)n, st);
   if (e != cudaSuccess) return e;
   const Affine stride = lcg_power((uint64_t)n);
-  dim3 grid((unsigned)cdiv<int64_t>(n, kRows), (unsigned)cdiv<int64_t>(n, kChunk));
-  gen_matrix_kernel<<<grid, kRows, 0, st>>>(n, seed, A, lda, sums, stride);
+  const int chunk = gen_chunk(n);
+  dim3 grid((unsigned)cdiv<int64_t>(n, kRows), (unsigned)cdiv<int64_t>(n, chunk));
+  gen_matrix_kernel<<<grid, kRows, 0, st>>>(n, seed, A, lda, sums, stride, chunk);
   gen_diag_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, seed, margin, mode, A, lda, sums);
   if (nrhs > 0) {
     const int64_t work = cdiv<int64_t>(n, 64) * nrhs;
