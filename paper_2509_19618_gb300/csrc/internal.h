@@ -146,6 +146,10 @@ struct GemmArgs {
 cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st);
 cudaError_t gemm_simt(const GemmArgs& g, cudaStream_t st);
 
+// Tensor map of a column-major fp64 matrix (rows x cols, 16-byte aligned
+// columns), boxes of box_rows x box_cols, no swizzle, zeros outside.
+bool encode_f64_map(CUtensorMap* tm, const double* base, int64_t rows, int64_t cols, int64_t ld, int box_rows,
+                    int box_cols);
 // Grouped launches of the tensor-core engine: several independent products of
 // the same kind (same mode, sign, format and K, 16-bit operands, K < 256 so
 // all take 128-row tiles, R given for all or none) in ONE launch, the
@@ -188,6 +192,34 @@ hpmxp_status factor(int64_t n, const double* A, int64_t lda, int prec, int nb, v
 cudaError_t lu_f64(int64_t n, double* A, int64_t ld, uint32_t* status, cudaStream_t st);
 cudaError_t lu_solve_f64(int64_t n, const double* LU, int64_t ld, double* X, int64_t ldx, int64_t nrhs,
                          cudaStream_t st);
+
+// gemv_tc.cu: fp64 products A X (K <= 8 columns) from exact digit products on
+// the tensor cores, for the refinement's kernels in ir.cu.
+// The work is cut evenly: the 512-row tiles' lists of `blocks` 64-column
+// blocks, concatenated, in `ctas` contiguous ranges; a tile's sums come in
+// one piece per range that meets it.
+constexpr int kGemvTileRows = 512;
+struct GemvSplit {
+  int blocks = 0, total = 0, ctas = 0;   // ctas 0: not split this way
+  __host__ __device__ int begin(int cta) const { return (int)((long long)cta * total / ctas); }
+  // the first range that holds part of tile's list [tile * blocks, (tile + 1) * blocks)
+  __host__ __device__ int first_cta(int tile) const { return cta_of(tile * blocks); }
+  __host__ __device__ int pieces(int tile) const { return cta_of((tile + 1) * blocks - 1) - first_cta(tile) + 1; }
+  __host__ __device__ int cta_of(int q) const {
+    int c = (int)((long long)q * ctas / total);
+    while (begin(c + 1) <= q) ++c;
+    return c;
+  }
+};
+// The split for order n; false where a tile could meet more than max_pieces
+// ranges, or A's columns are not 16-byte aligned.
+bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, GemvSplit* split);
+// P[c][r][i] = the partial sums of row i in its tile's piece c; with abs_sums
+// also RS[c][i], the fp32 estimates of the |A| row sums.  prep: gemv_tc_bytes(n)
+// of scratch, 16-byte aligned.
+size_t gemv_tc_bytes(int64_t n);
+cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
+                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st);
 
 // ir.cu
 size_t solve_batched_ws_bytes(const hpmxp_problem* probs, int count, int restart);

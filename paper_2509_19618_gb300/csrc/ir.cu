@@ -253,43 +253,58 @@ __global__ void __launch_bounds__(kGemvThreads) gemv32_partial_kernel(int64_t n,
 // out(i, r) = B(i, r) - sum_c P[c](i, r), or + sum_c P[c](i, r) when B is NULL
 // (chunks in order); max-reduces
 // |out|, |X| (when xn) and the row sums (when abs_mode) into the states.
-__global__ void gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P,
-                                   const double* __restrict__ B, int64_t ldb, double* __restrict__ out,
-                                   int64_t ldo, const double* __restrict__ X, int64_t ldx, int abs_mode,
-                                   const void* __restrict__ RS, RhsState* st, int track_norms) {
+// One right-hand side per grid row; a warp's maxima by shuffles, one atomic per
+// warp and maximum.
+__device__ inline unsigned long long warp_max(unsigned long long v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__global__ void __launch_bounds__(256) gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P,
+                                                          const double* __restrict__ B, int64_t ldb,
+                                                          double* __restrict__ out, int64_t ldo,
+                                                          const double* __restrict__ X, int64_t ldx, int abs_mode,
+                                                          const void* __restrict__ RS, RhsState* st, int track_norms,
+                                                          GemvSplit split) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  __shared__ unsigned long long smax[3 * kMaxK + 1];
-  if (threadIdx.x < 3 * kMaxK + 1) smax[threadIdx.x] = 0;
-  __syncthreads();
-  if (i < n) {
-    for (int r = 0; r < K; ++r) {
-      double s = 0.0;
-      for (int c = 0; c < nchunk; ++c) s += P[(int64_t)c * n * K + i + r * n];
-      const double v = B ? B[i + r * ldb] - s : s;
-      out[i + r * ldo] = v;
-      if (track_norms) {
-        atomicMax(&smax[r], dbits(fabs(v)));
-        atomicMax(&smax[kMaxK + r], dbits(fabs(X[i + r * ldx])));
-        if (B) atomicMax(&smax[2 * kMaxK + r], dbits(fabs(B[i + r * ldb])));
+  const int r = blockIdx.y;
+  if (split.ctas) nchunk = split.pieces((int)(min(i, n - 1) / kGemvTileRows));   // the tile's own count
+  const bool in = i < n;
+  double v = 0.0;
+  if (in) {
+    double s = 0.0;
+    const double* p = P + i + r * n;
+#pragma unroll 4
+    for (int c = 0; c < nchunk; ++c, p += n * K) s += *p;
+    v = B ? B[i + r * ldb] - s : s;
+    out[i + r * ldo] = v;
+  }
+  if (!track_norms) return;
+  const bool lead = (threadIdx.x & 31) == 0;
+  const unsigned long long rn = warp_max(dbits(fabs(v)));
+  const unsigned long long xn = warp_max(in ? dbits(fabs(X[i + r * ldx])) : 0ull);
+  if (lead) {
+    atomicMax(&st[r].rn_bits, rn);
+    atomicMax(&st[r].xn_bits, xn);
+  }
+  if (B) {
+    const unsigned long long bn = warp_max(in ? dbits(fabs(B[i + r * ldb])) : 0ull);
+    if (lead) atomicMax(&st[r].bn_bits, bn);
+  }
+  if (abs_mode && r == 0) {
+    double s = 0.0;
+    if (in) {
+      if (abs_mode == 1) {
+        float f = 0.0f;
+        for (int c = 0; c < nchunk; ++c) f += ((const float*)RS)[(int64_t)c * n + i];
+        s = (double)f;
+      } else {
+        for (int c = 0; c < nchunk; ++c) s += ((const double*)RS)[(int64_t)c * n + i];
       }
     }
-    if (abs_mode == 1) {
-      float s = 0.0f;
-      for (int c = 0; c < nchunk; ++c) s += ((const float*)RS)[(int64_t)c * n + i];
-      atomicMax(&smax[3 * kMaxK], dbits((double)s));
-    } else if (abs_mode == 2) {
-      double s = 0.0;
-      for (int c = 0; c < nchunk; ++c) s += ((const double*)RS)[(int64_t)c * n + i];
-      atomicMax(&smax[3 * kMaxK], dbits(s));
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < K && track_norms) {
-    const int r = threadIdx.x;
-    atomicMax(&st[r].rn_bits, smax[r]);
-    atomicMax(&st[r].xn_bits, smax[kMaxK + r]);
-    if (B) atomicMax(&st[r].bn_bits, smax[2 * kMaxK + r]);
-    if (abs_mode) atomicMax(&st[r].an_bits, smax[3 * kMaxK]);
+    const unsigned long long an = warp_max(dbits(s));
+    if (lead)
+      for (int k = 0; k < K; ++k) atomicMax(&st[k].an_bits, an);
   }
 }
 
@@ -1125,27 +1140,51 @@ cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int
   return cudaGetLastError();
 }
 
+// Which products go to the tensor cores (gemv_tc.cu): fp64 ones that do not
+// also copy A to fp32, from the order at which two launches for X's digits and
+// 226 KB of shared memory per SM pay.  Both kernels timed, microseconds, digit
+// products / fp64 FMAs: one right-hand side 30 / 26 at n = 2048, 53 / 57 at 4096,
+// 121 / 131 at 8192, 1570 / 1777 at 32768; two 34 / 25 at 1536, 31 / 35 at 2048,
+// 125 / 239 at 8192; six 35 / 38 at 1024; eight 155 / 885 at 8192, 1860 / 13800 at 32768.
+bool gemv_on_tensor_cores(int64_t n, int K, const double* A, int64_t lda, int abs_mode, const SolveWs& w,
+                          GemvSplit* split) {
+  const int64_t min_n = K == 1 ? 4096 : K < 6 ? 2048 : 1024;
+  if (!(abs_mode == 0 || (abs_mode == 1 && !w.a32)) || n < min_n) return false;
+  const size_t cap = (size_t)gemv_chunks(n);
+  if (round_up<size_t>(sizeof(float) * cap * n, 256) + gemv_tc_bytes(n) > sizeof(double) * cap * n) return false;
+  GemvSplit s;
+  if (!gemv_tc_split(n, A, lda, (int)cap, &s)) return false;
+  *split = s;
+  return true;
+}
+
 // out = b - A X (b may be NULL: out = -A X), with optional norm tracking.
 cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx,
                      const double* B, int64_t ldb, double* out, int64_t ldo, int abs_mode, int track,
                      const SolveWs& w, cudaStream_t st) {
-  const int nchunk = gemv_chunks(n, K);
+  int nchunk = gemv_chunks(n, K);
   cudaError_t e;
   void* tok = prof_begin(st);
-  switch (K) {
-    case 1: e = gemv_k<1>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-    case 2: e = gemv_k<2>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-    case 3: e = gemv_k<3>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-    case 4: e = gemv_k<4>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-    case 5: e = gemv_k<5>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-    case 6: e = gemv_k<6>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-    case 7: e = gemv_k<7>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-    default: e = gemv_k<8>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+  GemvSplit split;
+  if (gemv_on_tensor_cores(n, K, A, lda, abs_mode, w, &split)) {
+    // the digits live in the upper half of the row-sum scratch (fp64-sized; mode 1 keeps fp32 sums)
+    void* prep = (char*)w.RS + round_up<size_t>(sizeof(float) * (size_t)gemv_chunks(n) * n, 256);
+    e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st);
+  } else {
+    switch (K) {
+      case 1: e = gemv_k<1>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      case 2: e = gemv_k<2>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      case 3: e = gemv_k<3>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      case 4: e = gemv_k<4>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      case 5: e = gemv_k<5>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      case 6: e = gemv_k<6>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      case 7: e = gemv_k<7>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      default: e = gemv_k<8>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+    }
   }
   if (e != cudaSuccess) return e;
-  gemv_finish_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx,
-                                                                      abs_mode == 3 ? 0 : abs_mode, w.RS, w.st,
-                                                                      track);
+  gemv_finish_kernel<<<dim3((unsigned)cdiv<int64_t>(n, 256), K), 256, 0, st>>>(
+      n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split);
   prof_end(tok, abs_mode == 3 ? kProfGemv32 : kProfGemv, 8.0 * (double)n * (double)n, st);
   count_launches(2);
   return cudaGetLastError();
@@ -1676,7 +1715,7 @@ hpmxp_status residual_vector(int64_t n, const double* A, int64_t lda, const doub
                              const double* b, int64_t ldb, int64_t nrhs, double* r, int64_t ldr, void* ws,
                              cudaStream_t st) {
   SolveWs w = carve_solve(ws, n, nrhs, 1);
-  cudaError_t e = cudaMemsetAsync(w.st, 0, sizeof(RhsState) * kMaxK, st);
+  cudaError_t e = cudaMemsetAsync(w.status, 0, 4, st);
   if (e == cudaSuccess) e = residual(n, (int)nrhs, A, lda, x, ldx, b, ldb, r, ldr, 0, 0, w, st);
   return status_from_cuda(e);
 }
