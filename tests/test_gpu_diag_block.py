@@ -27,10 +27,13 @@ def _matrix(n, kind):
     elif kind == "ones":         # pivots start at BF16's all-ones significand; lower triangular
         A[np.arange(n), np.arange(n)] = 255.0 * 2.0**-7
         A -= np.triu(A, 1) + np.tril(A, -1) * (1 - 2.0**-9)
+    elif kind == "below_pow2":   # pivots one fp32 ulp below a power of two
+        A = np.abs(A) * 0.5
+        A[np.arange(n), np.arange(n)] = 2048.0
     return np.asfortranarray(A)
 
 
-@pytest.mark.parametrize("kind", ["plain", "zeros", "tiny", "graded", "ones"])
+@pytest.mark.parametrize("kind", ["plain", "zeros", "tiny", "graded", "ones", "below_pow2"])
 @pytest.mark.parametrize("n", [1, 16, 17, 40, 128, 200, 300])
 def test_diagonal_block_bit_exact(n, kind, monkeypatch):
     A_o = _matrix(n, kind)
