@@ -253,57 +253,54 @@ __global__ void __launch_bounds__(kGemvThreads) gemv32_partial_kernel(int64_t n,
 // out(i, r) = B(i, r) - sum_c P[c](i, r), or + sum_c P[c](i, r) when B is NULL
 // (chunks in order); max-reduces
 // |out|, |X| (when xn) and the row sums (when abs_mode) into the states.
-// One right-hand side per grid row; a warp's maxima by shuffles, one atomic per
-// warp and maximum.
+// One right-hand side per grid row; eight threads share a row's chunks (a small
+// system's few rows would otherwise wait for each load in turn: 6.0 us at n =
+// 1024, 67 us at 8192 with eight right-hand sides) and are summed in order; the
+// rows' maxima by shuffles, one atomic per CTA and maximum.
 __device__ inline unsigned long long warp_max(unsigned long long v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   return v;
 }
-__global__ void __launch_bounds__(256) gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P,
-                                                          const double* __restrict__ B, int64_t ldb,
-                                                          double* __restrict__ out, int64_t ldo,
-                                                          const double* __restrict__ X, int64_t ldx, int abs_mode,
-                                                          const void* __restrict__ RS, RhsState* st, int track_norms,
-                                                          GemvSplit split) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+constexpr int kFinRows = 32, kFinGroups = 8;   // rows of a CTA, threads that share a row's pieces
+__global__ void __launch_bounds__(kFinRows * kFinGroups)
+gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P, const double* __restrict__ B,
+                   int64_t ldb, double* __restrict__ out, int64_t ldo, const double* __restrict__ X, int64_t ldx,
+                   int abs_mode, const void* __restrict__ RS, RhsState* st, int track_norms, GemvSplit split) {
+  __shared__ double sh[2][kFinGroups][kFinRows];
+  const int tx = threadIdx.x % kFinRows, ty = threadIdx.x / kFinRows;
+  const int64_t i = (int64_t)blockIdx.x * kFinRows + tx;
   const int r = blockIdx.y;
+  const bool in = i < n, rows_too = track_norms && abs_mode && r == 0;
   if (split.ctas) nchunk = split.pieces((int)(min(i, n - 1) / kGemvTileRows));   // the tile's own count
-  const bool in = i < n;
-  double v = 0.0;
+  double s = 0.0, a = 0.0;
   if (in) {
-    double s = 0.0;
-    const double* p = P + i + r * n;
-#pragma unroll 4
-    for (int c = 0; c < nchunk; ++c, p += n * K) s += *p;
-    v = B ? B[i + r * ldb] - s : s;
-    out[i + r * ldo] = v;
+    for (int c = ty; c < nchunk; c += kFinGroups) s += P[((int64_t)c * K + r) * n + i];
+    if (rows_too)
+      for (int c = ty; c < nchunk; c += kFinGroups)
+        a += abs_mode == 1 ? (double)((const float*)RS)[(int64_t)c * n + i] : ((const double*)RS)[(int64_t)c * n + i];
   }
+  sh[0][ty][tx] = s;
+  sh[1][ty][tx] = a;
+  __syncthreads();
+  if (ty != 0) return;
+#pragma unroll
+  for (int g = 1; g < kFinGroups; ++g) {
+    s += sh[0][g][tx];
+    a += sh[1][g][tx];
+  }
+  const double v = B && in ? B[i + r * ldb] - s : s;
+  if (in) out[i + r * ldo] = v;
   if (!track_norms) return;
-  const bool lead = (threadIdx.x & 31) == 0;
-  const unsigned long long rn = warp_max(dbits(fabs(v)));
+  const unsigned long long rn = warp_max(in ? dbits(fabs(v)) : 0ull);
   const unsigned long long xn = warp_max(in ? dbits(fabs(X[i + r * ldx])) : 0ull);
-  if (lead) {
+  const unsigned long long bn = B ? warp_max(in ? dbits(fabs(B[i + r * ldb])) : 0ull) : 0ull;
+  const unsigned long long an = rows_too ? warp_max(dbits(a)) : 0ull;
+  if (tx == 0) {
     atomicMax(&st[r].rn_bits, rn);
     atomicMax(&st[r].xn_bits, xn);
-  }
-  if (B) {
-    const unsigned long long bn = warp_max(in ? dbits(fabs(B[i + r * ldb])) : 0ull);
-    if (lead) atomicMax(&st[r].bn_bits, bn);
-  }
-  if (abs_mode && r == 0) {
-    double s = 0.0;
-    if (in) {
-      if (abs_mode == 1) {
-        float f = 0.0f;
-        for (int c = 0; c < nchunk; ++c) f += ((const float*)RS)[(int64_t)c * n + i];
-        s = (double)f;
-      } else {
-        for (int c = 0; c < nchunk; ++c) s += ((const double*)RS)[(int64_t)c * n + i];
-      }
-    }
-    const unsigned long long an = warp_max(dbits(s));
-    if (lead)
+    if (B) atomicMax(&st[r].bn_bits, bn);
+    if (rows_too)
       for (int k = 0; k < K; ++k) atomicMax(&st[k].an_bits, an);
   }
 }
@@ -332,48 +329,107 @@ template <> __device__ inline float u16_to<float>(uint16_t h, int fmt) { return 
 template <> __device__ inline double u16_to<double>(uint16_t h, int fmt) { return u16_to_f64(h, fmt); }
 
 // Inverse of diagonal block c (c < nb) of the unit-lower L (which == 0) or of
-// U (which == 1) in T arithmetic, from the 16-bit factors: one thread per
-// column, column-oriented substitution.  Output inv[(which * nb + c) * 128 *
-// 128 + j * 128 + i] = inverse(i, j).
+// U (which == 1) in T arithmetic, from the 16-bit factors.  Output inv[(which *
+// nb + c) * 128 * 128 + j * 128 + i] = inverse(i, j).  A CTA makes 32 columns
+// (grid z), one per lane: row by row, the finished row's term is added to the
+// rows still open, which are dealt out to the warps and kept in registers, so
+// that the FMAs between two barriers are independent.  Bound by the 128 steps'
+// latency (fp32) and the fp64 unit, where a warp's FMA takes 64 clocks of its
+// scheduler (fp64).  46 us in fp32 at n = 1024 and 210 us at 32768, 239 us in
+// fp64 at 4096; one thread per column, a chain of dependent FMAs on one SM per
+// block, took 80, 328 and 667 us.
+constexpr int kInvCols = 32, kInvPitch = kInvCols + 1, kInvThreads = 256;
 template <class T>
-__global__ void __launch_bounds__(128) diag_inv_kernel(int64_t n, const uint16_t* __restrict__ LU, int64_t ld,
-                                                       int fmt, T* __restrict__ inv) {
+__device__ inline T quotient(T s, T d, T r);   // s / d with r = 1 / d
+template <>
+__device__ inline float quotient<float>(float s, float d, float r) { return __fdiv_rn(s, d); }
+// one correction of s * r: the plain fp64 division costs about ten fp64 instructions
+template <>
+__device__ inline double quotient<double>(double s, double d, double r) {
+  const double q = s * r;
+  const double x = __fma_rn(__fma_rn(-q, d, s), r, q);
+  return isfinite(x) ? x : s / d;   // (a subnormal or infinite r)
+}
+template <class T>
+__global__ void __launch_bounds__(kInvThreads) diag_inv_kernel(int64_t n, const uint16_t* __restrict__ LU, int64_t ld,
+                                                               int fmt, T* __restrict__ inv) {
   extern __shared__ __align__(16) unsigned char dsm_raw[];
-  float* t = reinterpret_cast<float*>(dsm_raw);                         // t[j * 129 + i] = block(i, j)
-  T* x = reinterpret_cast<T*>(dsm_raw + sizeof(float) * kTB32 * 130);   // x[j * 129 + i] = inverse(i, j)
+  T* t = reinterpret_cast<T*>(dsm_raw);      // t[k * 128 + i] = block(i, k)
+  T* x = t + kTB32 * kTB32;                  // x[i * kInvPitch + lane] = inverse(i, j0 + lane) when row i is done
+  T* dg = x + kTB32 * kInvPitch;             // U's diagonal and its reciprocals
+  T* rd = dg + kTB32;
   const int nb = (int)cdiv<int64_t>(n, kTB32);
-  const int c = blockIdx.x, which = blockIdx.y, tid = threadIdx.x;
+  const int c = blockIdx.x, j0 = blockIdx.z * kInvCols, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool upper = blockIdx.y == 1;
   const int64_t base = (int64_t)c * kTB32;
-  for (int idx = tid; idx < kTB32 * kTB32; idx += 128) {
-    const int i = idx % kTB32, j = idx / kTB32;
-    const bool in = base + i < n && base + j < n;
-    t[j * 129 + i] = in ? u16_to_f32(LU[base + i + (base + j) * ld], fmt) : (i == j ? 1.0f : 0.0f);
+  // the part of the block these columns need: rows and columns j0 .. 127 of L, 0 .. j0 + 31 of U
+  const int lo = upper ? 0 : j0, hi = upper ? j0 + kInvCols : kTB32;
+  // 16-byte loads, all in flight (the columns are 16-byte aligned and padded to 8 rows)
+  uint4 raw[kTB32 * kTB32 / 8 / kInvThreads];
+#pragma unroll
+  for (int q = 0; q < kTB32 * kTB32 / 8 / kInvThreads; ++q) {
+    const int chunk = tid + q * kInvThreads, k = chunk >> 4, i = (chunk & 15) * 8;
+    raw[q] = make_uint4(0, 0, 0, 0);
+    if (i + 8 > lo && i < hi && k >= lo && k < hi && base + k < n && base + i < n)
+      raw[q] = *reinterpret_cast<const uint4*>(LU + base + i + (base + k) * ld);
+  }
+#pragma unroll
+  for (int q = 0; q < kTB32 * kTB32 / 8 / kInvThreads; ++q) {
+    const int chunk = tid + q * kInvThreads, k = chunk >> 4, i0 = (chunk & 15) * 8;
+    const uint32_t w[4] = {raw[q].x, raw[q].y, raw[q].z, raw[q].w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int i = i0 + e;
+      const bool in = base + i < n && base + k < n;
+      const T v = in ? u16_to<T>((uint16_t)(w[e >> 1] >> (16 * (e & 1))), fmt) : (T)0;
+      // the strict triangle only, zeros elsewhere: a finished row's term is then a no-op for
+      // the rows that are closed; U's diagonal apart
+      t[k * kTB32 + i] = (upper ? i < k : i > k) ? v : (T)0;
+      if (upper && i == k) dg[i] = in ? v : (T)1;
+    }
   }
   __syncthreads();
-  const int j = tid;   // column of the inverse
-  if (which == 0) {    // L X = I, unit lower: X(i, j) = -sum_{k=j}^{i-1} L(i, k) X(k, j)
-    for (int i = 0; i < kTB32; ++i) x[j * 129 + i] = i == j ? (T)1 : (T)0;
-    for (int i = j + 1; i < kTB32; ++i) {
-      T s = (T)0;
-      for (int k = j; k < i; ++k) s = fma_t<T>((T)t[k * 129 + i], x[j * 129 + k], s);
-      x[j * 129 + i] = -s;
+  if (upper && tid < kTB32) rd[tid] = (T)1 / dg[tid];
+  __syncthreads();
+  // rows warp + kWarps r of the lane's column, in registers
+  constexpr int kWarps = kInvThreads / 32, kRows = kTB32 / kWarps;
+  T acc[kRows];
+#pragma unroll
+  for (int r = 0; r < kRows; ++r) acc[r] = warp + kWarps * r == j0 + lane ? (T)1 : (T)0;
+#pragma unroll 1
+  for (int step = 0; step < hi - lo; ++step) {
+    const int k = upper ? hi - 1 - step : lo + step;
+    // row k's warp finishes and publishes it (U: divided by the diagonal)
+    if (warp == k % kWarps) {
+      T xk = (T)0;
+#pragma unroll
+      for (int r = 0; r < kRows; ++r)
+        if (k == warp + kWarps * r) xk = acc[r];
+      x[k * kInvPitch + lane] = upper ? quotient<T>(xk, dg[k], rd[k]) : xk;
     }
-  } else {             // U Y = I: Y(i, j) = (delta - sum_{k=i+1}^{j} U(i, k) Y(k, j)) / U(i, i)
-    for (int i = 0; i < kTB32; ++i) x[j * 129 + i] = (T)0;
-    x[j * 129 + j] = (T)1 / (T)t[j * 129 + j];
-    for (int i = j - 1; i >= 0; --i) {
-      T s = (T)0;
-      for (int k = i + 1; k <= j; ++k) s = fma_t<T>((T)t[k * 129 + i], x[j * 129 + k], s);
-      x[j * 129 + i] = -s / (T)t[i * 129 + i];
+    __syncthreads();
+    const T xk = -x[k * kInvPitch + lane];
+    const T* tk = t + k * kTB32 + warp;
+#pragma unroll
+    for (int g = 0; g < kRows; g += 4) {   // four rows at a time, skipped when all are closed
+      if (upper ? warp + kWarps * g >= k : warp + kWarps * (g + 3) <= k) continue;
+#pragma unroll
+      for (int r = g; r < g + 4; ++r) acc[r] = fma_t<T>(tk[kWarps * r], xk, acc[r]);
     }
   }
+  for (int idx = tid; idx < kTB32 * kInvCols; idx += kInvThreads) {   // rows outside lo .. hi - 1 are zero
+    const int i = idx / kInvCols;
+    if (i < lo || i >= hi) x[i * kInvPitch + idx % kInvCols] = (T)0;
+  }
   __syncthreads();
-  T* out = inv + ((int64_t)which * nb + c) * kTB32 * kTB32;
-  for (int idx = tid; idx < kTB32 * kTB32; idx += 128) out[idx] = x[(idx / kTB32) * 129 + idx % kTB32];
+  T* out = inv + ((int64_t)blockIdx.y * nb + c) * kTB32 * kTB32 + (int64_t)j0 * kTB32;
+  for (int idx = tid; idx < kTB32 * kInvCols; idx += kInvThreads)
+    out[idx] = x[(idx % kTB32) * kInvPitch + idx / kTB32];
 }
 
 template <class T>
-size_t diag_inv_smem() { return sizeof(float) * kTB32 * 130 + sizeof(T) * kTB32 * 129; }
+constexpr size_t diag_inv_smem() { return sizeof(T) * (kTB32 * kTB32 + kTB32 * kInvPitch + 2 * kTB32); }
+static_assert(diag_inv_smem<double>() <= 232448, "shared memory per CTA");
 
 // Chain blocks of the fp64 preconditioner, once per solve: forward
 // P_c = Linv_c L(c, c-1) (c >= 1), backward Q_c = Uinv_c U(c, c+1) (c <= nb-2),
@@ -381,36 +437,43 @@ size_t diag_inv_smem() { return sizeof(float) * kTB32 * 130 + sizeof(T) * kTB32 
 // ascending).  out[((which * nb + c) * 128 + j) * 128 + i] = P(i, j).  With
 // them the wavefront's dependent step is one product: z_{c+1} = y_{c+1} -
 // P_{c+1} z_c, y_{c+1} = Linv_{c+1} (v_{c+1} - sum_{k<c} L(c+1,k) z_k) being
-// known before z_c is.
+// known before z_c is.  Bound by the fp64 FMAs: a CTA makes 32 columns (grid z:
+// a small system fills the SMs), the tile is decoded once, and a warp stops at
+// its rows' last nonzero of the triangular inverse (the two halves take the row
+// quarters in opposite order, so that every scheduler has the same work): 1190
+// -> 173 us at n = 4096.
+constexpr int kChainCols = 32;
 __global__ void __launch_bounds__(256) chain_blocks_kernel(int64_t n, const uint16_t* __restrict__ LU, int64_t ld,
                                                            int fmt, const double* __restrict__ dinv,
                                                            double* __restrict__ out) {
-  extern __shared__ __align__(16) unsigned char cb_raw[];
-  float* tile = reinterpret_cast<float*>(cb_raw);   // tile[t * 128 + j] = T(t, j)
+  __shared__ double tile[kTB32][kChainCols];   // tile[t][j] = T(t, j0 + j)
   const int nb = (int)cdiv<int64_t>(n, kTB32);
-  const int c = blockIdx.x, which = blockIdx.y, tid = threadIdx.x;
+  const int c = blockIdx.x, which = blockIdx.y, j0 = blockIdx.z * kChainCols, tid = threadIdx.x;
   const int nbr = which == 0 ? c - 1 : c + 1;   // block column of the neighbour tile
   if (nbr < 0 || nbr >= nb) return;
-  const int64_t r0 = (int64_t)c * kTB32, c0 = (int64_t)nbr * kTB32;
-  for (int idx = tid; idx < kTB32 * kTB32; idx += 256) {
+  const int64_t r0 = (int64_t)c * kTB32, c0 = (int64_t)nbr * kTB32 + j0;
+  for (int idx = tid; idx < kTB32 * kChainCols; idx += 256) {
     const int t = idx % kTB32, j = idx / kTB32;   // coalesced over t (column major source)
     const bool in = r0 + t < n && c0 + j < n;
-    tile[t * kTB32 + j] = in ? u16_to_f32(LU[r0 + t + (c0 + j) * ld], fmt) : 0.0f;
+    tile[t][j] = in ? u16_to_f64(LU[r0 + t + (c0 + j) * ld], fmt) : 0.0;
   }
   __syncthreads();
   const double* inv = dinv + ((int64_t)which * nb + c) * kTB32 * kTB32;
-  const int i = tid % kTB32, jh = (tid / kTB32) * 64;
-  double acc[64];
+  const int half = tid / kTB32, quarter = half ? 3 - ((tid >> 5) & 3) : (tid >> 5) & 3;
+  const int i = 32 * quarter + (tid & 31), jh = half * (kChainCols / 2);
+  const int t0 = which == 0 ? 0 : 32 * quarter, t1 = which == 0 ? 32 * quarter + 32 : kTB32;
+  double acc[kChainCols / 2];
 #pragma unroll
-  for (int q = 0; q < 64; ++q) acc[q] = 0.0;
-  for (int t = 0; t < kTB32; ++t) {
+  for (int q = 0; q < kChainCols / 2; ++q) acc[q] = 0.0;
+#pragma unroll 2
+  for (int t = t0; t < t1; ++t) {
     const double a = inv[(int64_t)t * kTB32 + i];
 #pragma unroll
-    for (int q = 0; q < 64; ++q) acc[q] = __fma_rn(a, (double)tile[t * kTB32 + jh + q], acc[q]);
+    for (int q = 0; q < kChainCols / 2; ++q) acc[q] = __fma_rn(a, tile[t][jh + q], acc[q]);
   }
   double* o = out + ((int64_t)which * nb + c) * kTB32 * kTB32;
 #pragma unroll
-  for (int q = 0; q < 64; ++q) o[(int64_t)(jh + q) * kTB32 + i] = acc[q];
+  for (int q = 0; q < kChainCols / 2; ++q) o[(int64_t)(j0 + jh + q) * kTB32 + i] = acc[q];
 }
 
 // words of one published value
@@ -784,19 +847,23 @@ __global__ void __launch_bounds__(kPrecondThreads<T>) precond_kernel(int64_t n, 
 
 // ---------------------------------------------------------------------------
 // Vector kernels.  Deterministic reductions: per-thread strided partials,
-// fixed-shape block tree, per-block partials summed in order by the last CTA.
+// fixed-shape block tree, per-block partials summed the same way by the last CTA.
 // ---------------------------------------------------------------------------
+// The sum of v over the block (a multiple of 32 threads), the same for every
+// thread: warps by shuffles, then their sums by each warp.
+__device__ inline double warp_sum(double v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
 __device__ inline double block_sum(double v, double* sh) {
-  const int tid = threadIdx.x;
-  sh[tid] = v;
+  const int lane = threadIdx.x & 31;
+  v = warp_sum(v);
+  if (lane == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (tid < s) sh[tid] += sh[tid + s];
-    __syncthreads();
-  }
-  const double r = sh[0];
+  v = warp_sum(lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0);
   __syncthreads();
-  return r;
+  return v;
 }
 
 // For every rhs r that is in an active cycle: optionally w -= h_prev v_prev
@@ -805,7 +872,7 @@ __device__ inline double block_sum(double v, double* sh) {
 __global__ void __launch_bounds__(256) mgs_kernel(int64_t n, int K, int m, int j, int i, double* W, int64_t ldw,
                                                   const double* V, int64_t ldv_col, int64_t ldv_rhs,
                                                   RhsState* st, double* partials, unsigned int* counter) {
-  __shared__ double sh[256];
+  __shared__ double sh[32];
   __shared__ bool last;
   for (int r = 0; r < K; ++r) {
     const bool act = st[r].cycle_active != 0;
@@ -830,11 +897,12 @@ __global__ void __launch_bounds__(256) mgs_kernel(int64_t n, int K, int m, int j
   __syncthreads();
   if (!last) return;
   __threadfence();
-  if (threadIdx.x < K) {
-    const int r = threadIdx.x;
-    if (st[r].cycle_active) {
-      double s = 0.0;
-      for (int b = 0; b < (int)gridDim.x; ++b) s += partials[(int64_t)r * kRedBlocks + b];
+  for (int r = 0; r < K; ++r) {
+    if (!st[r].cycle_active) continue;
+    double s = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += partials[(int64_t)r * kRedBlocks + b];
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) {
       if (i <= j) st[r].H[i + j * (m + 1)] = s;
       else st[r].hn = sqrt(s);
     }
@@ -842,22 +910,22 @@ __global__ void __launch_bounds__(256) mgs_kernel(int64_t n, int K, int m, int j
   if (threadIdx.x == 0) *counter = 0;
 }
 
-// The tail of Arnoldi step j in one CTA, for systems small enough that one SM
-// streams w and the basis faster than j + 4 launches would start: modified
-// Gram-Schmidt (for i = 0 .. j, H(i, j) = <w, v_i> then w -= H(i, j) v_i, and
-// hn = ||w||), the Givens update, and v_{j+1} = w / hn.  Every entry of w sees
-// the same operations as in mgs_kernel; the dot products are summed by this
-// CTA's fixed tree instead of across CTAs.
+// The tail of Arnoldi step j, one CTA per right-hand side, for systems small
+// enough that one SM streams w and the basis faster than j + 4 launches would
+// start: modified Gram-Schmidt (for i = 0 .. j, H(i, j) = <w, v_i> then w -=
+// H(i, j) v_i, and hn = ||w||), the Givens update, and v_{j+1} = w / hn.  Every
+// entry of w sees the same operations as in mgs_kernel; the dot products are
+// summed by this CTA's fixed tree instead of across CTAs.
 __device__ void givens_rhs(const SolveParams& sp, int j, RhsState* st, Brief* brief, int r);
 constexpr int kFusedMgsThreads = 1024;
 constexpr int64_t kFusedMgsMaxElems = 16384;   // n * K at most
-__global__ void __launch_bounds__(kFusedMgsThreads) arnoldi_tail_kernel(SolveParams sp, int64_t n, int K, int m,
-                                                                        int j, double* W, int64_t ldw, double* V,
+__global__ void __launch_bounds__(kFusedMgsThreads) arnoldi_tail_kernel(SolveParams sp, int64_t n, int m, int j,
+                                                                        double* W, int64_t ldw, double* V,
                                                                         int64_t ldv_col, int64_t ldv_rhs,
                                                                         RhsState* st, Brief* brief) {
-  __shared__ double sh[kFusedMgsThreads];
-  for (int r = 0; r < K; ++r) {
-    if (!st[r].cycle_active) continue;   // the same value for every thread
+  __shared__ double sh[32];
+  const int r = blockIdx.x;
+  if (st[r].cycle_active) {   // the same value for every thread
     double* w = W + r * ldw;
     double hprev = 0.0;
     for (int i = 0; i <= j + 1; ++i) {
@@ -869,7 +937,7 @@ __global__ void __launch_bounds__(kFusedMgsThreads) arnoldi_tail_kernel(SolvePar
         if (vprev) { wt = __fma_rn(-hprev, vprev[t], wt); w[t] = wt; }
         part = vi ? __fma_rn(wt, vi[t], part) : __fma_rn(wt, wt, part);
       }
-      const double s = block_sum(part, sh);   // ends with a barrier: w's updates are visible
+      const double s = block_sum(part, sh);
       if (threadIdx.x == 0) {
         if (i <= j) st[r].H[i + j * (m + 1)] = s;
         else st[r].hn = sqrt(s);
@@ -878,21 +946,19 @@ __global__ void __launch_bounds__(kFusedMgsThreads) arnoldi_tail_kernel(SolvePar
     }
   }
   __syncthreads();
-  if ((int)threadIdx.x < K) givens_rhs(sp, j, st, brief, threadIdx.x);
+  if (threadIdx.x == 0) givens_rhs(sp, j, st, brief, r);
   __syncthreads();
-  for (int r = 0; r < K; ++r) {
-    if (!st[r].cycle_active) continue;
-    const double hn = st[r].hn;
-    const double* w = W + r * ldw;
-    double* v = V + r * ldv_rhs + (int64_t)(j + 1) * ldv_col;
-    for (int64_t t = threadIdx.x; t < n; t += kFusedMgsThreads) v[t] = w[t] / hn;
-  }
+  if (!st[r].cycle_active) return;
+  const double hn = st[r].hn;
+  const double* w = W + r * ldw;
+  double* v = V + r * ldv_rhs + (int64_t)(j + 1) * ldv_col;
+  for (int64_t t = threadIdx.x; t < n; t += kFusedMgsThreads) v[t] = w[t] / hn;
 }
 
 // ||z||_2 for cycle start (beta), into st[r].beta, for rhs with outer_active.
 __global__ void __launch_bounds__(256) norm2_kernel(int64_t n, int K, const double* Z, int64_t ldz, RhsState* st,
                                                     double* partials, unsigned int* counter) {
-  __shared__ double sh[256];
+  __shared__ double sh[32];
   __shared__ bool last;
   for (int r = 0; r < K; ++r) {
     double part = 0.0;
@@ -910,11 +976,11 @@ __global__ void __launch_bounds__(256) norm2_kernel(int64_t n, int K, const doub
   __syncthreads();
   if (!last) return;
   __threadfence();
-  if (threadIdx.x < K) {
-    const int r = threadIdx.x;
+  for (int r = 0; r < K; ++r) {
     double s = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) s += partials[(int64_t)r * kRedBlocks + b];
-    st[r].beta = sqrt(s);
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) s += partials[(int64_t)r * kRedBlocks + b];
+    s = block_sum(s, sh);
+    if (threadIdx.x == 0) st[r].beta = sqrt(s);
   }
   if (threadIdx.x == 0) *counter = 0;
 }
@@ -1183,7 +1249,7 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
     }
   }
   if (e != cudaSuccess) return e;
-  gemv_finish_kernel<<<dim3((unsigned)cdiv<int64_t>(n, 256), K), 256, 0, st>>>(
+  gemv_finish_kernel<<<dim3((unsigned)cdiv<int64_t>(n, kFinRows), K), kFinRows * kFinGroups, 0, st>>>(
       n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split);
   prof_end(tok, abs_mode == 3 ? kProfGemv32 : kProfGemv, 8.0 * (double)n * (double)n, st);
   count_launches(2);
@@ -1244,10 +1310,11 @@ cudaError_t precond_launch(int K, int64_t n, const uint16_t* LU, int64_t ld, int
 
 template <class T>
 cudaError_t diag_inv_launch(int64_t n, const uint16_t* LU, int64_t ld, int fmt, void* dinv, cudaStream_t st) {
-  const size_t ism = diag_inv_smem<T>();
+  constexpr size_t ism = diag_inv_smem<T>();
   cudaError_t e = cudaFuncSetAttribute(diag_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism);
   if (e != cudaSuccess) return e;
-  diag_inv_kernel<T><<<dim3((unsigned)cdiv<int64_t>(n, kTB32), 2), 128, ism, st>>>(n, LU, ld, fmt, (T*)dinv);
+  diag_inv_kernel<T><<<dim3((unsigned)cdiv<int64_t>(n, kTB32), 2, kTB32 / kInvCols), kInvThreads, ism, st>>>(
+      n, LU, ld, fmt, (T*)dinv);
   count_launches(1);
   return cudaGetLastError();
 }
@@ -1285,21 +1352,23 @@ struct Solver {
     return e;
   }
 
+  // CTAs of the reductions over n: no more than hold an entry per thread
+  int red_blocks() const { return (int)std::min<int64_t>(kRedBlocks, cdiv<int64_t>(n, 256)); }
   cudaError_t read_brief() {
     return read_to_host(brief, w.brief, sizeof(Brief) * K, st);
   }
   // Arnoldi step j after w = M^{-1} A v_j: modified Gram-Schmidt, the Givens
-  // update (into the brief) and v_{j+1}; one CTA for small systems, else one
+  // update (into the brief) and v_{j+1}; one launch for small systems, else one
   // launch per projection, then the rotation and the scaling
   void arnoldi_tail(int j) {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     if (n * K <= kFusedMgsMaxElems) {
-      arnoldi_tail_kernel<<<1, kFusedMgsThreads, 0, st>>>(sp, n, K, m, j, w.w, n, w.V, n, ldv_rhs(), w.st, w.brief);
+      arnoldi_tail_kernel<<<K, kFusedMgsThreads, 0, st>>>(sp, n, m, j, w.w, n, w.V, n, ldv_rhs(), w.st, w.brief);
       count_launches(1);
       return;
     }
     for (int i = 0; i <= j + 1; ++i)
-      mgs_kernel<<<kRedBlocks, 256, 0, st>>>(n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st, w.partials, w.counter);
+      mgs_kernel<<<red_blocks(), 256, 0, st>>>(n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st, w.partials, w.counter);
     givens_kernel<<<1, 32, 0, st>>>(sp, j, w.st, w.brief);
     scale_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, w.w, n, w.V + (int64_t)(j + 1) * n, ldv_rhs(),
                                                                    w.st, 1);
@@ -1334,10 +1403,7 @@ struct Solver {
                          : diag_inv_launch<double>(n, LU, ldlu, fmt, w.dinv, st);
     if (e != cudaSuccess) return e;
     if (!prm.precond_fp32) {
-      constexpr size_t kChainSmem = sizeof(float) * kTB32 * kTB32;
-      e = cudaFuncSetAttribute(chain_blocks_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChainSmem);
-      if (e != cudaSuccess) return e;
-      chain_blocks_kernel<<<dim3((unsigned)cdiv<int64_t>(n, kTB32), 2), 256, kChainSmem, st>>>(
+      chain_blocks_kernel<<<dim3((unsigned)cdiv<int64_t>(n, kTB32), 2, kTB32 / kChainCols), 256, 0, st>>>(
           n, LU, ldlu, fmt, (const double*)w.dinv, w.pch);
       count_launches(1);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -1368,7 +1434,7 @@ struct Solver {
       if (!any(&Brief::outer_active)) break;
       // cycle start: z = M^{-1} r, beta, v0 = z / beta
       if ((e = precond(w.r, n, w.tmp, n)) != cudaSuccess) return e;
-      norm2_kernel<<<kRedBlocks, 256, 0, st>>>(n, K, w.tmp, n, w.st, w.partials, w.counter);
+      norm2_kernel<<<red_blocks(), 256, 0, st>>>(n, K, w.tmp, n, w.st, w.partials, w.counter);
       cycle_start_kernel<<<1, 32, 0, st>>>(sp, w.st, w.brief);
       scale_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, w.tmp, n, w.V, ldv_rhs(), w.st, 0);
       count_launches(3);
@@ -1618,7 +1684,7 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
         b.first = false;
       } else if (b.ph == kCycle) {
         e = s.precond(s.w.r, s.n, s.w.tmp, s.n);
-        norm2_kernel<<<kRedBlocks, 256, 0, st>>>(s.n, s.K, s.w.tmp, s.n, s.w.st, s.w.partials, s.w.counter);
+        norm2_kernel<<<s.red_blocks(), 256, 0, st>>>(s.n, s.K, s.w.tmp, s.n, s.w.st, s.w.partials, s.w.counter);
         cycle_start_kernel<<<1, 32, 0, st>>>(sp, s.w.st, s.w.brief);
         scale_kernel<<<(unsigned)cdiv<int64_t>(s.n, 256), 256, 0, st>>>(s.n, s.K, s.w.tmp, s.n, s.w.V, s.ldv_rhs(),
                                                                          s.w.st, 0);
