@@ -221,6 +221,27 @@ size_t gemv_tc_bytes(int64_t n);
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
                     void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st);
 
+// precond.cu: z = U^{-1} L^{-1} v (of diag(cs) U^{-1} L^{-1} diag(rs) with rs, cs)
+// for K right-hand sides, in fp32 or fp64.  Once per solve: a plan, the inverted
+// diagonal blocks and chain blocks (precond_inverse_bytes, precond_chain_bytes),
+// and zeroed publish words (precond_pub_bytes); each application takes a new
+// epoch >= 1.
+struct PrecondPlan {
+  int ctas = 0;
+  size_t smem = 0;
+  bool p1_smem = false;
+};
+size_t precond_inverse_bytes(int64_t n);
+size_t precond_chain_bytes(int64_t n);
+size_t precond_pub_bytes(int64_t n, int64_t K);
+bool precond_plan(int64_t n, int K, bool fp32, int sms, int budget, PrecondPlan* plan);
+cudaError_t precond_setup(int64_t n, const uint16_t* LU, int64_t ld, int fmt, bool fp32, void* dinv, void* chain,
+                          cudaStream_t st);
+cudaError_t precond_launch(const PrecondPlan& plan, bool fp32, int K, int64_t n, const uint16_t* LU, int64_t ld,
+                           int fmt, const void* dinv, const void* chain, const double* v, int64_t ldv, double* z,
+                           int64_t ldz, void* pub, int epoch, uint32_t* status, const double* rs, const double* cs,
+                           cudaStream_t st);
+
 // ir.cu
 size_t solve_batched_ws_bytes(const hpmxp_problem* probs, int count, int restart);
 size_t solve_ws_bytes(int64_t n, int64_t nrhs, int restart);

@@ -8,12 +8,7 @@
 //       column major) is read once for all columns, coalesced 16-byte loads,
 //       split over column chunks with a deterministic second pass.  The
 //       first pass can also accumulate |A| row sums (||A||_inf).
-//   precond_kernel<T>  z = U^{-1} L^{-1} v with the 16-bit factors, in T =
-//       float or double arithmetic, both sweeps in one cooperative launch:
-//       block rows of 128 are owned round-robin by the CTAs; the owner of a
-//       block solves it (a product with the inverted diagonal block) as soon
-//       as every earlier block has been applied, and publishes it as tagged
-//       64-bit words that the other CTAs poll (bounded).
+//   (the preconditioner z = U^{-1} L^{-1} v is in precond.cu)
 //   mgs_step / vec_norm / givens / cycle_start / cycle_finish / update:
 //       modified Gram-Schmidt Arnoldi, Givens least squares, x += V y.
 // All control decisions are taken on the device; the host reads a few
@@ -306,546 +301,6 @@ gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P, c
 }
 
 // ---------------------------------------------------------------------------
-// Preconditioner: 128-row blocks, the diagonal blocks of L and U inverted once
-// per solve (setup kernel below, in the arithmetic type T), so the diagonal
-// solve is a parallel 128 x 128 product.  Each published block is a run of
-// 64-bit words that carry their epoch: (fp32 value | epoch << 32) for T =
-// float, two words (high half | epoch << 32), (low half | epoch << 32) per
-// value for T = double; a reader's poll of the words delivers the data itself,
-// with no separate flag.  Before it waits for z_c, every CTA issues the copies
-// of what it will multiply z_c with: the owner of block c+1 its off-diagonal
-// tile (and, for float, the inverted diagonal block; the fp64 inverse, 128 KB,
-// is read from L2), and each CTA the tiles of its first two blocks that z_c
-// updates.
-// ---------------------------------------------------------------------------
-constexpr int kTB32 = 128;
-
-template <class T> __device__ inline T fma_t(T a, T b, T c);
-template <> __device__ inline float fma_t<float>(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-template <> __device__ inline double fma_t<double>(double a, double b, double c) { return __fma_rn(a, b, c); }
-// a 16-bit factor entry as T (exact either way; the fp64 one built with integer operations)
-template <class T> __device__ inline T u16_to(uint16_t h, int fmt);
-template <> __device__ inline float u16_to<float>(uint16_t h, int fmt) { return u16_to_f32(h, fmt); }
-template <> __device__ inline double u16_to<double>(uint16_t h, int fmt) { return u16_to_f64(h, fmt); }
-
-// Inverse of diagonal block c (c < nb) of the unit-lower L (which == 0) or of
-// U (which == 1) in T arithmetic, from the 16-bit factors.  Output inv[(which *
-// nb + c) * 128 * 128 + j * 128 + i] = inverse(i, j).  A CTA makes 32 columns
-// (grid z), one per lane: row by row, the finished row's term is added to the
-// rows still open, which are dealt out to the warps and kept in registers, so
-// that the FMAs between two barriers are independent.  Bound by the 128 steps'
-// latency (fp32) and the fp64 unit, where a warp's FMA takes 64 clocks of its
-// scheduler (fp64).  46 us in fp32 at n = 1024 and 210 us at 32768, 239 us in
-// fp64 at 4096; one thread per column, a chain of dependent FMAs on one SM per
-// block, took 80, 328 and 667 us.
-constexpr int kInvCols = 32, kInvPitch = kInvCols + 1, kInvThreads = 256;
-template <class T>
-__device__ inline T quotient(T s, T d, T r);   // s / d with r = 1 / d
-template <>
-__device__ inline float quotient<float>(float s, float d, float r) { return __fdiv_rn(s, d); }
-// one correction of s * r: the plain fp64 division costs about ten fp64 instructions
-template <>
-__device__ inline double quotient<double>(double s, double d, double r) {
-  const double q = s * r;
-  const double x = __fma_rn(__fma_rn(-q, d, s), r, q);
-  return isfinite(x) ? x : s / d;   // (a subnormal or infinite r)
-}
-template <class T>
-__global__ void __launch_bounds__(kInvThreads) diag_inv_kernel(int64_t n, const uint16_t* __restrict__ LU, int64_t ld,
-                                                               int fmt, T* __restrict__ inv) {
-  extern __shared__ __align__(16) unsigned char dsm_raw[];
-  T* t = reinterpret_cast<T*>(dsm_raw);      // t[k * 128 + i] = block(i, k)
-  T* x = t + kTB32 * kTB32;                  // x[i * kInvPitch + lane] = inverse(i, j0 + lane) when row i is done
-  T* dg = x + kTB32 * kInvPitch;             // U's diagonal and its reciprocals
-  T* rd = dg + kTB32;
-  const int nb = (int)cdiv<int64_t>(n, kTB32);
-  const int c = blockIdx.x, j0 = blockIdx.z * kInvCols, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool upper = blockIdx.y == 1;
-  const int64_t base = (int64_t)c * kTB32;
-  // the part of the block these columns need: rows and columns j0 .. 127 of L, 0 .. j0 + 31 of U
-  const int lo = upper ? 0 : j0, hi = upper ? j0 + kInvCols : kTB32;
-  // 16-byte loads, all in flight (the columns are 16-byte aligned and padded to 8 rows)
-  uint4 raw[kTB32 * kTB32 / 8 / kInvThreads];
-#pragma unroll
-  for (int q = 0; q < kTB32 * kTB32 / 8 / kInvThreads; ++q) {
-    const int chunk = tid + q * kInvThreads, k = chunk >> 4, i = (chunk & 15) * 8;
-    raw[q] = make_uint4(0, 0, 0, 0);
-    if (i + 8 > lo && i < hi && k >= lo && k < hi && base + k < n && base + i < n)
-      raw[q] = *reinterpret_cast<const uint4*>(LU + base + i + (base + k) * ld);
-  }
-#pragma unroll
-  for (int q = 0; q < kTB32 * kTB32 / 8 / kInvThreads; ++q) {
-    const int chunk = tid + q * kInvThreads, k = chunk >> 4, i0 = (chunk & 15) * 8;
-    const uint32_t w[4] = {raw[q].x, raw[q].y, raw[q].z, raw[q].w};
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-      const int i = i0 + e;
-      const bool in = base + i < n && base + k < n;
-      const T v = in ? u16_to<T>((uint16_t)(w[e >> 1] >> (16 * (e & 1))), fmt) : (T)0;
-      // the strict triangle only, zeros elsewhere: a finished row's term is then a no-op for
-      // the rows that are closed; U's diagonal apart
-      t[k * kTB32 + i] = (upper ? i < k : i > k) ? v : (T)0;
-      if (upper && i == k) dg[i] = in ? v : (T)1;
-    }
-  }
-  __syncthreads();
-  if (upper && tid < kTB32) rd[tid] = (T)1 / dg[tid];
-  __syncthreads();
-  // rows warp + kWarps r of the lane's column, in registers
-  constexpr int kWarps = kInvThreads / 32, kRows = kTB32 / kWarps;
-  T acc[kRows];
-#pragma unroll
-  for (int r = 0; r < kRows; ++r) acc[r] = warp + kWarps * r == j0 + lane ? (T)1 : (T)0;
-#pragma unroll 1
-  for (int step = 0; step < hi - lo; ++step) {
-    const int k = upper ? hi - 1 - step : lo + step;
-    // row k's warp finishes and publishes it (U: divided by the diagonal)
-    if (warp == k % kWarps) {
-      T xk = (T)0;
-#pragma unroll
-      for (int r = 0; r < kRows; ++r)
-        if (k == warp + kWarps * r) xk = acc[r];
-      x[k * kInvPitch + lane] = upper ? quotient<T>(xk, dg[k], rd[k]) : xk;
-    }
-    __syncthreads();
-    const T xk = -x[k * kInvPitch + lane];
-    const T* tk = t + k * kTB32 + warp;
-#pragma unroll
-    for (int g = 0; g < kRows; g += 4) {   // four rows at a time, skipped when all are closed
-      if (upper ? warp + kWarps * g >= k : warp + kWarps * (g + 3) <= k) continue;
-#pragma unroll
-      for (int r = g; r < g + 4; ++r) acc[r] = fma_t<T>(tk[kWarps * r], xk, acc[r]);
-    }
-  }
-  for (int idx = tid; idx < kTB32 * kInvCols; idx += kInvThreads) {   // rows outside lo .. hi - 1 are zero
-    const int i = idx / kInvCols;
-    if (i < lo || i >= hi) x[i * kInvPitch + idx % kInvCols] = (T)0;
-  }
-  __syncthreads();
-  T* out = inv + ((int64_t)blockIdx.y * nb + c) * kTB32 * kTB32 + (int64_t)j0 * kTB32;
-  for (int idx = tid; idx < kTB32 * kInvCols; idx += kInvThreads)
-    out[idx] = x[(idx % kTB32) * kInvPitch + idx / kTB32];
-}
-
-template <class T>
-constexpr size_t diag_inv_smem() { return sizeof(T) * (kTB32 * kTB32 + kTB32 * kInvPitch + 2 * kTB32); }
-static_assert(diag_inv_smem<double>() <= 232448, "shared memory per CTA");
-
-// Chain blocks of the fp64 preconditioner, once per solve: forward
-// P_c = Linv_c L(c, c-1) (c >= 1), backward Q_c = Uinv_c U(c, c+1) (c <= nb-2),
-// fp64 products of the fp64 inverses and the 16-bit factor tiles (terms t
-// ascending).  out[((which * nb + c) * 128 + j) * 128 + i] = P(i, j).  With
-// them the wavefront's dependent step is one product: z_{c+1} = y_{c+1} -
-// P_{c+1} z_c, y_{c+1} = Linv_{c+1} (v_{c+1} - sum_{k<c} L(c+1,k) z_k) being
-// known before z_c is.  Bound by the fp64 FMAs: a CTA makes 32 columns (grid z:
-// a small system fills the SMs), the tile is decoded once, and a warp stops at
-// its rows' last nonzero of the triangular inverse (the two halves take the row
-// quarters in opposite order, so that every scheduler has the same work): 1190
-// -> 173 us at n = 4096.
-constexpr int kChainCols = 32;
-__global__ void __launch_bounds__(256) chain_blocks_kernel(int64_t n, const uint16_t* __restrict__ LU, int64_t ld,
-                                                           int fmt, const double* __restrict__ dinv,
-                                                           double* __restrict__ out) {
-  __shared__ double tile[kTB32][kChainCols];   // tile[t][j] = T(t, j0 + j)
-  const int nb = (int)cdiv<int64_t>(n, kTB32);
-  const int c = blockIdx.x, which = blockIdx.y, j0 = blockIdx.z * kChainCols, tid = threadIdx.x;
-  const int nbr = which == 0 ? c - 1 : c + 1;   // block column of the neighbour tile
-  if (nbr < 0 || nbr >= nb) return;
-  const int64_t r0 = (int64_t)c * kTB32, c0 = (int64_t)nbr * kTB32 + j0;
-  for (int idx = tid; idx < kTB32 * kChainCols; idx += 256) {
-    const int t = idx % kTB32, j = idx / kTB32;   // coalesced over t (column major source)
-    const bool in = r0 + t < n && c0 + j < n;
-    tile[t][j] = in ? u16_to_f64(LU[r0 + t + (c0 + j) * ld], fmt) : 0.0;
-  }
-  __syncthreads();
-  const double* inv = dinv + ((int64_t)which * nb + c) * kTB32 * kTB32;
-  const int half = tid / kTB32, quarter = half ? 3 - ((tid >> 5) & 3) : (tid >> 5) & 3;
-  const int i = 32 * quarter + (tid & 31), jh = half * (kChainCols / 2);
-  const int t0 = which == 0 ? 0 : 32 * quarter, t1 = which == 0 ? 32 * quarter + 32 : kTB32;
-  double acc[kChainCols / 2];
-#pragma unroll
-  for (int q = 0; q < kChainCols / 2; ++q) acc[q] = 0.0;
-#pragma unroll 2
-  for (int t = t0; t < t1; ++t) {
-    const double a = inv[(int64_t)t * kTB32 + i];
-#pragma unroll
-    for (int q = 0; q < kChainCols / 2; ++q) acc[q] = __fma_rn(a, tile[t][jh + q], acc[q]);
-  }
-  double* o = out + ((int64_t)which * nb + c) * kTB32 * kTB32;
-#pragma unroll
-  for (int q = 0; q < kChainCols / 2; ++q) o[(int64_t)(j0 + jh + q) * kTB32 + i] = acc[q];
-}
-
-// words of one published value
-template <class T> constexpr int kWords = sizeof(T) / 4;
-// threads of the preconditioner's CTAs: each 128 x 128 product is split over
-// kPrecondThreads / 128 column groups (512 threads for fp32 measured no faster
-// than 256: the step is bound by the hand-off, not the products)
-template <class T> constexpr int kPrecondThreads = 256;
-
-__device__ inline unsigned long long tag_word(uint32_t bits, int epoch) {
-  return (unsigned long long)bits | ((unsigned long long)(unsigned)epoch << 32);
-}
-
-__device__ inline void cp_async16(uint32_t dst, const void* src, int bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
-}
-__device__ inline void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ inline void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-template <class T, int K>
-__global__ void __launch_bounds__(kPrecondThreads<T>) precond_kernel(int64_t n, const uint16_t* __restrict__ LU, int64_t ld,
-                                                      int fmt, const T* __restrict__ dinv,
-                                                      const double* __restrict__ pch,
-                                                      const double* __restrict__ v, int64_t ldv,
-                                                      double* __restrict__ z, int64_t ldz,
-                                                      unsigned long long* __restrict__ pub, int epoch,
-                                                      uint32_t* status, long long wait_polls,
-                                                      unsigned long long wait_ns, const double* __restrict__ rs,
-                                                      const double* __restrict__ cs) {
-  constexpr bool kInvInSmem = sizeof(T) == 4;   // the fp32 inverse (64 KB) is staged; the fp64 one stays in L2
-  constexpr int W = kWords<T>;
-  constexpr int NT = kPrecondThreads<T>;   // threads: NT / 128 groups of 128 rows ...
-  constexpr int HG = NT / kTB32;
-  constexpr int HC = kTB32 / HG;           // ... each multiplying HC of a tile's columns
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  const int nb = (int)cdiv<int64_t>(n, kTB32);
-  const int G = gridDim.x, me = blockIdx.x, tid = threadIdx.x;
-  const int nown = (nb - me + G - 1) / G;
-  uint16_t* tl = reinterpret_cast<uint16_t*>(sm_raw);             // 3 x [128][128] 16-bit tiles, tl[j*128+i]
-  float* ti = reinterpret_cast<float*>(tl + 3 * kTB32 * kTB32);   // [128][128] fp32 inverse (float only)
-  T* acc = reinterpret_cast<T*>(kInvInSmem ? (unsigned char*)(ti + kTB32 * kTB32) : (unsigned char*)ti);
-  T* zc = acc + (size_t)nown * kTB32 * K;                         // [128][K] block c
-  T* zs = zc + kTB32 * K;                                         // [128][K] block being solved
-  T* part = zs + kTB32 * K;                                       // [HG][128][K]
-  T* ys = part + HG * kTB32 * K;                                  // [128][K] y of the next block (fp64)
-  __shared__ int abort_flag;
-  if (tid == 0) abort_flag = 0;
-  unsigned long long* fpub = pub;
-  unsigned long long* bpub = pub + (size_t)nb * kTB32 * K * W;
-  for (int o = 0; o < nown; ++o)
-    for (int t = tid; t < kTB32 * K; t += NT) {
-      const int ii = t % kTB32, r = t / kTB32;
-      const int64_t i = (int64_t)(me + o * G) * kTB32 + ii;
-      // balanced factors (LU of diag(rs) A diag(cs)): M^{-1} v = diag(cs) U^{-1} L^{-1} diag(rs) v;
-      // rs and cs are powers of two, so the scalings are exact
-      acc[((size_t)o * kTB32 + ii) * K + r] = i < n ? (T)(rs ? v[i + r * ldv] * rs[i] : v[i + r * ldv]) : (T)0;
-    }
-  // abort_flag (and acc) must be written before any thread reads them: shared
-  // memory starts with whatever the SM's previous block left there
-  __syncthreads();
-
-  // asynchronous copies: 16-bit tile (rb, cb) of LU into buffer slot, zero outside the matrix
-  auto fetch_tile = [&](int slot, int rb, int cb) {
-    uint16_t* dst = tl + (size_t)slot * kTB32 * kTB32;
-    const int64_t i0 = (int64_t)rb * kTB32, j0 = (int64_t)cb * kTB32;
-#pragma unroll
-    for (int q = 0; q < 2048 / NT; ++q) {
-      const int chunk = tid + q * NT;             // 2048 chunks of 8 rows
-      const int jj = chunk >> 4, ii = (chunk & 15) * 8;
-      const int64_t i = i0 + ii, j = j0 + jj;
-      int bytes = 0;
-      if (j < n && i < n) bytes = (int)min((int64_t)16, (n - i) * 2);
-      const uint16_t* src = bytes ? LU + i + j * ld : LU;
-      cp_async16((uint32_t)__cvta_generic_to_shared(dst + jj * kTB32 + ii), src, bytes);
-    }
-  };
-  auto inv_block = [&](int which, int cb) { return dinv + ((int64_t)which * nb + cb) * kTB32 * kTB32; };
-  // fp64: the HC inverse entries a thread multiplies, M(ii, h*HC .. h*HC+HC-1),
-  // loaded into registers when the block becomes next; used by its solve
-  T invr[kInvInSmem ? 1 : HC];
-  auto fetch_inv = [&](int which, int cb) {
-    const T* src = inv_block(which, cb);
-    if constexpr (kInvInSmem) {
-#pragma unroll
-      for (int q = 0; q < 4096 / NT; ++q) {
-        const int chunk = tid + q * NT;           // 4096 chunks of 4 floats
-        cp_async16((uint32_t)__cvta_generic_to_shared(ti + chunk * 4), src + chunk * 4, 16);
-      }
-    } else {
-      const int ii = tid % kTB32, h = tid / kTB32;
-#pragma unroll
-      for (int q = 0; q < HC; ++q) invr[q] = __ldcg(src + (h * HC + q) * kTB32 + ii);
-    }
-  };
-  // fp64: the chain block P (which 0) / Q (which 1) of block cb into the same registers
-  auto fetch_chain = [&](int which, int cb) {
-    if constexpr (!kInvInSmem) {
-      const double* src = pch + ((int64_t)which * nb + cb) * kTB32 * kTB32;
-      const int ii = tid % kTB32, h = tid / kTB32;
-#pragma unroll
-      for (int q = 0; q < HC; ++q) invr[q] = __ldcg(src + (h * HC + q) * kTB32 + ii);
-    }
-  };
-  // out[i][r] (-)= sum_j M(i, j) w[j][r]; M a 16-bit tile (T16) or the inverse (Tinv, fp32 in
-  // shared memory or T in global memory)
-  auto product = [&](const uint16_t* T16, const T* Tinv, const T* w, T* out, bool subtract) {
-    const int ii = tid % kTB32, h = tid / kTB32;
-    T s[K];
-#pragma unroll
-    for (int r = 0; r < K; ++r) s[r] = (T)0;
-    if (T16) {
-#pragma unroll 8
-      for (int jj = h * HC; jj < h * HC + HC; ++jj) {
-        const T tv = u16_to<T>(T16[jj * kTB32 + ii], fmt);
-#pragma unroll
-        for (int r = 0; r < K; ++r) s[r] = fma_t<T>(tv, w[jj * K + r], s[r]);
-      }
-    } else {
-#pragma unroll 16
-      for (int jj = h * HC; jj < h * HC + HC; ++jj) {
-        const T tv = Tinv[jj * kTB32 + ii];
-#pragma unroll
-        for (int r = 0; r < K; ++r) s[r] = fma_t<T>(tv, w[jj * K + r], s[r]);
-      }
-    }
-#pragma unroll
-    for (int r = 0; r < K; ++r) part[(h * kTB32 + ii) * K + r] = s[r];
-    __syncthreads();
-    for (int t = tid; t < kTB32 * K; t += NT) {
-      T tot = part[t];
-#pragma unroll
-      for (int g = 1; g < HG; ++g) tot += part[g * kTB32 * K + t];
-      out[t] = subtract ? out[t] - tot : tot;
-    }
-    __syncthreads();
-  };
-  // all copies issued by this CTA have landed (ready) / all but the latest group (ready_prev)
-  auto ready = [&]() { cp_async_wait<0>(); __syncthreads(); };
-  auto ready_prev = [&]() { cp_async_wait<1>(); __syncthreads(); };
-  // wait for the tagged words of block c and unpack them into dst; a wait
-  // that runs out (at most wait_polls polls and wait_ns of the global timer)
-  // sets the timeout bit and the CTA's abort flag, and the other threads of
-  // the CTA stop polling once they see the flag
-  volatile int* abort_v = &abort_flag;
-  auto receive = [&](const unsigned long long* src, int c, T* dst) {
-    const unsigned long long* w = src + (size_t)c * kTB32 * K * W;
-    const unsigned long long t0 = global_ns();
-    for (int t = tid; t < kTB32 * K; t += NT) {
-      uint32_t bits[W];
-#pragma unroll
-      for (int h = 0; h < W; ++h) {
-        unsigned long long word = 0;
-        for (long long it = 0;; ++it) {
-          asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(word) : "l"(w + (size_t)t * W + h) : "memory");
-          if ((int)(word >> 32) == epoch) break;
-          if (it >= wait_polls || ((it & 63) == 63 && (global_ns() - t0 > wait_ns || *abort_v))) {
-            atomicOr(status, kErrTimeout);
-            *abort_v = 1;
-            break;
-          }
-        }
-        bits[h] = (uint32_t)(word & 0xffffffffu);
-      }
-      if constexpr (W == 1) dst[t] = __uint_as_float(bits[0]);
-      else dst[t] = __hiloint2double((int)bits[0], (int)bits[1]);
-    }
-    __syncthreads();
-  };
-  // fp64: out = M w (or from - M w) with M in the invr registers (thread: row ii,
-  // columns h*HC .. h*HC+HC-1), the column groups summed in order through `part`
-  auto reg_product = [&](const T* w, T* out, const T* from) {
-    const int ii = tid % kTB32, h = tid / kTB32;
-    T sr[K];
-#pragma unroll
-    for (int r = 0; r < K; ++r) sr[r] = (T)0;
-#pragma unroll
-    for (int q = 0; q < HC; ++q)
-#pragma unroll
-      for (int r = 0; r < K; ++r) sr[r] = fma_t<T>(invr[kInvInSmem ? 0 : q], w[(h * HC + q) * K + r], sr[r]);
-#pragma unroll
-    for (int r = 0; r < K; ++r) part[(h * kTB32 + ii) * K + r] = sr[r];
-    __syncthreads();
-    for (int t = tid; t < kTB32 * K; t += NT) {
-      T tot = part[t];
-#pragma unroll
-      for (int g = 1; g < HG; ++g) tot += part[g * kTB32 * K + t];
-      out[t] = from ? from[t] - tot : tot;
-    }
-    __syncthreads();
-  };
-  // zs = Tinv acc_o (or, with chain, zs as computed by the caller), stored back
-  // into acc_o and published (backward: also into z)
-  auto solve = [&](int o, int c, bool backward, unsigned long long* dst, bool chained = false) {
-    T* a = acc + (size_t)o * kTB32 * K;
-    if (!chained) {
-      if constexpr (kInvInSmem) product(nullptr, reinterpret_cast<const T*>(ti), a, zs, false);
-      else reg_product(a, zs, nullptr);
-    }
-    unsigned long long* wd = dst + (size_t)c * kTB32 * K * W;
-    for (int t = tid; t < kTB32 * K; t += NT) {
-      a[t] = zs[t];
-      if constexpr (W == 1) {
-        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(wd + t), "l"(tag_word(__float_as_uint(zs[t]), epoch))
-                     : "memory");
-      } else {
-        const double d = zs[t];
-        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(wd + 2 * t),
-                     "l"(tag_word((uint32_t)__double2hiint(d), epoch)) : "memory");
-        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(wd + 2 * t + 1),
-                     "l"(tag_word((uint32_t)__double2loint(d), epoch)) : "memory");
-      }
-      if (backward) {
-        const int ii = t / K, r = t % K;
-        const int64_t i = (int64_t)c * kTB32 + ii;
-        if (i < n) z[i + r * ldz] = cs ? (double)zs[t] * cs[i] : (double)zs[t];
-      }
-    }
-    __syncthreads();
-  };
-  // The first two owned blocks that block c updates (past c in the sweep's
-  // direction, other than `skip`): their tiles go to slots 1 and 2 before z_c
-  // is awaited, since the tiles do not depend on it.  Returns how many.
-  int pre_o[2];
-  auto prefetch_updates = [&](int c, bool forward, int skip) {
-    int k = 0;
-    for (int o = 0; o < nown && k < 2; ++o) {
-      const int rb = me + o * G;
-      if (o == skip || (forward ? rb <= c : rb >= c)) continue;
-      fetch_tile(1 + k, rb, c);
-      pre_o[k++] = o;
-    }
-    return k;
-  };
-  // updates of the owned blocks by z_c: the `npre` prefetched ones from slots 1, 2, then
-  // the rest with tiles double buffered in slots 1, 2
-  auto stream_updates = [&](int c, bool forward, int skip, int npre) {
-    for (int k = 0; k < npre; ++k)
-      product(tl + (size_t)(1 + k) * kTB32 * kTB32, nullptr, zc, acc + (size_t)pre_o[k] * kTB32 * K, true);
-    int pending = -1, slot = 1;
-    for (int o = 0; o < nown; ++o) {
-      const int rb = me + o * G;
-      if (o == skip || (forward ? rb <= c : rb >= c)) continue;
-      bool done = false;
-      for (int k = 0; k < npre; ++k) done = done || pre_o[k] == o;
-      if (done) continue;
-      if (pending < 0) { fetch_tile(slot, rb, c); cp_async_commit(); pending = o; continue; }
-      // compute the pending one while the next streams in
-      fetch_tile(3 - slot, rb, c);
-      cp_async_commit();
-      ready_prev();
-      product(tl + (size_t)slot * kTB32 * kTB32, nullptr, zc, acc + (size_t)pending * kTB32 * K, true);
-      pending = o;
-      slot = 3 - slot;
-    }
-    if (pending >= 0) {
-      ready();
-      product(tl + (size_t)slot * kTB32 * kTB32, nullptr, zc, acc + (size_t)pending * kTB32 * K, true);
-    }
-  };
-
-  // fp32: once a CTA has solved block b, the tile and inverse that its next
-  // block b' = b +- G will take on the chain are fetched at the end of that
-  // iteration (into slot 0 and the inverse buffer, unused until then), so they
-  // have landed when z_{b'-+1} arrives; `early` names b'
-  int early = -1;
-  auto fetch_early = [&](int nx, int which, bool forward) {
-    if constexpr (kInvInSmem) {
-      if (nx >= 0 && nx < nb) {
-        fetch_tile(0, nx, forward ? nx - 1 : nx + 1);
-        fetch_inv(which, nx);
-        cp_async_commit();
-        early = nx;
-      }
-    }
-  };
-
-  // ---------------- forward: L y = v ----------------
-  if (me == 0) { fetch_inv(0, 0); cp_async_commit(); ready(); solve(0, 0, false, fpub); }
-  for (int c = 0; c < nb && !abort_flag; ++c) {
-    const bool next_mine = c + 1 < nb && (c + 1) % G == me;
-    if (c % G != me) {
-      const int last = me + (nown - 1) * G;
-      if (nown == 0 || last <= c) continue;
-    }
-    const int skip = next_mine ? (c + 1) / G : -1;
-    if (next_mine) {
-      if constexpr (kInvInSmem) {
-        if (early != c + 1) {
-          fetch_tile(0, c + 1, c);
-          fetch_inv(0, c + 1);
-        }
-      } else {
-        // fp64: y = Linv_{c+1} acc_{c+1} before z_c is awaited (acc_{c+1} has every
-        // term but z_c's), then the chain block P_{c+1} into the registers
-        fetch_inv(0, c + 1);
-        reg_product(acc + (size_t)skip * kTB32 * K, ys, nullptr);
-        fetch_chain(0, c + 1);
-      }
-    }
-    const int npre = prefetch_updates(c, true, skip);
-    cp_async_commit();
-    if (c % G == me) {
-      for (int t = tid; t < kTB32 * K; t += NT) zc[t] = acc[(size_t)(c / G) * kTB32 * K + t];
-    } else {
-      receive(fpub, c, zc);
-      if (abort_flag) break;
-    }
-    ready();
-    if (next_mine) {
-      if constexpr (kInvInSmem) {
-        product(tl, nullptr, zc, acc + (size_t)skip * kTB32 * K, true);
-        solve(skip, c + 1, false, fpub);
-      } else {
-        reg_product(zc, zs, ys);   // z_{c+1} = y_{c+1} - P_{c+1} z_c
-        solve(skip, c + 1, false, fpub, true);
-      }
-    }
-    stream_updates(c, true, skip, npre);
-    if (next_mine) fetch_early(c + 1 + G, 0, true);
-  }
-  ready();
-  early = -1;
-
-  // ---------------- backward: U z = y ----------------
-  if ((nb - 1) % G == me && !abort_flag) {
-    fetch_inv(1, nb - 1);
-    cp_async_commit();
-    ready();
-    solve((nb - 1) / G, nb - 1, true, bpub);
-  }
-  for (int c = nb - 1; c >= 0 && !abort_flag; --c) {
-    const bool next_mine = c - 1 >= 0 && (c - 1) % G == me;
-    if (c % G != me && (nown == 0 || me >= c)) continue;
-    const int skip = next_mine ? (c - 1) / G : -1;
-    if (next_mine) {
-      if constexpr (kInvInSmem) {
-        if (early != c - 1) {
-          fetch_tile(0, c - 1, c);
-          fetch_inv(1, c - 1);
-        }
-      } else {
-        fetch_inv(1, c - 1);
-        reg_product(acc + (size_t)skip * kTB32 * K, ys, nullptr);
-        fetch_chain(1, c - 1);
-      }
-    }
-    const int npre = prefetch_updates(c, false, skip);
-    cp_async_commit();
-    if (c % G == me) {
-      for (int t = tid; t < kTB32 * K; t += NT) zc[t] = acc[(size_t)(c / G) * kTB32 * K + t];
-    } else {
-      receive(bpub, c, zc);
-      if (abort_flag) break;
-    }
-    ready();
-    if (next_mine) {
-      if constexpr (kInvInSmem) {
-        product(tl, nullptr, zc, acc + (size_t)skip * kTB32 * K, true);
-        solve(skip, c - 1, true, bpub);
-      } else {
-        reg_product(zc, zs, ys);   // z_{c-1} = y_{c-1} - Q_{c-1} z_c
-        solve(skip, c - 1, true, bpub, true);
-      }
-    }
-    stream_updates(c, false, skip, npre);
-    if (next_mine) fetch_early(c - 1 - G, 1, false);
-  }
-  ready();
-}
-
-// ---------------------------------------------------------------------------
 // Vector kernels.  Deterministic reductions: per-thread strided partials,
 // fixed-shape block tree, per-block partials summed the same way by the last CTA.
 // ---------------------------------------------------------------------------
@@ -1130,8 +585,8 @@ struct SolveWs {
   double* P;         // nchunk x n x K
   void* RS;          // nchunk x n (fp64 size)
   void* pub;         // 2 sweeps x round_up(n, 128) x K values x (1 or 2) 8-byte tagged words
-  void* dinv;        // 2 x nb128 x 128 x 128 inverted diagonal blocks (float or double)
-  double* pch;       // 2 x nb128 x 128 x 128 chain blocks of the fp64 preconditioner
+  void* dinv;        // inverted diagonal blocks of L and U (precond.cu)
+  void* chain;       // the blocks next to them, multiplied by the inverses
   float* a32;        // optional fp32 copy of A (ld32), written by the first residual, NULL if none
   int64_t ld32;
   size_t bytes;
@@ -1148,9 +603,6 @@ int gemv_chunks(int64_t n, int K = kMaxK) {
   c = std::max<int64_t>(1, std::min<int64_t>(c, cdiv<int64_t>(n, 8)));
   return (int)c;
 }
-
-// tagged words of both sweeps, sized for fp64 values (two words each)
-size_t pub_bytes(int64_t n, int64_t K) { return sizeof(unsigned long long) * 2 * 2 * round_up<int64_t>(n, kTB32) * K; }
 
 SolveWs carve_solve(void* base, int64_t n, int64_t K, int m) {
   SolveWs w{};
@@ -1172,9 +624,9 @@ SolveWs carve_solve(void* base, int64_t n, int64_t K, int m) {
   w.V = (double*)take(sizeof(double) * n * (m + 1) * K);
   w.P = (double*)take(sizeof(double) * nchunk * n * K);
   w.RS = take(sizeof(double) * nchunk * n);
-  w.pub = take(pub_bytes(n, K));
-  w.dinv = take(sizeof(double) * 2 * round_up<int64_t>(n, kTB32) * kTB32);
-  w.pch = (double*)take(sizeof(double) * 2 * round_up<int64_t>(n, kTB32) * kTB32);
+  w.pub = take(precond_pub_bytes(n, K));
+  w.dinv = take(precond_inverse_bytes(n));
+  w.chain = take(precond_chain_bytes(n));
   w.bytes = off;
   return w;
 }
@@ -1256,69 +708,6 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
   return cudaGetLastError();
 }
 
-// Dynamic shared memory cap of the preconditioner kernels (the attribute is
-// set to this one value, never to a per-call size).
-constexpr size_t kMaxPrecondSmem = 200 * 1024;
-
-template <class T>
-size_t precond_smem(int64_t n, int K, int G) {
-  const int nb = (int)cdiv<int64_t>(n, kTB32);
-  const int nown = cdiv(nb, G);
-  const size_t inv = sizeof(T) == 4 ? sizeof(float) * kTB32 * kTB32 : 0;
-  const size_t groups = kPrecondThreads<T> / kTB32;
-  return sizeof(uint16_t) * 3 * kTB32 * kTB32 + inv +
-         sizeof(T) * ((size_t)nown * kTB32 * K + 2 * kTB32 * K + groups * kTB32 * K + kTB32 * K) + 64;
-}
-
-template <class T, int K>
-cudaError_t precond_launch_k(int64_t n, const uint16_t* LU, int64_t ld, int fmt, const T* dinv, const double* pch,
-                             const double* v,
-                             int64_t ldv, double* z, int64_t ldz, unsigned long long* pub, int epoch,
-                             uint32_t* status, int G, size_t smem, cudaStream_t st, const double* rs,
-                             const double* cs) {
-  auto kern = precond_kernel<T, K>;
-  // one value for every call: concurrent solves on other threads set the same cap
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxPrecondSmem);
-  if (e != cudaSuccess) return e;
-  const WaitBudget wb = wait_budget();
-  long long polls = wb.polls;
-  unsigned long long ns = wb.ns;
-  void* args[] = {&n,  (void*)&LU, &ld,     &fmt,   (void*)&dinv, (void*)&pch, (void*)&v,  &ldv, &z,
-                  &ldz, &pub,      &epoch, &status, &polls,      &ns,         (void*)&rs, (void*)&cs};
-  return cudaLaunchCooperativeKernel((const void*)kern, dim3(G), dim3(kPrecondThreads<T>), args, smem, st);
-}
-
-template <class T>
-cudaError_t precond_launch(int K, int64_t n, const uint16_t* LU, int64_t ld, int fmt, const T* dinv,
-                           const double* pch, const double* v, int64_t ldv, double* z, int64_t ldz, unsigned long long* pub,
-                           int epoch, uint32_t* status, int G, size_t smem, cudaStream_t st, const double* rs,
-                           const double* cs) {
-#define HPMXP_PRECOND_K(KK) \
-  precond_launch_k<T, KK>(n, LU, ld, fmt, dinv, pch, v, ldv, z, ldz, pub, epoch, status, G, smem, st, rs, cs)
-  switch (K) {
-    case 1: return HPMXP_PRECOND_K(1);
-    case 2: return HPMXP_PRECOND_K(2);
-    case 3: return HPMXP_PRECOND_K(3);
-    case 4: return HPMXP_PRECOND_K(4);
-    case 5: return HPMXP_PRECOND_K(5);
-    case 6: return HPMXP_PRECOND_K(6);
-    case 7: return HPMXP_PRECOND_K(7);
-    default: return HPMXP_PRECOND_K(8);
-  }
-#undef HPMXP_PRECOND_K
-}
-
-template <class T>
-cudaError_t diag_inv_launch(int64_t n, const uint16_t* LU, int64_t ld, int fmt, void* dinv, cudaStream_t st) {
-  constexpr size_t ism = diag_inv_smem<T>();
-  cudaError_t e = cudaFuncSetAttribute(diag_inv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism);
-  if (e != cudaSuccess) return e;
-  diag_inv_kernel<T><<<dim3((unsigned)cdiv<int64_t>(n, kTB32), 2, kTB32 / kInvCols), kInvThreads, ism, st>>>(
-      n, LU, ld, fmt, (T*)dinv);
-  count_launches(1);
-  return cudaGetLastError();
-}
-
 struct Solver {
   int64_t n;
   int K, m;
@@ -1332,8 +721,7 @@ struct Solver {
   SolveWs w;
   cudaStream_t st;
   int epoch = 0;
-  int G = 0;
-  size_t psmem = 0;
+  PrecondPlan plan;
   Brief brief[kMaxK];
 
   int64_t ldv_rhs() const { return n * (m + 1); }
@@ -1341,12 +729,8 @@ struct Solver {
   cudaError_t precond(const double* v, int64_t ldv, double* z, int64_t ldz) {
     ++epoch;
     void* tok = prof_begin(st);
-    unsigned long long* pub = (unsigned long long*)w.pub;
-    cudaError_t e = prm.precond_fp32
-                        ? precond_launch<float>(K, n, LU, ldlu, fmt, (const float*)w.dinv, nullptr, v, ldv, z, ldz,
-                                                pub, epoch, w.status, G, psmem, st, rs, cs)
-                        : precond_launch<double>(K, n, LU, ldlu, fmt, (const double*)w.dinv, w.pch, v, ldv, z, ldz,
-                                                 pub, epoch, w.status, G, psmem, st, rs, cs);
+    const cudaError_t e = precond_launch(plan, prm.precond_fp32 != 0, K, n, LU, ldlu, fmt, w.dinv, w.chain, v, ldv, z,
+                                         ldz, w.pub, epoch, w.status, rs, cs, st);
     prof_end(tok, kProfPrecond, 2.0 * (double)n * (double)n, st);
     count_launches(1);
     return e;
@@ -1385,29 +769,10 @@ struct Solver {
     int dev = 0, sms = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    // one CTA per SM at most: a cooperative launch keeps all of them resident
-    const int nb = (int)cdiv<int64_t>(n, kTB32);
-    // one CTA per owned share of block rows; an SM budget takes fewer CTAs as
-    // long as their shares still fit in shared memory
-    const int budget = sm_budget();
-    const int gmax = std::max(1, std::min(nb, sms));
-    G = std::max(1, std::min(gmax, budget > 0 ? budget : gmax));
-    auto smem_for = [&](int g) {
-      return prm.precond_fp32 ? precond_smem<float>(n, K, g) : precond_smem<double>(n, K, g);
-    };
-    while (G < gmax && smem_for(G) > kMaxPrecondSmem) ++G;
-    psmem = smem_for(G);
-    if (psmem > kMaxPrecondSmem) return cudaErrorInvalidValue;
-    if ((e = cudaMemsetAsync(w.pub, 0, pub_bytes(n, K), st)) != cudaSuccess) return e;
-    e = prm.precond_fp32 ? diag_inv_launch<float>(n, LU, ldlu, fmt, w.dinv, st)
-                         : diag_inv_launch<double>(n, LU, ldlu, fmt, w.dinv, st);
-    if (e != cudaSuccess) return e;
-    if (!prm.precond_fp32) {
-      chain_blocks_kernel<<<dim3((unsigned)cdiv<int64_t>(n, kTB32), 2, kTB32 / kChainCols), 256, 0, st>>>(
-          n, LU, ldlu, fmt, (const double*)w.dinv, w.pch);
-      count_launches(1);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    const bool fp32 = prm.precond_fp32 != 0;
+    if (!precond_plan(n, K, fp32, sms, sm_budget(), &plan)) return cudaErrorInvalidValue;
+    if ((e = cudaMemsetAsync(w.pub, 0, precond_pub_bytes(n, K), st)) != cudaSuccess) return e;
+    if ((e = precond_setup(n, LU, ldlu, fmt, fp32, w.dinv, w.chain, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(w.st, 0, sizeof(RhsState) * kMaxK, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(w.counter, 0, 256, st)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(w.status, 0, 4, st)) != cudaSuccess) return e;
