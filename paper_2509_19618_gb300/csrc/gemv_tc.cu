@@ -87,9 +87,10 @@ static_assert(gemv_smem<8>() <= 232448, "shared memory per CTA");
 
 // f_r: 2^f_r > max_j |x_jr| (one CTA per right-hand side)
 __global__ void __launch_bounds__(1024) xscale_kernel(int64_t n, const double* __restrict__ X, int64_t ldx,
-                                                      int* __restrict__ fr) {
+                                                      int* __restrict__ fr, Gate gate) {
   __shared__ int sh[32];
   pdl_wait();
+  if (gate.closed()) return;
   pdl_trigger();
   const double* x = X + blockIdx.x * ldx;
   int m = 0;
@@ -111,13 +112,14 @@ __global__ void __launch_bounds__(1024) xscale_kernel(int64_t n, const double* _
 // and flag (1: an x that is not finite or too small for them).
 __global__ void __launch_bounds__(512) digit_kernel(int64_t n, int K, const double* __restrict__ X, int64_t ldx,
                                                     int* __restrict__ fr, uint8_t* __restrict__ dig,
-                                                    int* __restrict__ ex) {
+                                                    int* __restrict__ ex, Gate gate) {
   __shared__ int es[8][kBlk];
   __shared__ int bad;
   const int jl = threadIdx.x & (kBlk - 1), r = threadIdx.x / kBlk;
   const int64_t j = (int64_t)blockIdx.x * kBlk + jl;
   if (threadIdx.x == 0) bad = 0;
   pdl_wait();
+  if (gate.closed()) return;
   pdl_trigger();
   double v = 0.0;
   int f = 0;
@@ -222,10 +224,15 @@ struct GemvTc {
   uint32_t* status;
   long long wait_polls;
   unsigned long long wait_ns;
+  Gate gate;
 };
 
 template <int K, bool kAbs>
 __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant__ CUtensorMap tmA, GemvTc p) {
+  if (p.gate.flag) {
+    pdl_wait();
+    if (p.gate.closed()) return;
+  }
   extern __shared__ uint8_t raw_smem[];
   uint8_t* smem = raw_smem + ((1024u - (smem_u32(raw_smem) & 1023u)) & 1023u);
   uint8_t* ring = smem + kBArea;                                                    // [group][stage][8 columns][128 rows]
@@ -619,7 +626,7 @@ bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, Gemv
 }
 
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
-                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st) {
+                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate) {
   const int nkb = (int)cdiv<int64_t>(n, kBlk);
   GemvTc p{};
   p.n = n; p.A = A; p.lda = lda; p.X = X; p.ldx = ldx;
@@ -634,11 +641,12 @@ cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double
   const WaitBudget wb = wait_budget();
   p.wait_polls = wb.polls;
   p.wait_ns = wb.ns;
+  p.gate = gate;
   CUtensorMap tm;
   if (!encode_f64_map(&tm, A, n, n, lda, kRowsT, kCols)) return cudaErrorInvalidValue;
   count_launches(3);
-  cudaError_t e = launch_pdl(xscale_kernel, dim3(K), dim3(1024), 0, st, n, X, ldx, fr);
-  if (e == cudaSuccess) e = launch_pdl(digit_kernel, dim3(nkb), dim3(512), 0, st, n, K, X, ldx, fr, dig, ex);
+  cudaError_t e = launch_pdl(xscale_kernel, dim3(K), dim3(1024), 0, st, n, X, ldx, fr, gate);
+  if (e == cudaSuccess) e = launch_pdl(digit_kernel, dim3(nkb), dim3(512), 0, st, n, K, X, ldx, fr, dig, ex, gate);
   if (e != cudaSuccess) return e;
 #define HPMXP_GEMV_K(KK) \
   case KK: return abs_sums ? launch_k<KK, true>(tm, p, st) : launch_k<KK, false>(tm, p, st)

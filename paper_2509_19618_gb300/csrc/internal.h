@@ -193,6 +193,20 @@ cudaError_t lu_f64(int64_t n, double* A, int64_t ld, uint32_t* status, cudaStrea
 cudaError_t lu_solve_f64(int64_t n, const double* LU, int64_t ld, double* X, int64_t ldx, int64_t nrhs,
                          cudaStream_t st);
 
+// A launch that the host issued before it knew whether the work is wanted: the
+// kernel returns at once when none of `count` device flags, `stride` ints apart,
+// is set.  No flags: always wanted.
+struct Gate {
+  const int* flag = nullptr;
+  int count = 0, stride = 0;
+  __device__ bool closed() const {
+    if (!flag) return false;
+    int any = 0;
+    for (int r = 0; r < count; ++r) any |= flag[(size_t)r * stride];
+    return any == 0;
+  }
+};
+
 // gemv_tc.cu: fp64 products A X (K <= 8 columns) from exact digit products on
 // the tensor cores, for the refinement's kernels in ir.cu.
 // The work is cut evenly: the 512-row tiles' lists of `blocks` 64-column
@@ -219,7 +233,7 @@ bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, Gemv
 // of scratch, 16-byte aligned.
 size_t gemv_tc_bytes(int64_t n);
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
-                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st);
+                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate);
 
 // precond.cu: z = U^{-1} L^{-1} v (of diag(cs) U^{-1} L^{-1} diag(rs) with rs, cs)
 // for K right-hand sides, in fp32 or fp64.  Once per solve: a plan, the inverted
@@ -240,7 +254,7 @@ cudaError_t precond_setup(int64_t n, const uint16_t* LU, int64_t ld, int fmt, bo
 cudaError_t precond_launch(const PrecondPlan& plan, bool fp32, int K, int64_t n, const uint16_t* LU, int64_t ld,
                            int fmt, const void* dinv, const void* chain, const double* v, int64_t ldv, double* z,
                            int64_t ldz, void* pub, int epoch, uint32_t* status, const double* rs, const double* cs,
-                           cudaStream_t st);
+                           cudaStream_t st, Gate gate = {});
 
 // ir.cu
 size_t solve_batched_ws_bytes(const hpmxp_problem* probs, int count, int restart);

@@ -73,6 +73,13 @@ struct Brief {          // copied to the host after each control kernel
   double sr;
 };
 
+// What the host reads in one copy: the status word and the briefs.
+struct Report {
+  uint32_t status;
+  uint32_t pad[15];
+  Brief brief[kMaxK];
+};
+
 struct SolveParams {
   int n_rhs, m, max_iters;
   double inner_tol, theta, accept;
@@ -95,7 +102,9 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_partial_kernel(int64_t n, c
                                                                     int64_t lda, const double* __restrict__ X,
                                                                     int64_t ldx, int64_t chunk,
                                                                     float* __restrict__ A32, int64_t ld32,
-                                                                    double* __restrict__ P, void* __restrict__ RS) {
+                                                                    double* __restrict__ P, void* __restrict__ RS,
+                                                                    Gate gate) {
+  if (gate.closed()) return;
   __shared__ double xs[kGemvChunkElems];   // xs[r * chunk + jj]
   const int64_t i = (int64_t)blockIdx.x * kGemvRows + 2 * threadIdx.x;
   const int64_t j0 = (int64_t)blockIdx.y * chunk, j1 = min(j0 + chunk, n);
@@ -190,7 +199,8 @@ template <int K>
 __global__ void __launch_bounds__(kGemvThreads) gemv32_partial_kernel(int64_t n, const float* __restrict__ A32,
                                                                       int64_t ld32, const double* __restrict__ X,
                                                                       int64_t ldx, int64_t chunk,
-                                                                      double* __restrict__ P) {
+                                                                      double* __restrict__ P, Gate gate) {
+  if (gate.closed()) return;
   __shared__ double xs[kGemvChunkElems];
   const int64_t i = (int64_t)blockIdx.x * kGemv32Rows + 4 * threadIdx.x;
   const int64_t j0 = (int64_t)blockIdx.y * chunk, j1 = min(j0 + chunk, n);
@@ -261,7 +271,8 @@ constexpr int kFinRows = 32, kFinGroups = 8;   // rows of a CTA, threads that sh
 __global__ void __launch_bounds__(kFinRows * kFinGroups)
 gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P, const double* __restrict__ B,
                    int64_t ldb, double* __restrict__ out, int64_t ldo, const double* __restrict__ X, int64_t ldx,
-                   int abs_mode, const void* __restrict__ RS, RhsState* st, int track_norms, GemvSplit split) {
+                   int abs_mode, const void* __restrict__ RS, RhsState* st, int track_norms, GemvSplit split, Gate gate) {
+  if (gate.closed()) return;
   __shared__ double sh[2][kFinGroups][kFinRows];
   const int tx = threadIdx.x % kFinRows, ty = threadIdx.x / kFinRows;
   const int64_t i = (int64_t)blockIdx.x * kFinRows + tx;
@@ -326,7 +337,8 @@ __device__ inline double block_sum(double v, double* sh) {
 // (into hn, as a square root) when i == j + 1.
 __global__ void __launch_bounds__(256) mgs_kernel(int64_t n, int K, int m, int j, int i, double* W, int64_t ldw,
                                                   const double* V, int64_t ldv_col, int64_t ldv_rhs,
-                                                  RhsState* st, double* partials, unsigned int* counter) {
+                                                  RhsState* st, double* partials, unsigned int* counter, Gate gate) {
+  if (gate.closed()) return;
   __shared__ double sh[32];
   __shared__ bool last;
   for (int r = 0; r < K; ++r) {
@@ -573,10 +585,12 @@ __global__ void update_kernel(int64_t n, int K, double* X, int64_t ldx, const do
 // Host side
 // ---------------------------------------------------------------------------
 struct SolveWs {
+  Report* report;    // the solve's words for the host; status and brief point into it
   uint32_t* status;
   RhsState* st;
   Brief* brief;
   unsigned int* counter;
+  size_t control_bytes;   // report .. counter, zeroed at the start of a solve
   double* partials;  // kMaxK * kRedBlocks
   double* r;         // n x K
   double* w;         // n x K
@@ -613,10 +627,12 @@ SolveWs carve_solve(void* base, int64_t n, int64_t K, int m) {
     return p;
   };
   const int nchunk = gemv_chunks(n);
-  w.status = (uint32_t*)take(256);
+  w.report = (Report*)take(sizeof(Report));
+  w.status = (uint32_t*)w.report;
+  w.brief = base ? w.report->brief : nullptr;
   w.st = (RhsState*)take(sizeof(RhsState) * kMaxK);
-  w.brief = (Brief*)take(sizeof(Brief) * kMaxK);
   w.counter = (unsigned int*)take(256);
+  w.control_bytes = off;
   w.partials = (double*)take(sizeof(double) * kMaxK * kRedBlocks);
   w.r = (double*)take(sizeof(double) * n * K);
   w.w = (double*)take(sizeof(double) * n * K);
@@ -636,7 +652,7 @@ SolveWs carve_solve(void* base, int64_t n, int64_t K, int m) {
 // product (from w.a32 when there is one)
 template <int K>
 cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int64_t ldx, int abs_mode,
-                   const SolveWs& w, int nchunk, cudaStream_t st) {
+                   const SolveWs& w, int nchunk, cudaStream_t st, Gate gate) {
   const int64_t chunk = cdiv<int64_t>(n, nchunk);
   if (chunk * K > kGemvChunkElems) return cudaErrorInvalidValue;
   dim3 grid((unsigned)cdiv<int64_t>(n, kGemvRows), (unsigned)nchunk);
@@ -645,15 +661,15 @@ cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int
   void* RS = w.RS;
   if (abs_mode == 3 && w.a32) {
     dim3 g32((unsigned)cdiv<int64_t>(n, kGemv32Rows), (unsigned)nchunk);
-    gemv32_partial_kernel<K><<<g32, T, 0, st>>>(n, w.a32, w.ld32, X, ldx, chunk, P);
+    gemv32_partial_kernel<K><<<g32, T, 0, st>>>(n, w.a32, w.ld32, X, ldx, chunk, P, gate);
   } else if (abs_mode == 3) {
-    gemv_partial_kernel<K, 0, true><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS);
+    gemv_partial_kernel<K, 0, true><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
   } else if (abs_mode == 0) {
-    gemv_partial_kernel<K, 0><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS);
+    gemv_partial_kernel<K, 0><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
   } else if (abs_mode == 1) {
-    gemv_partial_kernel<K, 1><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, w.a32, w.ld32, P, RS);
+    gemv_partial_kernel<K, 1><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, w.a32, w.ld32, P, RS, gate);
   } else {
-    gemv_partial_kernel<K, 2><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS);
+    gemv_partial_kernel<K, 2><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
   }
   return cudaGetLastError();
 }
@@ -679,7 +695,7 @@ bool gemv_on_tensor_cores(int64_t n, int K, const double* A, int64_t lda, int ab
 // out = b - A X (b may be NULL: out = -A X), with optional norm tracking.
 cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx,
                      const double* B, int64_t ldb, double* out, int64_t ldo, int abs_mode, int track,
-                     const SolveWs& w, cudaStream_t st) {
+                     const SolveWs& w, cudaStream_t st, Gate gate = {}) {
   int nchunk = gemv_chunks(n, K);
   cudaError_t e;
   void* tok = prof_begin(st);
@@ -687,22 +703,22 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
   if (gemv_on_tensor_cores(n, K, A, lda, abs_mode, w, &split)) {
     // the digits live in the upper half of the row-sum scratch (fp64-sized; mode 1 keeps fp32 sums)
     void* prep = (char*)w.RS + round_up<size_t>(sizeof(float) * (size_t)gemv_chunks(n) * n, 256);
-    e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st);
+    e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st, gate);
   } else {
     switch (K) {
-      case 1: e = gemv_k<1>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-      case 2: e = gemv_k<2>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-      case 3: e = gemv_k<3>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-      case 4: e = gemv_k<4>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-      case 5: e = gemv_k<5>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-      case 6: e = gemv_k<6>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-      case 7: e = gemv_k<7>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
-      default: e = gemv_k<8>(n, A, lda, X, ldx, abs_mode, w, nchunk, st); break;
+      case 1: e = gemv_k<1>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
+      case 2: e = gemv_k<2>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
+      case 3: e = gemv_k<3>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
+      case 4: e = gemv_k<4>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
+      case 5: e = gemv_k<5>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
+      case 6: e = gemv_k<6>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
+      case 7: e = gemv_k<7>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
+      default: e = gemv_k<8>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
     }
   }
   if (e != cudaSuccess) return e;
   gemv_finish_kernel<<<dim3((unsigned)cdiv<int64_t>(n, kFinRows), K), kFinRows * kFinGroups, 0, st>>>(
-      n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split);
+      n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split, gate);
   prof_end(tok, abs_mode == 3 ? kProfGemv32 : kProfGemv, 8.0 * (double)n * (double)n, st);
   count_launches(2);
   return cudaGetLastError();
@@ -722,15 +738,21 @@ struct Solver {
   cudaStream_t st;
   int epoch = 0;
   PrecondPlan plan;
-  Brief brief[kMaxK];
+  Report rep;
+
+  size_t report_bytes() const { return offsetof(Report, brief) + sizeof(Brief) * K; }
+  // Gates of launches issued ahead of the host's knowledge: some right-hand side
+  // still wants refinement / Arnoldi steps
+  Gate outer_gate() const { return {&w.st->outer_active, K, (int)(sizeof(RhsState) / sizeof(int))}; }
+  Gate cycle_gate() const { return {&w.st->cycle_active, K, (int)(sizeof(RhsState) / sizeof(int))}; }
 
   int64_t ldv_rhs() const { return n * (m + 1); }
 
-  cudaError_t precond(const double* v, int64_t ldv, double* z, int64_t ldz) {
+  cudaError_t precond(const double* v, int64_t ldv, double* z, int64_t ldz, Gate gate = {}) {
     ++epoch;
     void* tok = prof_begin(st);
     const cudaError_t e = precond_launch(plan, prm.precond_fp32 != 0, K, n, LU, ldlu, fmt, w.dinv, w.chain, v, ldv, z,
-                                         ldz, w.pub, epoch, w.status, rs, cs, st);
+                                         ldz, w.pub, epoch, w.status, rs, cs, st, gate);
     prof_end(tok, kProfPrecond, 2.0 * (double)n * (double)n, st);
     count_launches(1);
     return e;
@@ -738,13 +760,10 @@ struct Solver {
 
   // CTAs of the reductions over n: no more than hold an entry per thread
   int red_blocks() const { return (int)std::min<int64_t>(kRedBlocks, cdiv<int64_t>(n, 256)); }
-  cudaError_t read_brief() {
-    return read_to_host(brief, w.brief, sizeof(Brief) * K, st);
-  }
   // Arnoldi step j after w = M^{-1} A v_j: modified Gram-Schmidt, the Givens
   // update (into the brief) and v_{j+1}; one launch for small systems, else one
   // launch per projection, then the rotation and the scaling
-  void arnoldi_tail(int j) {
+  void arnoldi_tail(int j, Gate gate) {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     if (n * K <= kFusedMgsMaxElems) {
       arnoldi_tail_kernel<<<K, kFusedMgsThreads, 0, st>>>(sp, n, m, j, w.w, n, w.V, n, ldv_rhs(), w.st, w.brief);
@@ -752,7 +771,8 @@ struct Solver {
       return;
     }
     for (int i = 0; i <= j + 1; ++i)
-      mgs_kernel<<<red_blocks(), 256, 0, st>>>(n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st, w.partials, w.counter);
+      mgs_kernel<<<red_blocks(), 256, 0, st>>>(n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st, w.partials, w.counter,
+                                               gate);
     givens_kernel<<<1, 32, 0, st>>>(sp, j, w.st, w.brief);
     scale_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, w.w, n, w.V + (int64_t)(j + 1) * n, ldv_rhs(),
                                                                    w.st, 1);
@@ -760,7 +780,7 @@ struct Solver {
   }
   bool any(int Brief::*f) const {
     for (int r = 0; r < K; ++r)
-      if (brief[r].*f) return true;
+      if (rep.brief[r].*f) return true;
     return false;
   }
 
@@ -773,55 +793,84 @@ struct Solver {
     if (!precond_plan(n, K, fp32, sms, sm_budget(), &plan)) return cudaErrorInvalidValue;
     if ((e = cudaMemsetAsync(w.pub, 0, precond_pub_bytes(n, K), st)) != cudaSuccess) return e;
     if ((e = precond_setup(n, LU, ldlu, fmt, fp32, w.dinv, w.chain, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(w.st, 0, sizeof(RhsState) * kMaxK, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(w.counter, 0, 256, st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(w.status, 0, 4, st)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(w.report, 0, w.control_bytes, st)) != cudaSuccess) return e;
     init_kernel<<<1, 32, 0, st>>>(K, w.st);
     count_launches(1);
     return cudaGetLastError();
   }
 
+  // z = M^{-1} r, beta, v0 = z / beta
+  // ahead (here and below): issued before the host knows that it is wanted
+  cudaError_t cycle_start(bool ahead) {
+    const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
+    const cudaError_t e = precond(w.r, n, w.tmp, n, ahead ? outer_gate() : Gate{});
+    if (e != cudaSuccess) return e;
+    norm2_kernel<<<red_blocks(), 256, 0, st>>>(n, K, w.tmp, n, w.st, w.partials, w.counter);
+    cycle_start_kernel<<<1, 32, 0, st>>>(sp, w.st, w.brief);
+    scale_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, w.tmp, n, w.V, ldv_rhs(), w.st, 0);
+    count_launches(3);
+    return cudaGetLastError();
+  }
+  // w = M^{-1} (A v_j), orthogonalised; the product in fp32 or fp64 as matvec_fp32 says
+  cudaError_t arnoldi_step(int j, bool ahead) {
+    const Gate gate = ahead ? cycle_gate() : Gate{};
+    cudaError_t e = residual(n, K, A, lda, w.V + (int64_t)j * n, ldv_rhs(), nullptr, 0, w.tmp, n,
+                             prm.matvec_fp32 ? 3 : 0, 0, w, st, gate);
+    if (e != cudaSuccess) return e;
+    if ((e = precond(w.tmp, n, w.w, n, gate)) != cudaSuccess) return e;
+    arnoldi_tail(j, gate);
+    return cudaGetLastError();
+  }
+  // x += V y
+  cudaError_t cycle_finish() {
+    const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
+    cycle_finish_kernel<<<1, 32, 0, st>>>(sp, w.st);
+    update_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, X, ldx, w.V, n, ldv_rhs(), w.st);
+    count_launches(2);
+    return cudaGetLastError();
+  }
+  // r = b - A x, norms; decide
+  cudaError_t outer_check(bool first) {
+    const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
+    const cudaError_t e = residual(n, K, A, lda, X, ldx, B, ldb, w.r, n, first ? 1 : 0, 1, w, st);
+    if (e != cudaSuccess) return e;
+    check_kernel<<<1, 32, 0, st>>>(sp, w.st, w.brief, first ? 1 : 0);
+    count_launches(1);
+    return cudaGetLastError();
+  }
+
+  // The decisions are made on the device (RhsState); the host learns them by
+  // reading the report, 15 to 20 us in which the GPU idles.  The first cycle
+  // does not wait for the first check, and no cycle's first Arnoldi step waits
+  // for the cycle's start: either is wanted as a rule, and its gates close where
+  // it is not.  Issuing the later steps ahead as well gained nothing: the step
+  // after a cycle's last one costs 25 us (n = 1024) to 90 us with its gates
+  // closed.  628 -> 574 us at n = 1024; 24 mixed systems in one batch 9.30 -> 8.83
+  // ms.  With the kernel timers on, nothing is issued ahead.
   cudaError_t run() {
+    const bool ahead = !prof_on();
+    auto report = [&] { return read_to_host(&rep, w.report, report_bytes(), st); };
     cudaError_t e = setup();
     if (e != cudaSuccess) return e;
-    SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
-
-    // x0 = U^{-1} L^{-1} b
-    if ((e = precond(B, ldb, X, ldx)) != cudaSuccess) return e;
-    bool first = true;
-    for (;;) {
-      // r = b - A x, norms; decide
-      if ((e = residual(n, K, A, lda, X, ldx, B, ldb, w.r, n, first ? 1 : 0, 1, w, st)) != cudaSuccess) return e;
-      check_kernel<<<1, 32, 0, st>>>(sp, w.st, w.brief, first ? 1 : 0);
-      count_launches(1);
-      first = false;
-      if ((e = read_brief()) != cudaSuccess) return e;
-      if (!any(&Brief::outer_active)) break;
-      // cycle start: z = M^{-1} r, beta, v0 = z / beta
-      if ((e = precond(w.r, n, w.tmp, n)) != cudaSuccess) return e;
-      norm2_kernel<<<red_blocks(), 256, 0, st>>>(n, K, w.tmp, n, w.st, w.partials, w.counter);
-      cycle_start_kernel<<<1, 32, 0, st>>>(sp, w.st, w.brief);
-      scale_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, w.tmp, n, w.V, ldv_rhs(), w.st, 0);
-      count_launches(3);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-      if ((e = read_brief()) != cudaSuccess) return e;
-      if (!any(&Brief::outer_active)) break;
-      for (int j = 0; j < m && any(&Brief::cycle_active); ++j) {
-        // w = M^{-1} (A v_j); the product in fp32 or fp64 as matvec_fp32 says
-        if ((e = residual(n, K, A, lda, w.V + (int64_t)j * n, ldv_rhs(), nullptr, 0, w.tmp, n,
-                          prm.matvec_fp32 ? 3 : 0, 0, w, st)) != cudaSuccess)
-          return e;
-        if ((e = precond(w.tmp, n, w.w, n)) != cudaSuccess) return e;
-        arnoldi_tail(j);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = read_brief()) != cudaSuccess) return e;
+    if ((e = precond(B, ldb, X, ldx)) != cudaSuccess) return e;   // x0 = U^{-1} L^{-1} b
+    for (bool first = true;; first = false) {
+      if ((e = outer_check(first)) != cudaSuccess) return e;
+      if (!(first && ahead)) {   // a later check is the last one as a rule
+        if ((e = report()) != cudaSuccess) return e;
+        if (!any(&Brief::outer_active)) return cudaSuccess;
       }
-      cycle_finish_kernel<<<1, 32, 0, st>>>(sp, w.st);
-      update_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, X, ldx, w.V, n, ldv_rhs(), w.st);
-      count_launches(2);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      if ((e = cycle_start(first && ahead)) != cudaSuccess) return e;
+      if (!ahead) {
+        if ((e = report()) != cudaSuccess) return e;
+        if (!any(&Brief::outer_active)) return cudaSuccess;
+      }
+      for (int j = 0; j < m && ((j == 0 && ahead) || any(&Brief::cycle_active)); ++j) {
+        if ((e = arnoldi_step(j, j == 0 && ahead)) != cudaSuccess) return e;
+        if ((e = report()) != cudaSuccess) return e;
+        if (j == 0 && ahead && !any(&Brief::outer_active)) return cudaSuccess;
+      }
+      if ((e = cycle_finish()) != cudaSuccess) return e;
     }
-    return cudaSuccess;
   }
 };
 
@@ -890,21 +939,17 @@ hpmxp_status solve_ir(int64_t n, const double* A, int64_t lda, const void* LU, i
   s.st = st;
   cudaError_t e = s.run();
   if (e != cudaSuccess) return status_from_cuda(e);
-  uint32_t word = 0;
-  e = read_to_host(&word, s.w.status, 4, st);
-  if (e == cudaSuccess) e = s.read_brief();
-  if (e != cudaSuccess) return status_from_cuda(e);
-  if (word) return status_from_word(word);
+  if (s.rep.status) return status_from_word(s.rep.status);
   int worst = HPMXP_OK;
   for (int r = 0; r < s.K; ++r) {
     if (info) {
-      info[r].iters = s.brief[r].iters;
-      info[r].outer = s.brief[r].outer;
-      info[r].scaled_resid = s.brief[r].sr;
-      info[r].status = s.brief[r].status;
+      info[r].iters = s.rep.brief[r].iters;
+      info[r].outer = s.rep.brief[r].outer;
+      info[r].scaled_resid = s.rep.brief[r].sr;
+      info[r].status = s.rep.brief[r].status;
       info[r].reserved = 0;
     }
-    if (s.brief[r].status != HPMXP_OK && worst == HPMXP_OK) worst = s.brief[r].status;
+    if (s.rep.brief[r].status != HPMXP_OK && worst == HPMXP_OK) worst = s.rep.brief[r].status;
   }
   return (hpmxp_status)worst;
 }
@@ -942,7 +987,7 @@ StreamPool& stream_pool(int dev) {
   return p;
 }
 
-enum Phase { kResid, kCycle, kArnoldi, kDone };
+enum Phase { kResid, kCycle, kArnoldi, kDone };   // kCycle with Arnoldi step 0 where that is issued ahead
 
 struct BatchItem {
   Solver s;
@@ -951,7 +996,7 @@ struct BatchItem {
   bool first = true;    // the first residual also takes ||A||
   bool finish = false;  // cycle_finish + update to issue before the next residual
   cudaEvent_t ev = nullptr;
-  Brief* host = nullptr;   // pinned copy of the brief
+  Report* host = nullptr;   // pinned copy of the report
 };
 
 size_t batch_solve_bytes(const hpmxp_problem* probs, int count, int restart) {
@@ -975,7 +1020,7 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
   std::lock_guard<std::mutex> lk(pool.mu);   // one batched solve drives a device's pool at a time
   // pinned briefs and per-system events, kept by the calling thread
   struct HostSide {
-    Brief* pinned = nullptr;
+    Report* pinned = nullptr;
     size_t cap = 0;
     std::vector<cudaEvent_t> ev;
     ~HostSide() {
@@ -984,12 +1029,12 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
     }
   };
   thread_local HostSide hs;
-  const size_t need = (size_t)count * kMaxK;
+  const size_t need = (size_t)count;
   if (hs.cap < need) {
     if (hs.pinned) cudaFreeHost(hs.pinned);
     hs.pinned = nullptr;
     hs.cap = 0;
-    if ((e = cudaMallocHost(&hs.pinned, sizeof(Brief) * need)) != cudaSuccess) return status_from_cuda(e);
+    if ((e = cudaMallocHost(&hs.pinned, sizeof(Report) * need)) != cudaSuccess) return status_from_cuda(e);
     hs.cap = need;
   }
   while ((int)hs.ev.size() < count) {
@@ -1010,7 +1055,7 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
     base += round_up<size_t>(s.w.bytes, 256);
     s.st = pool.st[q % kPoolStreams];
     it[q].ev = hs.ev[q];
-    it[q].host = hs.pinned + (size_t)q * kMaxK;
+    it[q].host = hs.pinned + q;
   }
   // fork from the caller's stream
   cudaEvent_t fork_ev = pool.ev[0];
@@ -1023,9 +1068,10 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
   }
   auto any = [](const BatchItem& b, int Brief::*f) {
     for (int r = 0; r < b.s.K; ++r)
-      if (b.host[r].*f) return true;
+      if (b.host->brief[r].*f) return true;
     return false;
   };
+  const bool ahead = !prof_on();
   int active = count;
   while (active > 0 && e == cudaSuccess) {
     // issue every active system's next phase
@@ -1033,38 +1079,26 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
       BatchItem& b = it[q];
       if (b.ph == kDone) continue;
       Solver& s = b.s;
-      const SolveParams sp{s.K, s.m, s.prm.max_iters, s.prm.inner_tol, s.prm.theta, s.prm.accept, s.n};
-      const cudaStream_t st = s.st;
       if (b.finish) {
-        cycle_finish_kernel<<<1, 32, 0, st>>>(sp, s.w.st);
-        update_kernel<<<(unsigned)cdiv<int64_t>(s.n, 256), 256, 0, st>>>(s.n, s.K, s.X, s.ldx, s.w.V, s.n,
-                                                                         s.ldv_rhs(), s.w.st);
-        count_launches(2);
+        e = s.cycle_finish();
         b.finish = false;
       }
+      if (e != cudaSuccess) break;
+      bool unchecked = false;
       if (b.ph == kResid) {
-        e = residual(s.n, s.K, s.A, s.lda, s.X, s.ldx, s.B, s.ldb, s.w.r, s.n, b.first ? 1 : 0, 1, s.w, st);
-        check_kernel<<<1, 32, 0, st>>>(sp, s.w.st, s.w.brief, b.first ? 1 : 0);
-        count_launches(1);
+        e = s.outer_check(b.first);
+        unchecked = b.first && ahead;
+        if (unchecked) b.ph = kCycle;   // what Solver::run issues ahead
         b.first = false;
-      } else if (b.ph == kCycle) {
-        e = s.precond(s.w.r, s.n, s.w.tmp, s.n);
-        norm2_kernel<<<s.red_blocks(), 256, 0, st>>>(s.n, s.K, s.w.tmp, s.n, s.w.st, s.w.partials, s.w.counter);
-        cycle_start_kernel<<<1, 32, 0, st>>>(sp, s.w.st, s.w.brief);
-        scale_kernel<<<(unsigned)cdiv<int64_t>(s.n, 256), 256, 0, st>>>(s.n, s.K, s.w.tmp, s.n, s.w.V, s.ldv_rhs(),
-                                                                         s.w.st, 0);
-        count_launches(3);
-      } else {   // Arnoldi step j
-        const int j = b.j;
-        e = residual(s.n, s.K, s.A, s.lda, s.w.V + (int64_t)j * s.n, s.ldv_rhs(), nullptr, 0, s.w.tmp, s.n,
-                     s.prm.matvec_fp32 ? 3 : 0, 0, s.w, st);
-        if (e == cudaSuccess) e = s.precond(s.w.tmp, s.n, s.w.w, s.n);
-        s.arnoldi_tail(j);
+      } else if (b.ph == kArnoldi) {
+        e = s.arnoldi_step(b.j, false);
       }
-      if (e == cudaSuccess) e = cudaGetLastError();
-      if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b.host, s.w.brief, sizeof(Brief) * s.K, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaEventRecord(b.ev, st);
+      if (e == cudaSuccess && b.ph == kCycle) {
+        e = s.cycle_start(unchecked);
+        if (e == cudaSuccess && ahead) e = s.arnoldi_step(0, true);
+      }
+      if (e == cudaSuccess) e = cudaMemcpyAsync(b.host, s.w.report, s.report_bytes(), cudaMemcpyDeviceToHost, s.st);
+      if (e == cudaSuccess) e = cudaEventRecord(b.ev, s.st);
     }
     if (e != cudaSuccess) break;
     // one decision point for the batch
@@ -1077,9 +1111,9 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
       } else if (b.ph == kCycle) {
         if (!any(b, &Brief::outer_active)) {
           b.ph = kDone;
-        } else if (any(b, &Brief::cycle_active) && b.s.m > 0) {
+        } else if (any(b, &Brief::cycle_active) && b.s.m > (ahead ? 1 : 0)) {
           b.ph = kArnoldi;
-          b.j = 0;
+          b.j = ahead ? 1 : 0;
         } else {
           b.finish = true;
           b.ph = kResid;
@@ -1104,18 +1138,17 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
   int64_t off = 0;
   for (int q = 0; q < count; ++q) {
     BatchItem& b = it[q];
-    uint32_t word = 0;
-    if ((e = read_to_host(&word, b.s.w.status, 4, caller)) != cudaSuccess) return status_from_cuda(e);
-    if (word && worst == HPMXP_OK) worst = status_from_word(word);
+    // the status word came with the last report
+    if (b.host->status && worst == HPMXP_OK) worst = status_from_word(b.host->status);
     for (int r = 0; r < b.s.K; ++r) {
       if (info) {
-        info[off + r].iters = b.host[r].iters;
-        info[off + r].outer = b.host[r].outer;
-        info[off + r].scaled_resid = b.host[r].sr;
-        info[off + r].status = b.host[r].status;
+        info[off + r].iters = b.host->brief[r].iters;
+        info[off + r].outer = b.host->brief[r].outer;
+        info[off + r].scaled_resid = b.host->brief[r].sr;
+        info[off + r].status = b.host->brief[r].status;
         info[off + r].reserved = 0;
       }
-      if (b.host[r].status != HPMXP_OK && worst == HPMXP_OK) worst = b.host[r].status;
+      if (b.host->brief[r].status != HPMXP_OK && worst == HPMXP_OK) worst = b.host->brief[r].status;
     }
     off += b.s.K;
   }

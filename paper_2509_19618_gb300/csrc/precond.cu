@@ -291,6 +291,7 @@ struct PrecondArgs {
   unsigned long long wait_ns;
   const double* rs;
   const double* cs;
+  Gate gate;
 };
 
 template <class T, int K>
@@ -303,6 +304,7 @@ __global__ void __launch_bounds__(2 * kGrp) precond_kernel(PrecondArgs p) {
   constexpr int kR = sizeof(T) == 8 ? 1 : K <= 3 ? 4 : 2, kRB = sizeof(T) == 8 ? 2 : kR;
   constexpr int kQ = K * sizeof(T) <= 16 || (sizeof(T) == 8 && K <= 4) ? 4 : K % 2 == 0 || sizeof(T) == 8 ? 2 : 1;   // columns of a run
   constexpr int kUnroll = K * sizeof(T) <= 8 ? 4 : sizeof(T) == 4 || K == 2 ? 2 : 1;   // runs read ahead, against registers
+  if (p.gate.closed()) return;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ volatile int ready;   // owned blocks of the sweep whose updates are complete
   const int nb = (int)cdiv<int64_t>(p.n, TB);
@@ -725,10 +727,10 @@ cudaError_t precond_setup(int64_t n, const uint16_t* LU, int64_t ld, int fmt, bo
 cudaError_t precond_launch(const PrecondPlan& plan, bool fp32, int K, int64_t n, const uint16_t* LU, int64_t ld,
                            int fmt, const void* dinv, const void* chain, const double* v, int64_t ldv, double* z,
                            int64_t ldz, void* pub, int epoch, uint32_t* status, const double* rs, const double* cs,
-                           cudaStream_t st) {
+                           cudaStream_t st, Gate gate) {
   const WaitBudget wb = wait_budget();
   const PrecondArgs a{n, LU, ld, fmt, dinv, chain, v, ldv, z, ldz, (unsigned long long*)pub, epoch,
-                      plan.p1_smem ? 1 : 0, status, wb.polls, wb.ns, rs, cs};
+                      plan.p1_smem ? 1 : 0, status, wb.polls, wb.ns, rs, cs, gate};
   return fp32 ? launch<float>(K, a, plan, st) : launch<double>(K, a, plan, st);
 }
 
