@@ -125,6 +125,7 @@ __device__ inline void tmem_ld64(uint32_t taddr, uint32_t (&r)[64]) {
 struct TcParams {
   int M, N, nkb;          // output rows, columns, K stages (128 bytes of K each)
   int tiles_i, ntiles;
+  int split;              // tiles from here on belong to the launch's second product (TcSecond)
   int mode;
   float sign;
   int fmt;
@@ -143,6 +144,15 @@ struct TcParams {
   // all-ones minus the latest CTA end (global timer, ns; both kept by
   // atomicMin from all-ones), NULL when not measured
   unsigned long long* span;
+};
+
+// The second of two independent products of one launch (same depth, mode and
+// types): the row panel and the column panel of a step, 128 wide each, would
+// otherwise take turns, 7 us for a second launch of a few tiles.
+struct TcSecond {
+  CUtensorMap a, b, c;
+  int M, N, tiles_i;
+  uint16_t* R; int64_t ldr;
 };
 
 // Two floats rounded to nearest even into one 32-bit word of 16-bit values (lo
@@ -169,7 +179,7 @@ template <int TI, int CB>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, TcParams p, const GemmGroupItem* __restrict__ items,
-               int nitems) {
+               int nitems, const __grid_constant__ TcSecond second) {
   using Cfg = TileCfg<TI, CB>;
   constexpr int kStages = Cfg::kStages, kStageB = Cfg::kStageB, kCTile = Cfg::kCTile, kCBufs = Cfg::kCBufs;
   constexpr int kBoxes = Cfg::kBoxes, kBoxRows = Cfg::kBoxRows;
@@ -195,7 +205,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   // tile t -> its product (grouped launch: the last item starting at or before t)
   auto locate = [&](int t) {
     TileLoc L;
-    if (items == nullptr) {
+    if (items == nullptr && t >= p.split) {
+      t -= p.split;
+      L.a = &second.a; L.b = &second.b; L.c = &second.c;
+      L.i0 = (t % second.tiles_i) * TI; L.j0 = (t / second.tiles_i) * kTJ;
+      L.M = second.M; L.N = second.N; L.R = second.R; L.ldr = second.ldr;
+    } else if (items == nullptr) {
       L.a = &tmA; L.b = &tmB; L.c = &tmC;
       L.i0 = (t % p.tiles_i) * TI; L.j0 = (t / p.tiles_i) * kTJ;
       L.M = p.M; L.N = p.N; L.R = p.R; L.ldr = p.ldr;
@@ -547,7 +562,7 @@ int grid_cap() {
 namespace {
 
 template <int TI, int CB = 2>
-cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st) {
+cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st, const GemmArgs* also = nullptr) {
   using Cfg = TileCfg<TI, CB>;
   static_assert(CB == 2 || TI == 128, "fp32 C on 128-row tiles only");
   if (CB == 4 && (g.mode != kEpiSub || g.R || !g.C)) return cudaErrorInvalidValue;
@@ -570,6 +585,19 @@ cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st) {
   p.M = g.M; p.N = g.N; p.nkb = (int)(kbytes / kRowBytes);
   p.tiles_i = cdiv(g.M, TI);
   p.ntiles = p.tiles_i * cdiv(g.N, kTJ);
+  p.split = p.ntiles;
+  TcSecond second{};
+  if (also) {
+    const GemmArgs& h = *also;
+    if (h.fp8 || h.c32 || h.K != g.K || h.mode != g.mode || h.sign != g.sign || h.fmt != g.fmt || !h.C || !g.C ||
+        !make_map(&second.a, h.A, kbytes / 2, (uint64_t)h.M, (uint64_t)h.lda * esz, kRowBytes / 2, TI) ||
+        !make_map(&second.b, h.B, kbytes / 2, (uint64_t)h.N, (uint64_t)h.ldb * esz, kRowBytes / 2, kTJ) ||
+        !make_map(&second.c, h.C, (uint64_t)h.M, (uint64_t)h.N, (uint64_t)h.ldc * CB, Cfg::kBoxRows, kTJ, CB == 4))
+      return cudaErrorInvalidValue;
+    second.M = h.M; second.N = h.N; second.tiles_i = cdiv(h.M, TI);
+    second.R = (uint16_t*)h.R; second.ldr = h.ldr;
+    p.ntiles += second.tiles_i * cdiv(h.N, kTJ);
+  }
   p.mode = g.mode; p.sign = g.sign; p.fmt = g.fmt; p.fp8 = g.fp8;
   p.R = (uint16_t*)g.R; p.ldr = g.ldr;
   p.sA = g.sA; p.sa_ld = g.sa_ld; p.sB = g.sB; p.sb_ld = g.sb_ld;
@@ -598,17 +626,21 @@ cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st) {
     configured_for.store(dev);
   }
   const int grid = std::min(p.ntiles, g.max_ctas > 0 ? std::min(g.max_ctas, grid_cap()) : grid_cap());
-  const double flops = 2.0 * g.M * (double)g.N * g.K;
   // algorithmic DRAM bytes: both operands once, C read (subtract mode) and
   // written once, the optional row-major copy written once
-  const double mn = (double)g.M * (double)g.N;
-  const double bytes = ((double)g.M + (double)g.N) * (double)g.K * esz +
-                       (p.has_c ? mn * CB * (g.mode == kEpiSub ? 2.0 : 1.0) : 0.0) + (g.R ? mn * 2.0 : 0.0);
+  double flops = 0.0, bytes = 0.0;
+  for (const GemmArgs* h : {&g, also}) {
+    if (!h) continue;
+    const double mn = (double)h->M * (double)h->N;
+    flops += 2.0 * mn * h->K;
+    bytes += ((double)h->M + (double)h->N) * (double)h->K * esz +
+             (p.has_c ? mn * CB * (h->mode == kEpiSub ? 2.0 : 1.0) : 0.0) + (h->R ? mn * 2.0 : 0.0);
+  }
   void* tok = prof_begin(st);
   p.span = prof_device_span(tok);
   const cudaError_t e =
       launch_pdl(gemm_tc_kernel<TI, CB>, dim3(grid), dim3(kThreads), Cfg::kSmem, st, ta, tb, tc, p,
-                 (const GemmGroupItem*)nullptr, 0);
+                 (const GemmGroupItem*)nullptr, 0, second);
   prof_end(tok, g.mode == kEpiSub ? kProfGemm : kProfGemmStore, flops, st, bytes);
   count_launches(1);
   return e;
@@ -635,7 +667,7 @@ bool gemm_group_encode(const GemmArgs* gs, int count, GemmGroupItem* items, int*
   for (int c = 0; c < count; ++c) {
     const GemmArgs& g = gs[c];
     if (g.fp8 || g.c32 || g.K <= 0 || g.K >= 256 || (g.K % 128) || g.K != gs[0].K || g.mode != gs[0].mode ||
-        (!g.R) != (!gs[0].R) || !g.C || g.M <= 0 || g.N <= 0)
+        !g.C || g.M <= 0 || g.N <= 0)
       return false;
     const uint64_t kbytes = (uint64_t)g.K * 2;
     CUtensorMap* ta = reinterpret_cast<CUtensorMap*>(items[c].maps[0]);
@@ -665,7 +697,7 @@ cudaError_t gemm_tc_grouped(const GemmArgs& g, const GemmGroupItem* dev_items, i
   p.has_c = 1;
   p.nkb = (int)((uint64_t)g.K * 2 / kRowBytes);
   p.tiles_i = 1;
-  p.ntiles = total_tiles;
+  p.ntiles = p.split = total_tiles;
   p.mode = g.mode; p.sign = g.sign; p.fmt = g.fmt; p.fp8 = 0;
   p.status = g.status;
   const WaitBudget wb = wait_budget();
@@ -689,7 +721,7 @@ cudaError_t gemm_tc_grouped(const GemmArgs& g, const GemmGroupItem* dev_items, i
   void* tok = prof_begin(st);
   p.span = prof_device_span(tok);
   const cudaError_t e = launch_pdl(gemm_tc_kernel<128, 2>, dim3(grid), dim3(kThreads), Cfg::kSmem, st, none, none,
-                                   none, p, dev_items, nitems);
+                                   none, p, dev_items, nitems, TcSecond{});
   prof_end(tok, g.mode == kEpiSub ? kProfGemm : kProfGemmStore, flops, st, bytes);
   count_launches(1);
   return e;
@@ -710,6 +742,14 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   // enough depth (K >= 256) for one C buffer to keep up
   if (!g.fp8 && g.M >= 256 && g.K >= 256 && wide_tiles_enabled()) return gemm_tc_tiles<256>(g, st);
   return gemm_tc_tiles<128>(g, st);
+}
+
+// Two independent 16-bit products of the same depth in one launch, on 128-row
+// tiles (either may be empty).
+cudaError_t gemm_tc_pair(const GemmArgs& g, const GemmArgs& h, cudaStream_t st) {
+  if (g.M <= 0 || g.N <= 0) return gemm_tc(h, st);
+  if (h.M <= 0 || h.N <= 0) return gemm_tc(g, st);
+  return gemm_tc_tiles<128>(g, st, &h);
 }
 
 }  // namespace hpmxp

@@ -144,6 +144,7 @@ struct GemmArgs {
   int c32;              // 1: C is fp32 column major (ldc in elements), mode kEpiSub: C = fl32(C - acc)
 };
 cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st);
+cudaError_t gemm_tc_pair(const GemmArgs& g, const GemmArgs& h, cudaStream_t st);   // two products of one depth, one launch
 cudaError_t gemm_simt(const GemmArgs& g, cudaStream_t st);
 
 // Tensor map of a column-major fp64 matrix (rows x cols, 16-byte aligned
