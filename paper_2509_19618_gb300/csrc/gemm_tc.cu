@@ -15,8 +15,8 @@
 //
 // Roles: warp 0 TMA producer of the operand ring; warp 1 TMEM owner and MMA
 // issuer; warps 2..9 epilogue in two groups of four (warp w reads TMEM lanes
-// 32*(w%4)..+31; group g takes rows TI/2 g .. of the tile), which also
-// prefetch C tiles ahead and issue the TMA stores.
+// 32*(w%4)..+31; group g takes rows TI/2 g .. of the tile); warps 10 and 11
+// move the groups' C: loads ahead, stores behind, by 64-row segments.
 // Accumulators are double buffered in TMEM (single buffered for 4-slice FP8),
 // so the epilogue of one tile overlaps the MMAs of the next.  The E4M3
 // variant keeps one accumulator per 128-deep K slice and folds them with the
@@ -25,9 +25,7 @@
 // Every wait is bounded (a poll count and a global-timer limit passed in
 // TcParams); a wait that runs out sets kErrTimeout in the status word, skips
 // the remaining work and still drains its copies and tensor-core work (with
-// the default bound) and frees tensor memory before the CTA exits.  The four
-// warps of an epilogue group take each tile's go / give-up decision together,
-// so none of them is left waiting at the group's named barrier.
+// the default bound) and frees tensor memory before the CTA exits.
 #include "tcgen05.h"
 
 #include <cudaTypedefs.h>
@@ -47,7 +45,8 @@ constexpr int kStageA = kTJ * kRowBytes;      // MMA A operand: rows j (16 KiB)
 constexpr int kCBox = kTJ * 128;              // one C box: 128 bytes of rows x 128 columns (16 KiB)
 constexpr int kEpiGroups = 2;                 // epilogue groups, one per half of the tile's rows
 constexpr int kEpiThreads = 128;              // threads per epilogue group (one warp per TMEM lane quarter)
-constexpr int kThreads = 64 + kEpiGroups * kEpiThreads;
+constexpr int kEpiWarps = kEpiThreads / 32;
+constexpr int kThreads = 64 + kEpiGroups * (kEpiThreads + 32);   // and one warp per group that moves its C
 
 // Tile height TI (output rows i per tile = MMA N): 128, or 256 for the large
 // 16-bit products, where every operand byte an SM receives feeds twice the
@@ -61,13 +60,14 @@ struct TileCfg {
   static constexpr int kBoxRows = 128 / CB;                 // rows of one 128-byte C box: 64 or 32
   static constexpr int kBoxes = TI / 2 / kBoxRows;          // C boxes per epilogue group
   static constexpr int kCTile = kEpiGroups * kBoxes * kCBox;  // 32, 64 KiB (16-bit) or 64 KiB (fp32)
-  // C tile buffers: with three, one is in the epilogue, one being stored and
-  // one loading; the 256-row and the fp32 tiles have room for one only
+  // C tile buffers; the 256-row and the fp32 tiles have room for one only
   static constexpr int kCBufs = (TI == 128 && CB == 2) ? 3 : 1;
-  static constexpr int kAhead = kCBufs >= 2 ? kCBufs - 1 : 1;   // C prefetch distance (local tiles)
-  static constexpr int kReadWait = kCBufs >= 2 ? kCBufs - 2 : 0; // stores allowed to be still reading
+  static constexpr int kSegs = TI / 128;                    // 64-row segments of an epilogue group's TI/2 rows
+  static constexpr int kSegBoxes = kBoxes / kSegs;          // C boxes of a segment
+  static constexpr int kCSlots = kCBufs * kEpiGroups * kSegs;
+  static constexpr int kBars = 2 * kStages + 5 + 2 * kCSlots;
   static constexpr size_t kSmem = 1024 + (size_t)kStages * (kStageA + kStageB) + (size_t)kCBufs * kCTile +
-                                  8 * (2 * kStages + 5 + 2 * kCBufs) + 16;
+                                  8 * kBars + 16;
 };
 // 227 KB of dynamic shared memory per CTA; two TI-column fp32 accumulators in
 // the 512 TMEM columns; a TMA box is at most 256 rows
@@ -76,21 +76,6 @@ static_assert(TileCfg<128>::kSmem <= 232448 && TileCfg<256>::kSmem <= 232448 && 
 template <int TI>
 constexpr bool tile_fits() { return 2 * TI <= 512 && TI <= 256 && TI % 128 == 0; }
 static_assert(tile_fits<128>() && tile_fits<256>(), "two accumulators in TMEM, one TMA box per stage");
-
-__device__ inline void epi_barrier(int group) {
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + group), "n"(kEpiThreads) : "memory");
-}
-// True for every thread of the epilogue group when v is true for all of them
-// (a barrier of the group's four warps with an AND reduction).
-__device__ inline bool epi_all(int group, bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"((uint32_t)v), "r"(1 + group), "n"(kEpiThreads)
-      : "memory");
-  return r != 0;
-}
 
 // 64 consecutive fp32 columns: two x32 loads in flight, one wait.
 __device__ inline void tmem_ld64(uint32_t taddr, uint32_t (&r)[64]) {
@@ -182,8 +167,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                int nitems, const __grid_constant__ TcSecond second) {
   using Cfg = TileCfg<TI, CB>;
   constexpr int kStages = Cfg::kStages, kStageB = Cfg::kStageB, kCTile = Cfg::kCTile, kCBufs = Cfg::kCBufs;
-  constexpr int kBoxes = Cfg::kBoxes, kBoxRows = Cfg::kBoxRows;
-  constexpr int kSegs = TI / 128;   // 64-row segments of an epilogue group's TI/2 rows
+  constexpr int kBoxes = Cfg::kBoxes, kBoxRows = Cfg::kBoxRows, kSegs = Cfg::kSegs, kSegBoxes = Cfg::kSegBoxes;
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   uint8_t* smem = smem_raw + ((1024u - (raw & 1023u)) & 1023u);   // swizzle atoms need 1024-byte alignment
@@ -196,9 +180,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   auto empty = [&](int s) { return bar0 + 8u * (uint32_t)(kStages + s); };
   auto acc_full = [&](int b) { return bar0 + 8u * (uint32_t)(2 * kStages + b); };
   auto acc_empty = [&](int b) { return bar0 + 8u * (uint32_t)(2 * kStages + 2 + b); };
-  auto c_full = [&](int b, int h) { return bar0 + 8u * (uint32_t)(2 * kStages + 4 + 2 * b + h); };
-  const uint32_t mma_drain = bar0 + 8u * (uint32_t)(2 * kStages + 4 + 2 * kCBufs);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5 + 2 * kCBufs);
+  // segment h of group g in buffer b: its C is there (or the buffer is free, where C is not read);
+  // the epilogue's four warps are done with it
+  auto c_full = [&](int b, int g, int h) {
+    return bar0 + 8u * (uint32_t)(2 * kStages + 4 + (b * kEpiGroups + g) * kSegs + h);
+  };
+  auto c_done = [&](int b, int g, int h) { return c_full(b, g, h) + 8u * (uint32_t)Cfg::kCSlots; };
+  const uint32_t mma_drain = bar0 + 8u * (uint32_t)(Cfg::kBars - 1);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + Cfg::kBars);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -242,12 +231,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int s = 0; s < kStages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
     for (int b = 0; b < 2; ++b) {
       mbar_init(acc_full(b), 1);
-      mbar_init(acc_empty(b), kEpiGroups * kEpiThreads / 32);
+      mbar_init(acc_empty(b), kEpiGroups * kEpiWarps);
     }
-    for (int b = 0; b < kCBufs; ++b) {
-      mbar_init(c_full(b, 0), 1);
-      mbar_init(c_full(b, 1), 1);
-    }
+    for (int b = 0; b < kCBufs; ++b)
+      for (int g = 0; g < kEpiGroups; ++g)
+        for (int h = 0; h < kSegs; ++h) {
+          mbar_init(c_full(b, g, h), 1);
+          mbar_init(c_done(b, g, h), kEpiWarps);
+        }
     mbar_init(mma_drain, 1);
     fence_mbar_init();
     if (items == nullptr) {
@@ -333,52 +324,102 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       tc_commit(mma_drain);
       if (!mbar_wait(mma_drain, 0)) atomicOr(p.status, kErrTimeout);
     }
+  } else if (warp >= 2 + kEpiGroups * kEpiWarps) {
+    // C mover of group g: a segment's C is loaded ahead of the epilogue, and
+    // stored and replaced by that of the buffer's next tile as soon as the
+    // epilogue is done with that segment, so that the round trip (store read,
+    // load) of one segment passes while the other is worked on.  With the group's
+    // leader moving whole tiles, the one buffer of a 256-row tile was the bound up
+    // to a depth of 512: C -= A B of order 16384, depth 256: 324 -> 228 us, depth
+    // 512: 316 -> 275 (what is left there is the operands' intake, 48 KB per 64
+    // of depth); order 28672, depth 512: 892 -> 880.
+    if (lane == 0 && p.has_c) {
+      const int g = warp - 2 - kEpiGroups * kEpiWarps;
+      const bool load_c = p.mode == kEpiSub;
+      int loading[kCBufs][kSegs];   // the phase of a load whose segment the epilogue has not finished, or -1
+      auto box = [&](int b, int h, int k) { return sC + b * kCTile + (g * kBoxes + h * kSegBoxes + k) * kCBox; };
+      auto row = [&](int h, int k) { return (TI / 2) * g + 64 * h + kBoxRows * k; };
+      auto arm = [&](const TileLoc& L, int b, int h, uint32_t phase) {
+        if (!load_c) {
+          mbar_arrive(c_full(b, g, h));
+          return;
+        }
+        loading[b][h] = (int)phase;
+        mbar_expect_tx(c_full(b, g, h), kSegBoxes * kCBox);
+#pragma unroll
+        for (int k = 0; k < kSegBoxes; ++k)
+          tma_load_2d(box(b, h, k), L.c, L.i0 + row(h, k), L.j0, c_full(b, g, h));
+      };
+      acquire_maps(2);
+#pragma unroll
+      for (int b = 0; b < kCBufs; ++b) {
+        const int t = (int)blockIdx.x + b * (int)gridDim.x;
+        TileLoc L{};
+        if (t < p.ntiles) L = locate(t);
+#pragma unroll
+        for (int h = 0; h < kSegs; ++h) {
+          loading[b][h] = -1;
+          if (t < p.ntiles) arm(L, b, h, 0);
+        }
+      }
+      bool ok = true;
+      int b = 0;
+      uint32_t phase = 0;
+      for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+        const TileLoc L = locate(t);
+#pragma unroll 1
+        for (int h = 0; h < kSegs; ++h) {
+          if (!mbar_wait(c_done(b, g, h), phase, p.wait_polls, p.wait_ns)) { ok = false; break; }
+          loading[b][h] = -1;
+#pragma unroll
+          for (int k = 0; k < kSegBoxes; ++k) tma_store_2d(L.c, L.i0 + row(h, k), L.j0, box(b, h, k));
+          bulk_commit();
+          if constexpr (kCBufs == 1) {
+            const int t2 = t + (int)gridDim.x;
+            if (t2 < p.ntiles) {
+              asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+              arm(locate(t2), b, h, phase ^ 1);
+            }
+          } else {   // the buffer before this one, whose store has been read by now
+            const int t2 = t + (kCBufs - 1) * (int)gridDim.x;
+            if (t != (int)blockIdx.x && t2 < p.ntiles) {
+              asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSegs) : "memory");
+              if (b > 0) arm(locate(t2), b - 1, h, phase ^ 1);
+              else arm(locate(t2), kCBufs - 1, h, phase);
+            }
+          }
+        }
+        if (++b == kCBufs) { b = 0; phase ^= 1; }
+      }
+      bulk_wait0();
+      if (!ok) {
+        atomicOr(p.status, kErrTimeout);
+        // C loads that the epilogue did not reach land before the CTA exits
+        for (int q = 0; q < kCBufs; ++q)
+          for (int h = 0; h < kSegs; ++h)
+            if (loading[q][h] >= 0) mbar_wait(c_full(q, g, h), (uint32_t)loading[q][h]);
+      }
+    }
   } else {
     // epilogue: group g = (warp - 2) / 4 owns rows i0 + (TI/2) g .. + TI/2 - 1 of the
-    // tile, as kBoxes C boxes of 64 rows; thread = output column j = j0 + jl,
+    // tile, as kSegs segments of 64 rows; thread = output column j = j0 + jl,
     // jl = 32 q + lane (its TMEM lane)
     const int q = warp & 3;
     const int g = (warp - 2) >> 2;
     const int jl = 32 * q + lane;
-    const bool leader = ((warp - 2) & 3) == 0 && lane == 0;
-    const bool load_c = p.has_c && p.mode == kEpiSub;
-    // C tile buffers rotate over local tiles: tile l uses buffer l % kCBufs.
-    // With three buffers the C of tile l + 2 is loaded into the buffer of tile
-    // l - 1 as soon as the store of tile l - 1 has been read, which is checked
-    // one tile later, when it is long done, so the epilogue never waits on its
-    // own store; with one buffer the C of tile l + 1 follows the store of l.
-    int issued_c[kCBufs];         // local tile whose C load is outstanding in each buffer
-    for (int b = 0; b < kCBufs; ++b) issued_c[b] = -1;
-    auto load_c_tile = [&](int tt, int b) {   // this group's boxes of tile tt's C into buffer b
-      const TileLoc Lc = locate(tt);
-      mbar_expect_tx(c_full(b, g), kBoxes * kCBox);
-#pragma unroll
-      for (int h = 0; h < kBoxes; ++h)
-        tma_load_2d(sC + b * kCTile + (g * kBoxes + h) * kCBox, Lc.c, Lc.i0 + (TI / 2) * g + kBoxRows * h, Lc.j0,
-                    c_full(b, g));
-    };
-    if (leader && p.has_c) acquire_maps(2);
-    if (leader && load_c) {       // prefetch the C of the first kAhead local tiles
-      int local = 0;
-      for (int t = blockIdx.x; t < p.ntiles && local < Cfg::kAhead; t += gridDim.x, ++local) {
-        load_c_tile(t, local % kCBufs);
-        issued_c[local % kCBufs] = local;
-      }
-    }
     bool ok = true;
     int local = 0;
-    for (int t = blockIdx.x; t < p.ntiles; t += gridDim.x, ++local) {
+    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++local) {
       const TileLoc L = locate(t);
       const int i0 = L.i0, j0 = L.j0;
       const int cb = local % kCBufs, ab = local % p.nbuf;
-      bool w = true;
-      if (load_c) w = mbar_wait(c_full(cb, g), (uint32_t)((local / kCBufs) & 1), p.wait_polls, p.wait_ns);
-      w = w && mbar_wait(acc_full(ab), (uint32_t)((local / p.nbuf) & 1), p.wait_polls, p.wait_ns);
-      // one decision for the whole group (warp-uniform for tcgen05.ld, and no
-      // warp of the group left behind at its named barrier)
-      w = epi_all(g, w);
-      if (!w) { ok = false; break; }
-      if (leader) issued_c[cb] = -1;
+      const uint32_t cphase = (uint32_t)((local / kCBufs) & 1);
+      // a decision per warp (uniform for tcgen05.ld); a warp that gives up leaves its
+      // segment undone, which the mover's and the other waits run out on
+      ok = !p.has_c || mbar_wait(c_full(cb, g, 0), cphase, p.wait_polls, p.wait_ns);
+      ok = ok && mbar_wait(acc_full(ab), (uint32_t)((local / p.nbuf) & 1), p.wait_polls, p.wait_ns);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
       tc_fence_after();
       const uint32_t lane_base = tmem + (uint32_t)ab * p.acc_cols + ((uint32_t)(32 * q) << 16) + (TI / 2) * g;
       float sc[4] = {1.0f, 1.0f, 1.0f, 1.0f};
@@ -386,11 +427,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int s2 = 0; s2 < p.nkb && s2 < 4; ++s2)
           sc[s2] = __fmul_rn(p.sA[(i0 / 128) * p.sa_ld + s2], p.sB[(j0 / 128) * p.sb_ld + s2]);
       const int64_t j = (int64_t)j0 + jl;
-      // one buffer, no C to load: the buffer's previous store was read (the
-      // leader waited for it before it reached this barrier)
-      if (kCBufs == 1 && p.has_c && !load_c) epi_barrier(g);
 #pragma unroll 1
       for (int h = 0; h < kSegs; ++h) {   // 64-row segments of the group's rows
+        if (h > 0 && p.has_c) {
+          ok = __all_sync(0xffffffffu, mbar_wait(c_full(cb, g, h), cphase, p.wait_polls, p.wait_ns));
+          if (!ok) break;
+        }
         const uint32_t lane_addr = lane_base + 64u * h;
         float acc[64];
         {
@@ -467,36 +509,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
         }
         }
-      }
-      if (p.has_c) {
-        fence_async_smem();
-        epi_barrier(g);
-        if (leader) {
-#pragma unroll
-          for (int h = 0; h < kBoxes; ++h)
-            tma_store_2d(L.c, i0 + (TI / 2) * g + kBoxRows * h, j0, sC + cb * kCTile + (g * kBoxes + h) * kCBox);
-          bulk_commit();
-          // the stores issued kCBufs - 1 tiles ago (one buffer: this tile's)
-          // have finished reading their buffer, which now receives the C of
-          // the tile kAhead ahead
-          asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(Cfg::kReadWait) : "memory");
-          const int t2 = t + Cfg::kAhead * (int)gridDim.x;
-          if (load_c && t2 < p.ntiles) {
-            const int b2 = (local + Cfg::kAhead) % kCBufs;
-            load_c_tile(t2, b2);
-            issued_c[b2] = local + Cfg::kAhead;
-          }
+        if (p.has_c) {
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(c_done(cb, g, h));
         }
       }
     }
     if (!ok && lane == 0) atomicOr(p.status, kErrTimeout);
-    if (leader) {
-      bulk_wait0();
-      // C loads issued for tiles this CTA did not reach (error path) land before exit
-      for (int b = 0; b < kCBufs; ++b)
-        if (issued_c[b] >= 0 && !mbar_wait(c_full(b, g), (uint32_t)((issued_c[b] / kCBufs) & 1)))
-          atomicOr(p.status, kErrTimeout);
-    }
   }
   tc_fence_before();
   __syncthreads();
