@@ -13,6 +13,12 @@
 // 128-byte-swizzled shared boxes of 64 rows and the epilogue touches them with
 // 16-byte, bank-conflict-free accesses.
 //
+// Large products of depth 512 run on pairs of CTAs (kPair): rank 0 issues the
+// MMAs of both, is told by rank 1's MMA warp when that CTA's operands are there
+// (arrivals without a cluster-scope acquire or release: only the tensor cores
+// read them, and those fences took 0.5 us a stage), and commits to both CTAs'
+// barriers; each CTA has its own producer, epilogue and C movers.
+//
 // Roles: warp 0 TMA producer of the operand ring; warp 1 TMEM owner and MMA
 // issuer; warps 2..9 epilogue in two groups of four (warp w reads TMEM lanes
 // 32*(w%4)..+31; group g takes rows TI/2 g .. of the tile); warps 10 and 11
@@ -53,10 +59,15 @@ constexpr int kThreads = 64 + kEpiGroups * (kEpiThreads + 32);   // and one warp
 // flops (the SM's operand intake is what bounds this kernel at K >= 256).
 // CB: bytes per C element, 2 (the 16-bit factor storage) or 4 (an fp32
 // trailing matrix: C = fl32(C - acc), 128-row tiles only).
-template <int TI, int CB = 2>
+// kPair: a cluster of two CTAs makes a tile of 256 rows and 256 columns, each
+// its own 128 columns of the accumulator; each stages 128 of the rows i, so that
+// an SM receives 32 instead of 48 KB per 64 of depth (942 -> 1157 TFLOP/s at
+// order 28672, depth 512; the n = 32768 factorization 36.7 -> 32.8 ms).
+template <int TI, int CB = 2, bool kPair = false>
 struct TileCfg {
-  static constexpr int kStages = TI == 128 ? 4 : 3;
-  static constexpr int kStageB = TI * kRowBytes;            // MMA B operand: rows i (16 or 32 KiB)
+  static constexpr int kStages = kPair ? 5 : TI == 128 ? 4 : 3;
+  static constexpr int kRowsB = kPair ? TI / 2 : TI;        // MMA B operand: rows i in this CTA
+  static constexpr int kStageB = kRowsB * kRowBytes;        // (16 or 32 KiB)
   static constexpr int kBoxRows = 128 / CB;                 // rows of one 128-byte C box: 64 or 32
   static constexpr int kBoxes = TI / 2 / kBoxRows;          // C boxes per epilogue group
   static constexpr int kCTile = kEpiGroups * kBoxes * kCBox;  // 32, 64 KiB (16-bit) or 64 KiB (fp32)
@@ -65,13 +76,13 @@ struct TileCfg {
   static constexpr int kSegs = TI / 128;                    // 64-row segments of an epilogue group's TI/2 rows
   static constexpr int kSegBoxes = kBoxes / kSegs;          // C boxes of a segment
   static constexpr int kCSlots = kCBufs * kEpiGroups * kSegs;
-  static constexpr int kBars = 2 * kStages + 5 + 2 * kCSlots;
+  static constexpr int kBars = 2 * kStages + 5 + 2 * kCSlots + (kPair ? kStages : 0);
   static constexpr size_t kSmem = 1024 + (size_t)kStages * (kStageA + kStageB) + (size_t)kCBufs * kCTile +
                                   8 * kBars + 16;
 };
 // 227 KB of dynamic shared memory per CTA; two TI-column fp32 accumulators in
 // the 512 TMEM columns; a TMA box is at most 256 rows
-static_assert(TileCfg<128>::kSmem <= 232448 && TileCfg<256>::kSmem <= 232448 && TileCfg<128, 4>::kSmem <= 232448,
+static_assert(TileCfg<128>::kSmem <= 232448 && TileCfg<256>::kSmem <= 232448 && TileCfg<256, 2, true>::kSmem <= 232448 && TileCfg<128, 4>::kSmem <= 232448,
               "shared memory per CTA");
 template <int TI>
 constexpr bool tile_fits() { return 2 * TI <= 512 && TI <= 256 && TI % 128 == 0; }
@@ -160,12 +171,12 @@ struct TileLoc {
   int64_t ldr;
 };
 
-template <int TI, int CB>
+template <int TI, int CB, bool kPair>
 __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, TcParams p, const GemmGroupItem* __restrict__ items,
                int nitems, const __grid_constant__ TcSecond second) {
-  using Cfg = TileCfg<TI, CB>;
+  using Cfg = TileCfg<TI, CB, kPair>;
   constexpr int kStages = Cfg::kStages, kStageB = Cfg::kStageB, kCTile = Cfg::kCTile, kCBufs = Cfg::kCBufs;
   constexpr int kBoxes = Cfg::kBoxes, kBoxRows = Cfg::kBoxRows, kSegs = Cfg::kSegs, kSegBoxes = Cfg::kSegBoxes;
   extern __shared__ uint8_t smem_raw[];
@@ -186,10 +197,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     return bar0 + 8u * (uint32_t)(2 * kStages + 4 + (b * kEpiGroups + g) * kSegs + h);
   };
   auto c_done = [&](int b, int g, int h) { return c_full(b, g, h) + 8u * (uint32_t)Cfg::kCSlots; };
-  const uint32_t mma_drain = bar0 + 8u * (uint32_t)(Cfg::kBars - 1);
+  const uint32_t mma_drain = bar0 + 8u * (uint32_t)(2 * kStages + 4 + 2 * Cfg::kCSlots);
+  // (pair, rank 0) the other CTA's operands of stage s are there
+  auto peer_full = [&](int s) { return mma_drain + 8u * (uint32_t)(1 + s); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + Cfg::kBars);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int rank = kPair ? (int)cluster_rank() : 0;
+  // tiles first(), first() + stride(), ...: read where used (as variables held from here on they
+  // cost the small products of the chain 2 us each)
+  auto first = [] { return kPair ? (int)blockIdx.x >> 1 : (int)blockIdx.x; };
+  auto stride = [] { return kPair ? (int)gridDim.x >> 1 : (int)gridDim.x; };
 
   // tile t -> its product (grouped launch: the last item starting at or before t)
   auto locate = [&](int t) {
@@ -201,7 +219,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       L.M = second.M; L.N = second.N; L.R = second.R; L.ldr = second.ldr;
     } else if (items == nullptr) {
       L.a = &tmA; L.b = &tmB; L.c = &tmC;
-      L.i0 = (t % p.tiles_i) * TI; L.j0 = (t / p.tiles_i) * kTJ;
+      L.i0 = (t % p.tiles_i) * TI; L.j0 = ((t / p.tiles_i) * (kPair ? 2 : 1) + rank) * kTJ;
       L.M = p.M; L.N = p.N; L.R = p.R; L.ldr = p.ldr;
     } else {
       int lo = 0, hi = nitems - 1;
@@ -231,7 +249,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int s = 0; s < kStages; ++s) { mbar_init(full(s), 1); mbar_init(empty(s), 1); }
     for (int b = 0; b < 2; ++b) {
       mbar_init(acc_full(b), 1);
-      mbar_init(acc_empty(b), kEpiGroups * kEpiWarps);
+      mbar_init(acc_empty(b), (kPair ? 2 : 1) * kEpiGroups * kEpiWarps);
     }
     for (int b = 0; b < kCBufs; ++b)
       for (int g = 0; g < kEpiGroups; ++g)
@@ -240,6 +258,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           mbar_init(c_done(b, g, h), kEpiWarps);
         }
     mbar_init(mma_drain, 1);
+    if (kPair)
+      for (int s = 0; s < kStages; ++s) mbar_init(peer_full(s), 1);
     fence_mbar_init();
     if (items == nullptr) {
       asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmA) : "memory");
@@ -248,11 +268,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     }
   }
   if (warp == 1) {
-    tmem_alloc(smem_u32(tmem_slot), p.ncols);
-    tmem_relinquish();
+    if constexpr (kPair) {
+      tmem_alloc_pair(smem_u32(tmem_slot), p.ncols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(smem_u32(tmem_slot), p.ncols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync();   // both CTAs' barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   // the setup above may run while the previous kernel of the stream finishes;
@@ -268,7 +294,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       bool ok = true;
       acquire_maps(0);
       acquire_maps(1);
-      for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+      for (int t = first(); t < p.ntiles && ok; t += stride()) {
         const TileLoc L = locate(t);
         const int i0 = L.i0, j0 = L.j0;
         for (int kb = 0; kb < p.nkb; ++kb, ++pos) {
@@ -280,7 +306,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           }
           mbar_expect_tx(full(s), kStageA + kStageB);
           tma_load_2d(sOpA + s * kStageA, L.b, kb * (kRowBytes / 2), j0, full(s));
-          tma_load_2d(sOpB + s * kStageB, L.a, kb * (kRowBytes / 2), i0, full(s));
+          tma_load_2d(sOpB + s * kStageB, L.a, kb * (kRowBytes / 2), i0 + rank * Cfg::kRowsB, full(s));
         }
       }
       if (!ok) atomicOr(p.status, kErrTimeout);
@@ -288,13 +314,32 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       for (long long q = (pos > kStages ? pos - kStages : 0); q < pos; ++q)
         if (!mbar_wait(full((int)(q % kStages)), (uint32_t)((q / kStages) & 1))) atomicOr(p.status, kErrTimeout);
     }
+  } else if (kPair && warp == 1 && rank == 1) {
+    // the MMAs are issued by rank 0, which is told when this CTA's operands are there
+    if (lane == 0) {
+      long long pos = 0;
+      bool ok = true;
+      for (int t = first(); t < p.ntiles && ok; t += stride())
+        for (int kb = 0; kb < p.nkb; ++kb, ++pos) {
+          const int s = (int)(pos % kStages);
+          if (!mbar_wait(full(s), (uint32_t)((pos / kStages) & 1), p.wait_polls, p.wait_ns)) { ok = false; break; }
+          mbar_arrive_at(peer_full(s), 0);
+        }
+      if (!ok) atomicOr(p.status, kErrTimeout);
+      // rank 0's MMAs, which read this CTA's shared memory and write its tensor memory, have completed
+      if (!mbar_wait(mma_drain, 0)) atomicOr(p.status, kErrTimeout);
+    }
   } else if (warp == 1) {
     if (lane == 0) {
-      const uint32_t idesc = p.fp8 ? make_idesc(0, TI) : make_idesc(p.fmt == kBF16 ? 1u : 0u, TI);
+      auto commit = [](uint32_t bar) {
+        if constexpr (kPair) tc_commit_pair(bar);
+        else tc_commit(bar);
+      };
+      const uint32_t idesc = p.fp8 ? make_idesc(0, TI) : make_idesc(p.fmt == kBF16 ? 1u : 0u, TI, kPair ? 256 : 128);
       long long pos = 0;
       bool ok = true;
       int local = 0;
-      for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++local) {
+      for (int t = first(); t < p.ntiles && ok; t += stride(), ++local) {
         const int ab = local % p.nbuf, ause = local / p.nbuf;
         if (ause > 0 && !mbar_wait(acc_empty(ab), (uint32_t)((ause - 1) & 1), p.wait_polls, p.wait_ns)) {
           ok = false;
@@ -304,24 +349,33 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         const uint32_t d0 = tmem + (uint32_t)ab * p.acc_cols;
         for (int kb = 0; kb < p.nkb; ++kb, ++pos) {
           const int s = (int)(pos % kStages);
-          if (!mbar_wait(full(s), (uint32_t)((pos / kStages) & 1), p.wait_polls, p.wait_ns)) { ok = false; break; }
+          const uint32_t ph = (uint32_t)((pos / kStages) & 1);
+          if (!mbar_wait(full(s), ph, p.wait_polls, p.wait_ns) ||
+              (kPair && !mbar_wait(peer_full(s), ph, p.wait_polls, p.wait_ns))) {
+            ok = false;
+            break;
+          }
           tc_fence_after();
           const uint32_t d = d0 + (p.fp8 ? (uint32_t)(kb * TI) : 0u);
           for (int kk = 0; kk < 4; ++kk) {   // 4 MMAs of 32 bytes of K each
             const uint64_t a = sdesc_sw128(sOpA + s * kStageA + kk * 32);
             const uint64_t b = sdesc_sw128(sOpB + s * kStageB + kk * 32);
             const uint32_t acc = p.fp8 ? (kk > 0) : (kb > 0 || kk > 0);
-            if (p.fp8) tc_mma_f8(d, a, b, idesc, acc);
-            else tc_mma_f16(d, a, b, idesc, acc);
+            if constexpr (kPair) {
+              tc_mma_f16_pair(d, a, b, idesc, acc);
+            } else {
+              if (p.fp8) tc_mma_f8(d, a, b, idesc, acc);
+              else tc_mma_f16(d, a, b, idesc, acc);
+            }
           }
-          tc_commit(empty(s));   // the stage is free once these MMAs have read it
+          commit(empty(s));   // the stage is free once these MMAs have read it
         }
-        tc_commit(acc_full(ab));
+        commit(acc_full(ab));
       }
       if (!ok) atomicOr(p.status, kErrTimeout);
       // every MMA issued has completed before TMEM is freed, also when an
       // epilogue group gave up before the last accumulator was written
-      tc_commit(mma_drain);
+      commit(mma_drain);
       if (!mbar_wait(mma_drain, 0)) atomicOr(p.status, kErrTimeout);
     }
   } else if (warp >= 2 + kEpiGroups * kEpiWarps) {
@@ -353,7 +407,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       acquire_maps(2);
 #pragma unroll
       for (int b = 0; b < kCBufs; ++b) {
-        const int t = (int)blockIdx.x + b * (int)gridDim.x;
+        const int t = first() + b * stride();
         TileLoc L{};
         if (t < p.ntiles) L = locate(t);
 #pragma unroll
@@ -365,24 +419,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       bool ok = true;
       int b = 0;
       uint32_t phase = 0;
-      for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x) {
+      for (int t = first(); t < p.ntiles && ok; t += stride()) {
         const TileLoc L = locate(t);
 #pragma unroll 1
         for (int h = 0; h < kSegs; ++h) {
           if (!mbar_wait(c_done(b, g, h), phase, p.wait_polls, p.wait_ns)) { ok = false; break; }
           loading[b][h] = -1;
 #pragma unroll
-          for (int k = 0; k < kSegBoxes; ++k) tma_store_2d(L.c, L.i0 + row(h, k), L.j0, box(b, h, k));
+          for (int k = 0; k < kSegBoxes && (!kPair || L.j0 < L.N); ++k) tma_store_2d(L.c, L.i0 + row(h, k), L.j0, box(b, h, k));
           bulk_commit();
           if constexpr (kCBufs == 1) {
-            const int t2 = t + (int)gridDim.x;
+            const int t2 = t + stride();
             if (t2 < p.ntiles) {
               asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
               arm(locate(t2), b, h, phase ^ 1);
             }
           } else {   // the buffer before this one, whose store has been read by now
-            const int t2 = t + (kCBufs - 1) * (int)gridDim.x;
-            if (t != (int)blockIdx.x && t2 < p.ntiles) {
+            const int t2 = t + (kCBufs - 1) * stride();
+            if (t != first() && t2 < p.ntiles) {
               asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSegs) : "memory");
               if (b > 0) arm(locate(t2), b - 1, h, phase ^ 1);
               else arm(locate(t2), kCBufs - 1, h, phase);
@@ -409,7 +463,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int jl = 32 * q + lane;
     bool ok = true;
     int local = 0;
-    for (int t = blockIdx.x; t < p.ntiles && ok; t += gridDim.x, ++local) {
+    for (int t = first(); t < p.ntiles && ok; t += stride(), ++local) {
       const TileLoc L = locate(t);
       const int i0 = L.i0, j0 = L.j0;
       const int cb = local % kCBufs, ab = local % p.nbuf;
@@ -455,7 +509,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           // accumulator buffer free for the MMA warp as soon as it is in registers
           tc_fence_before();
           __syncwarp();
-          if (lane == 0) mbar_arrive(acc_empty(ab));
+          if (lane == 0) {
+            if constexpr (kPair) mbar_arrive_at(acc_empty(ab), 0);
+            else mbar_arrive(acc_empty(ab));
+          }
         }
         if constexpr (CB == 4) {
           // fp32 C: two 32-row boxes; rows 32 q + 4 c8 .. +3 of column j in chunk c8 of box q
@@ -520,9 +577,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
   tc_fence_before();
   __syncthreads();
+  // neither CTA of a pair leaves while the other may still read its shared memory or arrive there
+  if constexpr (kPair) cluster_sync();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, p.ncols);
+    if constexpr (kPair) tmem_dealloc_pair(tmem, p.ncols);
+    else tmem_dealloc(tmem, p.ncols);
   }
   if (p.span && threadIdx.x == 0) atomicMin(p.span + 1, ~global_ns());
 }
@@ -581,16 +641,16 @@ int grid_cap() {
 
 namespace {
 
-template <int TI, int CB = 2>
+template <int TI, int CB = 2, bool kPair = false>
 cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st, const GemmArgs* also = nullptr) {
-  using Cfg = TileCfg<TI, CB>;
+  using Cfg = TileCfg<TI, CB, kPair>;
   static_assert(CB == 2 || TI == 128, "fp32 C on 128-row tiles only");
   if (CB == 4 && (g.mode != kEpiSub || g.R || !g.C)) return cudaErrorInvalidValue;
   const int esz = g.fp8 ? 1 : 2;
   const uint64_t kbytes = (uint64_t)g.K * esz;
   if (kbytes % kRowBytes) return cudaErrorInvalidValue;
   CUtensorMap ta, tb, tc;
-  if (!make_map(&ta, g.A, kbytes / 2, (uint64_t)g.M, (uint64_t)g.lda * esz, kRowBytes / 2, TI) ||
+  if (!make_map(&ta, g.A, kbytes / 2, (uint64_t)g.M, (uint64_t)g.lda * esz, kRowBytes / 2, Cfg::kRowsB) ||
       !make_map(&tb, g.B, kbytes / 2, (uint64_t)g.N, (uint64_t)g.ldb * esz, kRowBytes / 2, kTJ))
     return cudaErrorInvalidValue;
   TcParams p{};
@@ -604,7 +664,7 @@ cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st, const GemmArgs* al
   }
   p.M = g.M; p.N = g.N; p.nkb = (int)(kbytes / kRowBytes);
   p.tiles_i = cdiv(g.M, TI);
-  p.ntiles = p.tiles_i * cdiv(g.N, kTJ);
+  p.ntiles = p.tiles_i * cdiv(g.N, (kPair ? 2 : 1) * kTJ);
   p.split = p.ntiles;
   TcSecond second{};
   if (also) {
@@ -640,12 +700,13 @@ cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st, const GemmArgs* al
   int dev = 0;
   cudaGetDevice(&dev);
   if (configured_for.load() != dev) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<TI, CB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<TI, CB, kPair>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)Cfg::kSmem);
     if (e != cudaSuccess) return e;
     configured_for.store(dev);
   }
-  const int grid = std::min(p.ntiles, g.max_ctas > 0 ? std::min(g.max_ctas, grid_cap()) : grid_cap());
+  const int cap = g.max_ctas > 0 ? std::min(g.max_ctas, grid_cap()) : grid_cap();
+  const int grid = kPair ? 2 * std::min(p.ntiles, cap / 2) : std::min(p.ntiles, cap);
   // algorithmic DRAM bytes: both operands once, C read (subtract mode) and
   // written once, the optional row-major copy written once
   double flops = 0.0, bytes = 0.0;
@@ -659,7 +720,7 @@ cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st, const GemmArgs* al
   void* tok = prof_begin(st);
   p.span = prof_device_span(tok);
   const cudaError_t e =
-      launch_pdl(gemm_tc_kernel<TI, CB>, dim3(grid), dim3(kThreads), Cfg::kSmem, st, ta, tb, tc, p,
+      launch_pdl_cluster(gemm_tc_kernel<TI, CB, kPair>, kPair ? 2 : 1, dim3(grid), dim3(kThreads), Cfg::kSmem, st, ta, tb, tc, p,
                  (const GemmGroupItem*)nullptr, 0, second);
   prof_end(tok, g.mode == kEpiSub ? kProfGemm : kProfGemmStore, flops, st, bytes);
   count_launches(1);
@@ -730,7 +791,7 @@ cudaError_t gemm_tc_grouped(const GemmArgs& g, const GemmGroupItem* dev_items, i
   int dev = 0;
   cudaGetDevice(&dev);
   if (configured_for.load() != dev) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<128, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(gemm_tc_kernel<128, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)Cfg::kSmem);
     if (e != cudaSuccess) return e;
     configured_for.store(dev);
@@ -740,7 +801,7 @@ cudaError_t gemm_tc_grouped(const GemmArgs& g, const GemmGroupItem* dev_items, i
   memset(&none, 0, sizeof(none));   // the items' maps are used instead
   void* tok = prof_begin(st);
   p.span = prof_device_span(tok);
-  const cudaError_t e = launch_pdl(gemm_tc_kernel<128, 2>, dim3(grid), dim3(kThreads), Cfg::kSmem, st, none, none,
+  const cudaError_t e = launch_pdl(gemm_tc_kernel<128, 2, false>, dim3(grid), dim3(kThreads), Cfg::kSmem, st, none, none,
                                    none, p, dev_items, nitems, TcSecond{});
   prof_end(tok, g.mode == kEpiSub ? kProfGemm : kProfGemmStore, flops, st, bytes);
   count_launches(1);
@@ -760,7 +821,17 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   if (g.c32) return g.fp8 ? cudaErrorInvalidValue : gemm_tc_tiles<128, 4>(g, st);
   // 256-row tiles for the 16-bit products that fill them (M >= 256) and have
   // enough depth (K >= 256) for one C buffer to keep up
-  if (!g.fp8 && g.M >= 256 && g.K >= 256 && wide_tiles_enabled()) return gemm_tc_tiles<256>(g, st);
+  if (!g.fp8 && g.M >= 256 && g.K >= 256 && wide_tiles_enabled()) {
+    // Pairs of CTAs where the operands' intake is the bound: a depth of 512 and
+    // more tiles than SMs.  Pairs / single CTAs, C -= A B, us: order 28672, depth
+    // 512: 728 / 894; 16384: 257 / 284; 8192: 83 / 93; 3072: 29.5 / 30.3; 2048
+    // (fewer tiles than SMs): 25.7 / 25.1; depth 384 at 16384: 246 / 241; depth
+    // 256 at 28672: 699 / 687 (the C round trip bounds both).
+    const int cap = g.max_ctas > 0 ? std::min(g.max_ctas, grid_cap()) : grid_cap();
+    if (g.K >= 512 && cap >= 2 && 2LL * cdiv(g.M, 256) * cdiv(g.N, 2 * kTJ) > num_sms())
+      return gemm_tc_tiles<256, 2, true>(g, st);
+    return gemm_tc_tiles<256>(g, st);
+  }
   return gemm_tc_tiles<128>(g, st);
 }
 

@@ -294,20 +294,35 @@ struct SmBudgetScope {
   ~SmBudgetScope();
   int prev;
 };
+// `cluster` CTAs along x form a thread-block cluster (1: none).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                       Args&&... args) {
+cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), int cluster, dim3 grid, dim3 block, size_t smem,
+                               cudaStream_t st, Args&&... args) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  unsigned num = 0;
+  if (pdl_enabled()) {
+    attr[num].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[num++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[num].id = cudaLaunchAttributeClusterDimension;
+    attr[num].val.clusterDim.x = (unsigned)cluster;
+    attr[num].val.clusterDim.y = 1;
+    attr[num++].val.clusterDim.z = 1;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = pdl_enabled() ? 1 : 0;
+  cfg.numAttrs = num;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
+}
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       Args&&... args) {
+  return launch_pdl_cluster(kernel, 1, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
 
 void* prof_begin(cudaStream_t st);

@@ -91,6 +91,48 @@ __device__ inline void tc_mma_f8(uint32_t d, uint64_t a, uint64_t b, uint32_t id
 }
 
 
+// The same on a pair of CTAs (a cluster of two): one accumulator row block of
+// 128 lanes in each, A split by rows and B by columns between their shared
+// memories; issued by the CTA of rank 0, committed to the barriers at the same
+// offset in both.
+__device__ inline void tmem_alloc_pair(uint32_t slot, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(ncols)
+               : "memory");
+}
+__device__ inline void tmem_relinquish_pair() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ inline void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+}
+__device__ inline void tc_commit_pair(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ inline void tc_mma_f16_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n"
+      ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      : "memory");
+}
+__device__ inline uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ inline void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Arrive on the barrier at `bar`'s offset in CTA `rank` of the cluster.
+__device__ inline void mbar_arrive_at(uint32_t bar, uint32_t rank) {
+  asm volatile(
+      "{\n .reg .b32 a;\n mapa.shared::cluster.u32 a, %0, %1;\n"
+      " mbarrier.arrive.shared::cluster.b64 _, [a];\n}\n" ::"r"(bar), "r"(rank)
+      : "memory");
+}
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
 // 128 bytes, 8-row groups 1024 bytes apart (stride byte offset), leading byte
 // offset unused for this layout (set to 16 bytes), descriptor version 1.
@@ -99,11 +141,11 @@ __device__ inline uint64_t sdesc_sw128(uint32_t saddr) {
          ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
 }
 
-// Instruction descriptor: fp32 accumulator, K-major A and B, M = 128, N = n.
+// Instruction descriptor: fp32 accumulator, K-major A and B, M = m, N = n.
 // Operand format code: kind::f16 -> 0 F16, 1 BF16; kind::f8f6f4 -> 0 E4M3.
-__host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt_code, int n) {
+__host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt_code, int n, int m = 128) {
   return (1u << 4) | (fmt_code << 7) | (fmt_code << 10) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(128 >> 4) << 24);
+         ((uint32_t)(m >> 4) << 24);
 }
 
 }  // namespace
