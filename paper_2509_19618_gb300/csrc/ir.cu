@@ -104,6 +104,8 @@ __global__ void __launch_bounds__(kGemvThreads) gemv_partial_kernel(int64_t n, c
                                                                     float* __restrict__ A32, int64_t ld32,
                                                                     double* __restrict__ P, void* __restrict__ RS,
                                                                     Gate gate) {
+  pdl_wait();
+  pdl_trigger();
   if (gate.closed()) return;
   __shared__ double xs[kGemvChunkElems];   // xs[r * chunk + jj]
   const int64_t i = (int64_t)blockIdx.x * kGemvRows + 2 * threadIdx.x;
@@ -200,6 +202,8 @@ __global__ void __launch_bounds__(kGemvThreads) gemv32_partial_kernel(int64_t n,
                                                                       int64_t ld32, const double* __restrict__ X,
                                                                       int64_t ldx, int64_t chunk,
                                                                       double* __restrict__ P, Gate gate) {
+  pdl_wait();
+  pdl_trigger();
   if (gate.closed()) return;
   __shared__ double xs[kGemvChunkElems];
   const int64_t i = (int64_t)blockIdx.x * kGemv32Rows + 4 * threadIdx.x;
@@ -272,6 +276,8 @@ __global__ void __launch_bounds__(kFinRows * kFinGroups)
 gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P, const double* __restrict__ B,
                    int64_t ldb, double* __restrict__ out, int64_t ldo, const double* __restrict__ X, int64_t ldx,
                    int abs_mode, const void* __restrict__ RS, RhsState* st, int track_norms, GemvSplit split, Gate gate) {
+  pdl_wait();
+  pdl_trigger();
   if (gate.closed()) return;
   __shared__ double sh[2][kFinGroups][kFinRows];
   const int tx = threadIdx.x % kFinRows, ty = threadIdx.x / kFinRows;
@@ -338,6 +344,8 @@ __device__ inline double block_sum(double v, double* sh) {
 __global__ void __launch_bounds__(256) mgs_kernel(int64_t n, int K, int m, int j, int i, double* W, int64_t ldw,
                                                   const double* V, int64_t ldv_col, int64_t ldv_rhs,
                                                   RhsState* st, double* partials, unsigned int* counter, Gate gate) {
+  pdl_wait();
+  pdl_trigger();
   if (gate.closed()) return;
   __shared__ double sh[32];
   __shared__ bool last;
@@ -390,6 +398,8 @@ __global__ void __launch_bounds__(kFusedMgsThreads) arnoldi_tail_kernel(SolvePar
                                                                         double* W, int64_t ldw, double* V,
                                                                         int64_t ldv_col, int64_t ldv_rhs,
                                                                         RhsState* st, Brief* brief) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double sh[32];
   const int r = blockIdx.x;
   if (st[r].cycle_active) {   // the same value for every thread
@@ -425,6 +435,8 @@ __global__ void __launch_bounds__(kFusedMgsThreads) arnoldi_tail_kernel(SolvePar
 // ||z||_2 for cycle start (beta), into st[r].beta, for rhs with outer_active.
 __global__ void __launch_bounds__(256) norm2_kernel(int64_t n, int K, const double* Z, int64_t ldz, RhsState* st,
                                                     double* partials, unsigned int* counter) {
+  pdl_wait();
+  pdl_trigger();
   __shared__ double sh[32];
   __shared__ bool last;
   for (int r = 0; r < K; ++r) {
@@ -456,6 +468,8 @@ __global__ void __launch_bounds__(256) norm2_kernel(int64_t n, int K, const doub
 // for rhs whose flag (cycle_active or outer_active) is set.
 __global__ void scale_kernel(int64_t n, int K, const double* src, int64_t lds, double* dst, int64_t ldd,
                              const RhsState* st, int which) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   for (int r = 0; r < K; ++r) {
@@ -472,6 +486,8 @@ __global__ void init_kernel(int K, RhsState* st) {
 
 // Outer check: scaled residual from the max-reductions; decide per rhs.
 __global__ void check_kernel(SolveParams sp, RhsState* st, Brief* brief, int first) {
+  pdl_wait();
+  pdl_trigger();
   const int r = threadIdx.x;
   if (r >= sp.n_rhs) return;
   RhsState& s = st[r];
@@ -495,6 +511,8 @@ __global__ void check_kernel(SolveParams sp, RhsState* st, Brief* brief, int fir
 
 // Cycle start (after beta = ||M^{-1} r||): g = beta e1, tolerance.
 __global__ void cycle_start_kernel(SolveParams sp, RhsState* st, Brief* brief) {
+  pdl_wait();
+  pdl_trigger();
   const int r = threadIdx.x;
   if (r >= sp.n_rhs) return;
   RhsState& s = st[r];
@@ -551,11 +569,15 @@ __device__ void givens_rhs(const SolveParams& sp, int j, RhsState* st, Brief* br
   brief[r].iters = s.iters; brief[r].status = s.status;
 }
 __global__ void givens_kernel(SolveParams sp, int j, RhsState* st, Brief* brief) {
+  pdl_wait();
+  pdl_trigger();
   if ((int)threadIdx.x < sp.n_rhs) givens_rhs(sp, j, st, brief, threadIdx.x);
 }
 
 // y = H(0:k, 0:k)^{-1} g(0:k) by back substitution.
 __global__ void cycle_finish_kernel(SolveParams sp, RhsState* st) {
+  pdl_wait();
+  pdl_trigger();
   const int r = threadIdx.x;
   if (r >= sp.n_rhs) return;
   RhsState& s = st[r];
@@ -571,6 +593,8 @@ __global__ void cycle_finish_kernel(SolveParams sp, RhsState* st) {
 // x(:, r) += V_r(:, 0:k) y_r
 __global__ void update_kernel(int64_t n, int K, double* X, int64_t ldx, const double* V, int64_t ldv_col,
                               int64_t ldv_rhs, const RhsState* st) {
+  pdl_wait();
+  pdl_trigger();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= n) return;
   for (int r = 0; r < K; ++r) {
@@ -591,6 +615,7 @@ struct SolveWs {
   Brief* brief;
   unsigned int* counter;
   size_t control_bytes;   // report .. counter, zeroed at the start of a solve
+  bool pdl = true;        // programmatic launches (launch_vec)
   double* partials;  // kMaxK * kRedBlocks
   double* r;         // n x K
   double* w;         // n x K
@@ -647,6 +672,17 @@ SolveWs carve_solve(void* base, int64_t n, int64_t K, int m) {
   return w;
 }
 
+// The refinement's kernels: as programmatic dependents of one another for one
+// system, whose kernels of a few microseconds otherwise start 2 to 3 us apart (n =
+// 1024: 575 -> 500 us, 8192 with eight right-hand sides 5.40 -> 5.31 ms); as plain
+// launches for the systems of a batch, where the CTAs that wait take room from
+// other streams' kernels (24 mixed systems 8.55 ms, 8.80 as dependents).
+template <typename... KArgs, typename... Args>
+void launch_vec(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
+  if (pdl) launch_pdl(kernel, grid, block, 0, st, static_cast<Args&&>(args)...);
+  else kernel<<<grid, block, 0, st>>>(static_cast<Args&&>(args)...);
+}
+
 // abs_mode: 0 plain, 1 with the fp32 |A| estimate (the first residual; also
 // fills w.a32 when there is one), 2 exact |A| row sums, 3 the fp32 operator's
 // product (from w.a32 when there is one)
@@ -661,15 +697,16 @@ cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int
   void* RS = w.RS;
   if (abs_mode == 3 && w.a32) {
     dim3 g32((unsigned)cdiv<int64_t>(n, kGemv32Rows), (unsigned)nchunk);
-    gemv32_partial_kernel<K><<<g32, T, 0, st>>>(n, w.a32, w.ld32, X, ldx, chunk, P, gate);
+    launch_vec(w.pdl, gemv32_partial_kernel<K>, g32, dim3(T), st, n, w.a32, w.ld32, X, ldx, chunk, P, gate);
   } else if (abs_mode == 3) {
-    gemv_partial_kernel<K, 0, true><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
+    launch_vec(w.pdl, gemv_partial_kernel<K, 0, true>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS,
+               gate);
   } else if (abs_mode == 0) {
-    gemv_partial_kernel<K, 0><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
+    launch_vec(w.pdl, gemv_partial_kernel<K, 0>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
   } else if (abs_mode == 1) {
-    gemv_partial_kernel<K, 1><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, w.a32, w.ld32, P, RS, gate);
+    launch_vec(w.pdl, gemv_partial_kernel<K, 1>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, w.a32, w.ld32, P, RS, gate);
   } else {
-    gemv_partial_kernel<K, 2><<<grid, T, 0, st>>>(n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
+    launch_vec(w.pdl, gemv_partial_kernel<K, 2>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
   }
   return cudaGetLastError();
 }
@@ -717,8 +754,8 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
     }
   }
   if (e != cudaSuccess) return e;
-  gemv_finish_kernel<<<dim3((unsigned)cdiv<int64_t>(n, kFinRows), K), kFinRows * kFinGroups, 0, st>>>(
-      n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split, gate);
+  launch_vec(w.pdl, gemv_finish_kernel, dim3((unsigned)cdiv<int64_t>(n, kFinRows), K), dim3(kFinRows * kFinGroups), st,
+             n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split, gate);
   prof_end(tok, abs_mode == 3 ? kProfGemv32 : kProfGemv, 8.0 * (double)n * (double)n, st);
   count_launches(2);
   return cudaGetLastError();
@@ -766,16 +803,17 @@ struct Solver {
   void arnoldi_tail(int j, Gate gate) {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     if (n * K <= kFusedMgsMaxElems) {
-      arnoldi_tail_kernel<<<K, kFusedMgsThreads, 0, st>>>(sp, n, m, j, w.w, n, w.V, n, ldv_rhs(), w.st, w.brief);
+      launch_vec(w.pdl, arnoldi_tail_kernel, dim3(K), dim3(kFusedMgsThreads), st, sp, n, m, j, w.w, n, w.V, n,
+                 ldv_rhs(), w.st, w.brief);
       count_launches(1);
       return;
     }
     for (int i = 0; i <= j + 1; ++i)
-      mgs_kernel<<<red_blocks(), 256, 0, st>>>(n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st, w.partials, w.counter,
-                                               gate);
-    givens_kernel<<<1, 32, 0, st>>>(sp, j, w.st, w.brief);
-    scale_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, w.w, n, w.V + (int64_t)(j + 1) * n, ldv_rhs(),
-                                                                   w.st, 1);
+      launch_vec(w.pdl, mgs_kernel, dim3(red_blocks()), dim3(256), st, n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st,
+                 w.partials, w.counter, gate);
+    launch_vec(w.pdl, givens_kernel, dim3(1), dim3(32), st, sp, j, w.st, w.brief);
+    launch_vec(w.pdl, scale_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), st, n, K, w.w, n,
+               w.V + (int64_t)(j + 1) * n, ldv_rhs(), w.st, 1);
     count_launches(j + 4);
   }
   bool any(int Brief::*f) const {
@@ -805,9 +843,10 @@ struct Solver {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     const cudaError_t e = precond(w.r, n, w.tmp, n, ahead ? outer_gate() : Gate{});
     if (e != cudaSuccess) return e;
-    norm2_kernel<<<red_blocks(), 256, 0, st>>>(n, K, w.tmp, n, w.st, w.partials, w.counter);
-    cycle_start_kernel<<<1, 32, 0, st>>>(sp, w.st, w.brief);
-    scale_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, w.tmp, n, w.V, ldv_rhs(), w.st, 0);
+    launch_vec(w.pdl, norm2_kernel, dim3(red_blocks()), dim3(256), st, n, K, w.tmp, n, w.st, w.partials, w.counter);
+    launch_vec(w.pdl, cycle_start_kernel, dim3(1), dim3(32), st, sp, w.st, w.brief);
+    launch_vec(w.pdl, scale_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), st, n, K, w.tmp, n, w.V,
+               ldv_rhs(), w.st, 0);
     count_launches(3);
     return cudaGetLastError();
   }
@@ -824,8 +863,9 @@ struct Solver {
   // x += V y
   cudaError_t cycle_finish() {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
-    cycle_finish_kernel<<<1, 32, 0, st>>>(sp, w.st);
-    update_kernel<<<(unsigned)cdiv<int64_t>(n, 256), 256, 0, st>>>(n, K, X, ldx, w.V, n, ldv_rhs(), w.st);
+    launch_vec(w.pdl, cycle_finish_kernel, dim3(1), dim3(32), st, sp, w.st);
+    launch_vec(w.pdl, update_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), st, n, K, X, ldx, w.V, n,
+               ldv_rhs(), w.st);
     count_launches(2);
     return cudaGetLastError();
   }
@@ -834,7 +874,7 @@ struct Solver {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     const cudaError_t e = residual(n, K, A, lda, X, ldx, B, ldb, w.r, n, first ? 1 : 0, 1, w, st);
     if (e != cudaSuccess) return e;
-    check_kernel<<<1, 32, 0, st>>>(sp, w.st, w.brief, first ? 1 : 0);
+    launch_vec(w.pdl, check_kernel, dim3(1), dim3(32), st, sp, w.st, w.brief, first ? 1 : 0);
     count_launches(1);
     return cudaGetLastError();
   }
@@ -930,6 +970,7 @@ hpmxp_status solve_ir(int64_t n, const double* A, int64_t lda, const void* LU, i
   s.B = b; s.ldb = ldb; s.X = x; s.ldx = ldx;
   s.prm = prm;
   s.w = carve_solve(ws, n, nrhs, prm.restart);
+  s.w.pdl = sm_budget() <= 0;   // under a budget the call shares the chip, as a batch's systems do
   // room for the fp32 copy of A after the workspace proper: the fp32 Arnoldi
   // products then read 4 instead of 8 bytes per entry
   if (prm.matvec_fp32 && ws_bytes >= s.w.bytes + solve_a32_bytes(n)) {
@@ -1052,6 +1093,7 @@ hpmxp_status solve_ir_batched(const hpmxp_problem* probs, int count, int prec, c
     s.B = probs[q].b; s.ldb = probs[q].ldb; s.X = probs[q].x; s.ldx = probs[q].ldx;
     s.prm = prm;
     s.w = carve_solve(base, s.n, s.K, prm.restart);
+    s.w.pdl = false;
     base += round_up<size_t>(s.w.bytes, 256);
     s.st = pool.st[q % kPoolStreams];
     it[q].ev = hs.ev[q];

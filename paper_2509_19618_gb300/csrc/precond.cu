@@ -304,6 +304,7 @@ __global__ void __launch_bounds__(2 * kGrp) precond_kernel(PrecondArgs p) {
   constexpr int kR = sizeof(T) == 8 ? 1 : K <= 3 ? 4 : 2, kRB = sizeof(T) == 8 ? 2 : kR;
   constexpr int kQ = K * sizeof(T) <= 16 || (sizeof(T) == 8 && K <= 4) ? 4 : K % 2 == 0 || sizeof(T) == 8 ? 2 : 1;   // columns of a run
   constexpr int kUnroll = K * sizeof(T) <= 8 ? 4 : sizeof(T) == 4 || K == 2 ? 2 : 1;   // runs read ahead, against registers
+  pdl_trigger();   // every CTA is resident: the next kernel's may wait beside them
   if (p.gate.closed()) return;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ volatile int ready;   // owned blocks of the sweep whose updates are complete
