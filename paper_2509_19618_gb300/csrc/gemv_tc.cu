@@ -75,7 +75,7 @@ constexpr int kNoExp = -400;                 // exponent of a column whose x is 
 // non-finite entry (exponent 2047) in a column of exponent kNoExp would not exceed it
 constexpr int kMinE = 64, kMaxE = 2047 + kNoExp - 1;
 static_assert(7ll * kBlk * 255 * 128 < (1 << 24), "exact fp32 sums");
-constexpr int kBars = 2 * kBBufs + kGroups * kStages + kGroups;
+constexpr int kBars = 2 * kBBufs + kGroups * kStages + 2 * kGroups;
 
 template <int K>
 constexpr size_t gemv_smem() {
@@ -248,6 +248,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
   auto b_empty = [&](int b) { return bar0 + 8u * (uint32_t)(kBBufs + b); };
   auto a_full = [&](int gg, int s) { return bar0 + 8u * (uint32_t)(2 * kBBufs + gg * kStages + s); };
   const uint32_t bar_mma = bar0 + 8u * (uint32_t)(2 * kBBufs + kGroups * kStages + g);
+  const uint32_t bar_drain = bar_mma + 8u * (uint32_t)kGroups;
   auto digits_at = [&](int b) { return smem_u32(smem) + (uint32_t)(1 + b * (kSlices + 1)) * 1024; };
 
   for (int i = tid * 16; i < kBArea; i += kThr * 16) *reinterpret_cast<uint4*>(smem + i) = make_uint4(0, 0, 0, 0);
@@ -257,6 +258,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
     for (int k = 0; k < kGroups; ++k) {
       for (int s = 0; s < kStages; ++s) mbar_init(a_full(k, s), 1);
       mbar_init(bar0 + 8u * (uint32_t)(2 * kBBufs + kGroups * kStages + k), 1);
+      mbar_init(bar0 + 8u * (uint32_t)(2 * kBBufs + kGroups * kStages + kGroups + k), 1);
     }
     fence_mbar_init();
   }
@@ -507,6 +509,10 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
                   above |= (uint32_t)((__double2hiint(col[c * kRowsT]) & 0x7fffffff) + ej[c] > etop) << c;
+                // columns past the last one are zeros, but after a wait that ran out the stage and the
+                // exponents hold anything: x has n entries
+                const int64_t left = p.n - ((int64_t)kb * kBlk + 16 * sub + 8 * half);
+                if (left < 8) above &= left > 0 ? (1u << left) - 1u : 0u;
                 while (above) {
                   const int c = __ffs((int)above) - 1;
                   above &= above - 1;
@@ -539,8 +545,8 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
                 // that the column counts are multiples of 16)
                 tc_mma_ts(td + 16 * (s / 2), ta + 8 * s, sdesc_sw128(bd - (s & 1) * 1024),
                           make_idesc(0, 64 - 16 * (s / 2)), sub > 0 || s > 0);
-              tc_commit(bar_mma);
               if (sub == 3) tc_commit(b_empty(bb));
+              tc_commit(bar_mma);   // the last one, which the drain below waits for
             } else if (tg == 32) {   // every thread of the group has read this stage
               load_a(a_loads++);
               if (g == 0 && sub == 2) load_b(b_loads++);
@@ -573,6 +579,13 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
     // every MMA issued has completed before tensor memory is freed, and every copy has
     // landed before the CTA exits (default bound)
     if (issued && !mbar_wait(bar_mma, (issued - 1) & 1)) atomicOr(p.status, kErrTimeout);
+    // Where a wait ran out, several commits can be open, and bar_mma's parity is that of the one before
+    // the last as well: the issuing thread commits once more, to a barrier used for nothing else.  (If it
+    // does not see the flag, each of its own waits ended before its next MMAs, and one commit at most was open.)
+    if (tg == 0 && issued && *dead) {
+      tc_commit(bar_drain);
+      if (!mbar_wait(bar_drain, 0)) atomicOr(p.status, kErrTimeout);
+    }
     if (tg == 32 && *dead) {
       for (int s = 0; s < kStages; ++s)
         if (fills_a[s] && !mbar_wait(a_full(g, s), (fills_a[s] - 1) & 1)) atomicOr(p.status, kErrTimeout);
