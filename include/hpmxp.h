@@ -318,7 +318,10 @@ hpmxp_status hpmxp_residual(int64_t n, const double* A, int64_t lda, const doubl
                             void* ws, size_t ws_bytes, void* stream);
 
 /* r = b - A x for every column, fp64 (the refinement's residual kernels):
- *   r   out, n x nrhs fp64 (ldr >= n); the other arguments as hpmxp_residual. */
+ *   r   out, n x nrhs fp64 (ldr >= n); the other arguments as hpmxp_residual.
+ * Does not synchronize `stream`, so it never returns HPMXP_ETIMEOUT: should a
+ * device wait of its product run out, the call computes r again without waits
+ * (later on the stream, correct, and slower). */
 hpmxp_status hpmxp_residual_vector(int64_t n, const double* A, int64_t lda, const double* x, int64_t ldx,
                                    const double* b, int64_t ldb, int64_t nrhs, double* r, int64_t ldr, void* ws,
                                    size_t ws_bytes, void* stream);

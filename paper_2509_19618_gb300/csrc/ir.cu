@@ -266,6 +266,9 @@ __global__ void __launch_bounds__(kGemvThreads) gemv32_partial_kernel(int64_t n,
 // system's few rows would otherwise wait for each load in turn: 6.0 us at n =
 // 1024, 67 us at 8192 with eight right-hand sides) and are summed in order; the
 // rows' maxima by shuffles, one atomic per CTA and maximum.
+// With `redo`, the status word of a call that cannot report it: a set timeout bit
+// says that the partial sums are void, and the rows are summed here from A and X
+// by fp64 FMAs instead (the same eight threads, every eighth column each).
 __device__ inline unsigned long long warp_max(unsigned long long v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
@@ -275,7 +278,8 @@ constexpr int kFinRows = 32, kFinGroups = 8;   // rows of a CTA, threads that sh
 __global__ void __launch_bounds__(kFinRows * kFinGroups)
 gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P, const double* __restrict__ B,
                    int64_t ldb, double* __restrict__ out, int64_t ldo, const double* __restrict__ X, int64_t ldx,
-                   int abs_mode, const void* __restrict__ RS, RhsState* st, int track_norms, GemvSplit split, Gate gate) {
+                   int abs_mode, const void* __restrict__ RS, RhsState* st, int track_norms, GemvSplit split, Gate gate,
+                   const uint32_t* redo, const double* __restrict__ A, int64_t lda) {
   pdl_wait();
   pdl_trigger();
   if (gate.closed()) return;
@@ -286,7 +290,9 @@ gemv_finish_kernel(int64_t n, int K, int nchunk, const double* __restrict__ P, c
   const bool in = i < n, rows_too = track_norms && abs_mode && r == 0;
   if (split.ctas) nchunk = split.pieces((int)(min(i, n - 1) / kGemvTileRows));   // the tile's own count
   double s = 0.0, a = 0.0;
-  if (in) {
+  if (in && redo && (*redo & kErrTimeout)) {
+    for (int64_t j = ty; j < n; j += kFinGroups) s = __fma_rn(A[i + j * lda], X[j + r * ldx], s);
+  } else if (in) {
     for (int c = ty; c < nchunk; c += kFinGroups) s += P[((int64_t)c * K + r) * n + i];
     if (rows_too)
       for (int c = ty; c < nchunk; c += kFinGroups)
@@ -729,10 +735,11 @@ bool gemv_on_tensor_cores(int64_t n, int K, const double* A, int64_t lda, int ab
   return true;
 }
 
-// out = b - A X (b may be NULL: out = -A X), with optional norm tracking.
+// out = b - A X (b may be NULL: out = A X), with optional norm tracking.  redo:
+// for a caller that does not read w.status, make a void product good (without norms).
 cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx,
                      const double* B, int64_t ldb, double* out, int64_t ldo, int abs_mode, int track,
-                     const SolveWs& w, cudaStream_t st, Gate gate = {}) {
+                     const SolveWs& w, cudaStream_t st, Gate gate = {}, bool redo = false) {
   int nchunk = gemv_chunks(n, K);
   cudaError_t e;
   void* tok = prof_begin(st);
@@ -755,7 +762,8 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
   }
   if (e != cudaSuccess) return e;
   launch_vec(w.pdl, gemv_finish_kernel, dim3((unsigned)cdiv<int64_t>(n, kFinRows), K), dim3(kFinRows * kFinGroups), st,
-             n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split, gate);
+             n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split, gate,
+             redo ? (const uint32_t*)w.status : nullptr, A, lda);
   prof_end(tok, abs_mode == 3 ? kProfGemv32 : kProfGemv, 8.0 * (double)n * (double)n, st);
   count_launches(2);
   return cudaGetLastError();
@@ -1216,13 +1224,15 @@ hpmxp_status precond_apply(int64_t n, const void* LU, int64_t ldlu, int fmt, con
   return status_from_word(word);
 }
 
-// r = b - A x (fp64, the refinement's residual kernels), every column.
+// r = b - A x (fp64, the refinement's residual kernels), every column.  Ordered
+// on the stream like the work it launches, not waited for, so a wait that runs out
+// in the tensor-core product cannot be reported: the last pass makes it good.
 hpmxp_status residual_vector(int64_t n, const double* A, int64_t lda, const double* x, int64_t ldx,
                              const double* b, int64_t ldb, int64_t nrhs, double* r, int64_t ldr, void* ws,
                              cudaStream_t st) {
   SolveWs w = carve_solve(ws, n, nrhs, 1);
   cudaError_t e = cudaMemsetAsync(w.status, 0, 4, st);
-  if (e == cudaSuccess) e = residual(n, (int)nrhs, A, lda, x, ldx, b, ldb, r, ldr, 0, 0, w, st);
+  if (e == cudaSuccess) e = residual(n, (int)nrhs, A, lda, x, ldx, b, ldb, r, ldr, 0, 0, w, st, {}, true);
   return status_from_cuda(e);
 }
 
