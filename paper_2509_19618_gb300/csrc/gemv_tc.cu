@@ -85,23 +85,32 @@ static_assert(gemv_smem<8>() <= 232448, "shared memory per CTA");
 
 // --- X's digits ------------------------------------------------------------
 
-// f_r: 2^f_r > max_j |x_jr| (one CTA per right-hand side)
+// f_r: 2^f_r > max_j |x_jr| (one CTA per right-hand side), or kOut where r is
+// zero or not live: such a column takes no part in the column exponents, or it
+// would decide how the others' products are formed (a zero one would send them
+// all to fp64 FMAs, 8192 x 8: 1078 us instead of 157; one whose cycle has ended
+// is unwritten workspace).
+constexpr int kOut = 4096;
 __global__ void __launch_bounds__(1024) xscale_kernel(int64_t n, const double* __restrict__ X, int64_t ldx,
-                                                      int* __restrict__ fr, Gate gate) {
+                                                      int* __restrict__ fr, Gate gate, Gate live) {
   __shared__ int sh[32];
   pdl_wait();
   if (gate.closed()) return;
   pdl_trigger();
   const double* x = X + blockIdx.x * ldx;
   int m = 0;
-  for (int64_t j = threadIdx.x; j < n; j += 1024) m = max(m, __double2hiint(x[j]) & 0x7fffffff);
+  if (!live.flag || live.flag[(size_t)blockIdx.x * live.stride])
+    for (int64_t j = threadIdx.x; j < n; j += 1024) {
+      const double v = x[j];
+      m = max(m, (__double2hiint(v) & 0x7fffffff) | (__double2loint(v) != 0));
+    }
   m = __reduce_max_sync(0xffffffffu, m);
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x < 32) {
     m = __reduce_max_sync(0xffffffffu, sh[threadIdx.x]);
     if (threadIdx.x == 0) {
-      fr[blockIdx.x] = (m >> 20) - 1022;
+      fr[blockIdx.x] = m ? (m >> 20) - 1022 : kOut;
       if (blockIdx.x == 0) fr[8] = 0;   // digit_kernel counts the columns that are not robust
     }
   }
@@ -122,19 +131,20 @@ __global__ void __launch_bounds__(512) digit_kernel(int64_t n, int K, const doub
   if (gate.closed()) return;
   pdl_trigger();
   double v = 0.0;
-  int f = 0;
-  if (r < K && j < n) { v = X[j + r * ldx]; f = fr[r]; }
+  const int f = r < K ? fr[r] : kOut;
+  const bool skip = f == kOut;
+  if (!skip && j < n) v = X[j + r * ldx];
   const bool fin = isfinite(v);
   if (!fin) v = 0.0;
   const int ev = v == 0.0 ? kNoExp : ilogb(v) + 1 - f;   // |v| 2^-f < 2^ev
   const int e = max(ev, kNoExp);
-  es[r][jl] = e;
+  es[r][jl] = skip ? INT_MIN : e;
   __syncthreads();
   if (!fin || ev < kNoExp) bad = 1;
   int em = kNoExp;
   for (int k = 0; k < K; ++k) em = max(em, es[k][jl]);
   bool robust = true;   // every right-hand side has a sizeable x in this column (or none has any)
-  for (int k = 0; k < K; ++k) robust = robust && es[k][jl] >= em - 6;
+  for (int k = 0; k < K; ++k) robust = robust && (es[k][jl] == INT_MIN || es[k][jl] >= em - 6);
   long long q = em == kNoExp ? 0 : llrint(scalbn(v, 55 - f - em));
   uint8_t* out = dig + (size_t)blockIdx.x * kDig + r * 128 + (((jl >> 3) ^ r) << 4) + (jl & 7) * 2;
 #pragma unroll
@@ -639,7 +649,8 @@ bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, Gemv
 }
 
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
-                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate) {
+                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate,
+                    Gate live) {
   const int nkb = (int)cdiv<int64_t>(n, kBlk);
   GemvTc p{};
   p.n = n; p.A = A; p.lda = lda; p.X = X; p.ldx = ldx;
@@ -658,7 +669,7 @@ cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double
   CUtensorMap tm;
   if (!encode_f64_map(&tm, A, n, n, lda, kRowsT, kCols)) return cudaErrorInvalidValue;
   count_launches(3);
-  cudaError_t e = launch_pdl(xscale_kernel, dim3(K), dim3(1024), 0, st, n, X, ldx, fr, gate);
+  cudaError_t e = launch_pdl(xscale_kernel, dim3(K), dim3(1024), 0, st, n, X, ldx, fr, gate, live);
   if (e == cudaSuccess) e = launch_pdl(digit_kernel, dim3(nkb), dim3(512), 0, st, n, K, X, ldx, fr, dig, ex, gate);
   if (e != cudaSuccess) return e;
 #define HPMXP_GEMV_K(KK) \

@@ -231,10 +231,11 @@ struct GemvSplit {
 bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, GemvSplit* split);
 // P[c][r][i] = the partial sums of row i in its tile's piece c; with abs_sums
 // also RS[c][i], the fp32 estimates of the |A| row sums.  prep: gemv_tc_bytes(n)
-// of scratch, 16-byte aligned.
+// of scratch, 16-byte aligned.  live: the right-hand sides whose sums are wanted,
+// by their flags (none given: all).
 size_t gemv_tc_bytes(int64_t n);
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
-                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate);
+                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate, Gate live);
 
 // precond.cu: z = U^{-1} L^{-1} v (of diag(cs) U^{-1} L^{-1} diag(rs) with rs, cs)
 // for K right-hand sides, in fp32 or fp64.  Once per solve: a plan, the inverted

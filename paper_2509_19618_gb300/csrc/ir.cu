@@ -735,11 +735,14 @@ bool gemv_on_tensor_cores(int64_t n, int K, const double* A, int64_t lda, int ab
   return true;
 }
 
-// out = b - A X (b may be NULL: out = A X), with optional norm tracking.  redo:
-// for a caller that does not read w.status, make a void product good (without norms).
+// out = b - A X (b may be NULL: out = A X), with optional norm tracking.  live:
+// the right-hand sides whose columns are wanted (none given: all; out's others are
+// unspecified).  redo: for a caller that does not read w.status, make a void
+// product good (without norms).
 cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx,
                      const double* B, int64_t ldb, double* out, int64_t ldo, int abs_mode, int track,
-                     const SolveWs& w, cudaStream_t st, Gate gate = {}, bool redo = false) {
+                     const SolveWs& w, cudaStream_t st, Gate gate = {}, Gate live = {},
+                     bool redo = false) {
   int nchunk = gemv_chunks(n, K);
   cudaError_t e;
   void* tok = prof_begin(st);
@@ -747,7 +750,7 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
   if (gemv_on_tensor_cores(n, K, A, lda, abs_mode, w, &split)) {
     // the digits live in the upper half of the row-sum scratch (fp64-sized; mode 1 keeps fp32 sums)
     void* prep = (char*)w.RS + round_up<size_t>(sizeof(float) * (size_t)gemv_chunks(n) * n, 256);
-    e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st, gate);
+    e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st, gate, live);
   } else {
     switch (K) {
       case 1: e = gemv_k<1>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
@@ -786,8 +789,8 @@ struct Solver {
   Report rep;
 
   size_t report_bytes() const { return offsetof(Report, brief) + sizeof(Brief) * K; }
-  // Gates of launches issued ahead of the host's knowledge: some right-hand side
-  // still wants refinement / Arnoldi steps
+  // The right-hand sides that still want refinement / Arnoldi steps; as gates of
+  // launches issued ahead of the host's knowledge: some still does
   Gate outer_gate() const { return {&w.st->outer_active, K, (int)(sizeof(RhsState) / sizeof(int))}; }
   Gate cycle_gate() const { return {&w.st->cycle_active, K, (int)(sizeof(RhsState) / sizeof(int))}; }
 
@@ -862,7 +865,7 @@ struct Solver {
   cudaError_t arnoldi_step(int j, bool ahead) {
     const Gate gate = ahead ? cycle_gate() : Gate{};
     cudaError_t e = residual(n, K, A, lda, w.V + (int64_t)j * n, ldv_rhs(), nullptr, 0, w.tmp, n,
-                             prm.matvec_fp32 ? 3 : 0, 0, w, st, gate);
+                             prm.matvec_fp32 ? 3 : 0, 0, w, st, gate, cycle_gate());
     if (e != cudaSuccess) return e;
     if ((e = precond(w.tmp, n, w.w, n, gate)) != cudaSuccess) return e;
     arnoldi_tail(j, gate);
@@ -880,7 +883,7 @@ struct Solver {
   // r = b - A x, norms; decide
   cudaError_t outer_check(bool first) {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
-    const cudaError_t e = residual(n, K, A, lda, X, ldx, B, ldb, w.r, n, first ? 1 : 0, 1, w, st);
+    const cudaError_t e = residual(n, K, A, lda, X, ldx, B, ldb, w.r, n, first ? 1 : 0, 1, w, st, {}, outer_gate());
     if (e != cudaSuccess) return e;
     launch_vec(w.pdl, check_kernel, dim3(1), dim3(32), st, sp, w.st, w.brief, first ? 1 : 0);
     count_launches(1);
@@ -1232,7 +1235,7 @@ hpmxp_status residual_vector(int64_t n, const double* A, int64_t lda, const doub
                              cudaStream_t st) {
   SolveWs w = carve_solve(ws, n, nrhs, 1);
   cudaError_t e = cudaMemsetAsync(w.status, 0, 4, st);
-  if (e == cudaSuccess) e = residual(n, (int)nrhs, A, lda, x, ldx, b, ldb, r, ldr, 0, 0, w, st, {}, true);
+  if (e == cudaSuccess) e = residual(n, (int)nrhs, A, lda, x, ldx, b, ldb, r, ldr, 0, 0, w, st, {}, {}, true);
   return status_from_cuda(e);
 }
 
