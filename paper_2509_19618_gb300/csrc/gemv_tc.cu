@@ -10,18 +10,27 @@
 //   - Column j of A and X is scaled by 2^e_j (e_j the largest exponent of x_j
 //     over the right-hand sides, each right-hand side normalised by its own
 //     2^f_r), so that A's entries carry the size of their products.
-//   - Row i's scaled entries become 56-bit magnitudes relative to a running
-//     2^E (E_i at least the largest exponent met in the row), cut into seven
-//     8-bit digits d_s with the entry's sign; X's scaled values become 56-bit
-//     integers in seven signed 8-bit digits t_u.  Digits are exact in fp16.
+//   - Row i's scaled entries become 64-bit magnitudes below 2^(E + 1) of a
+//     running exponent E, cut into eight 8-bit digits d_s with the entry's sign;
+//     X's scaled values become 63-bit integers in eight signed 8-bit digits t_u.
+//     Digits are exact in fp16.
 //   - tcgen05 accumulates D_w = sum_{s+u=w} d_s t_u, w = 0 .. 7, over 64
-//     columns: integers below 7 * 64 * 255 * 128 < 2^24, so every fp32 sum is
-//     exact.  Digit pairs with s + u > 7 are below 2^-63 of the largest product.
+//     columns: integers below 8 * 64 * 255 * 128 < 2^24, so every fp32 sum is
+//     exact.
 //   - D is added to 64-bit integers per row, right-hand side and half of the
 //     weights; they become fp64 once per work unit.
-// What is lost is the entries' bits below 2^(E - 56), three bits below fp64's
-// own last place of the largest product in the row, where the plain kernel
-// rounds once per product.
+// What is lost, against M_i = the largest |a_ij| 2^e_j met in the row's work unit
+// (2^E <= 4 M_i): the bits of an entry below 2^(E - 63), none of one within 2^8
+// of M_i; the bits of x_jr below 2^(e_j - 64), none of one within 2^10 of the
+// largest x in its column; and the digit pairs with s + u > 7, at most 7 * 2^-64
+// times 2^(E + 1).  Per column that is at most 2^-57 M_i, which is 2^-56 of the
+// row's largest product for one right-hand side and, since E follows columns whose
+// x_jr differ by 2^6 at most, 2^-50 of a side's own largest for several; the signs
+// differ from column to column.  The plain kernel rounds every partial sum at
+// 2^-53.  With seven digits on both sides a
+// Gaussian A with a dominant diagonal was 1.5 to 2.3 times less accurate than the
+// plain kernel (rms, n = 2048, two right-hand sides), rows whose largest products
+// cancel 16 to 21 times; with eight 0.006 and 0.08.
 //
 // An entry above 2^E (a diagonally dominant row's diagonal; a non-finite
 // entry, whose exponent exceeds every E in use) has no digits: its product is
@@ -39,9 +48,10 @@
 // buffers that the groups share.  A thread cuts its row's digits with integer
 // instructions and stores them to TMEM (the MMA's A operand).  Slice s adds to D's
 // columns 8 (s + u) + r of the block's 64.  Bound by the integer pipe (half the
-// issue rate; 34 instructions per entry, 17 of them integer: it is 56 % busy) and
-// the group's barriers; 1.57 ms for one and 1.86 ms for eight right-hand sides at
-// n = 32768 (5.5 and 4.6 TB/s of A), against 1.78 and 13.8 ms of fp64 FMAs.
+// issue rate) and the group's barriers; with seven digits 34 instructions per
+// entry, 17 of them integer (56 % busy), and the eighth costs 5 %: 432 -> 456 us at
+// n = 16384 with four right-hand sides, 1.49 -> 1.57 ms at 32768 with one (5.5 TB/s
+// of A), against 1.76 and 1.78 ms of fp64 FMAs.
 #include "tcgen05.h"
 
 #include <cuda_fp16.h>
@@ -60,12 +70,12 @@ constexpr int kBlk = 64;                     // columns of a block (exactness: s
 constexpr int kGroups = 4;
 constexpr int kTileRows = kGroups * kRowsT;
 constexpr int kThr = kTileRows;
-constexpr int kSlices = 7;
-constexpr int kDig = kSlices * 1024;         // bytes of a block's X digits: 7 groups of 8 rows x 128 bytes
+constexpr int kSlices = 8;
+constexpr int kDig = kSlices * 1024;         // bytes of a block's X digits: 8 groups of 8 rows x 128 bytes
 constexpr int kExpW = 2 * kBlk + 4;          // a block's column exponents (all, and of robust columns) and flag
 constexpr int kExp = kExpW * 4;              // in bytes, whole 16-byte pieces
-constexpr int kBBufs = 3;                    // digit buffers, a zero group of 8 rows before, between and after them
-constexpr int kBArea = (kBBufs * (kSlices + 1) + 1) * 1024;
+constexpr int kBBufs = 3;                    // digit buffers, a zero group of 8 rows before each
+constexpr int kBArea = kBBufs * (kSlices + 1) * 1024;
 constexpr int kCols = 16;                    // columns of a ring stage (one MMA's depth)
 constexpr int kStage = kCols * kRowsT * 8;
 constexpr int kStages = 2;                   // per group
@@ -74,7 +84,7 @@ constexpr int kNoExp = -400;                 // exponent of a column whose x is 
 // E's range: below it zero and subnormal entries would get digits, above it a
 // non-finite entry (exponent 2047) in a column of exponent kNoExp would not exceed it
 constexpr int kMinE = 64, kMaxE = 2047 + kNoExp - 1;
-static_assert(7ll * kBlk * 255 * 128 < (1 << 24), "exact fp32 sums");
+static_assert((long long)kSlices * kBlk * 255 * 128 < (1 << 24), "exact fp32 sums");
 constexpr int kBars = 2 * kBBufs + kGroups * kStages + 2 * kGroups;
 
 template <int K>
@@ -145,7 +155,7 @@ __global__ void __launch_bounds__(512) digit_kernel(int64_t n, int K, const doub
   for (int k = 0; k < K; ++k) em = max(em, es[k][jl]);
   bool robust = true;   // every right-hand side has a sizeable x in this column (or none has any)
   for (int k = 0; k < K; ++k) robust = robust && (es[k][jl] == INT_MIN || es[k][jl] >= em - 6);
-  long long q = em == kNoExp ? 0 : llrint(scalbn(v, 55 - f - em));
+  long long q = em == kNoExp ? 0 : llrint(scalbn(v, 63 - f - em));
   uint8_t* out = dig + (size_t)blockIdx.x * kDig + r * 128 + (((jl >> 3) ^ r) << 4) + (jl & 7) * 2;
 #pragma unroll
   for (int u = kSlices - 1; u >= 0; --u) {
@@ -208,6 +218,11 @@ __device__ __forceinline__ int mad(int x, int y, int z) {
 __device__ __forceinline__ uint32_t hfma2(uint32_t x, uint32_t y, uint32_t z) {
   uint32_t r;
   asm("fma.rn.f16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(x), "r"(y), "r"(z));
+  return r;
+}
+__device__ __forceinline__ uint32_t hmul2(uint32_t x, uint32_t y) {
+  uint32_t r;
+  asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(y));
   return r;
 }
 // |a| as in the plain kernel's ||A||_inf estimate (ir.cu): fp32 from the top word
@@ -468,7 +483,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
             const uint32_t st = apos % kStages;
             wait(a_full(g, st), (apos / kStages) & 1);
 #pragma unroll
-            for (int half = 0; half < 2; ++half) {   // 8 columns at a time: their digits are 28 registers
+            for (int half = 0; half < 2; ++half) {   // 8 columns at a time: their digits are 32 registers
               const double* col = reinterpret_cast<const double*>(ring + (g * kStages + st) * kStage) + 8 * half * kRowsT + tg;
               const int* ej = e0 + 16 * sub + 8 * half;
               int tmax = INT_MIN;
@@ -502,14 +517,14 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
                   tmax = __vimax3_s32(tmax, t2[0], t2[1]);
                   // digits as fp16: 0x6400 | u is 1024 + u; times the sign, minus 1024 times the sign
                   const uint32_t sg = __byte_perm(hi2[0], hi2[1], 0x7030);
-                  const uint32_t one = (sg & 0x80008000u) | 0x3c003c00u, off = (sg & 0x80008000u) ^ 0xe400e400u;
+                  const uint32_t one = (sg & 0x80008000u) | 0x3c003c00u, off = hmul2(one, 0xe400e400u);
 #pragma unroll
                   for (int s = 0; s < kSlices; s += 2) {   // two bytes of both entries, then each with the exponent byte
                     const uint32_t by = s < 4 ? __byte_perm(vh[0], vh[1], s == 0 ? 0x6723 : 0x4501)
                                               : __byte_perm(vl[0], vl[1], s == 4 ? 0x6723 : 0x4501);
                     const uint32_t u0 = __byte_perm(by, 0x64646464u, 0x4240), u1 = __byte_perm(by, 0x64646464u, 0x4341);
                     sl[s][2 * c4 + h] = hfma2(u0, one, off);
-                    if (s + 1 < kSlices) sl[s + 1][2 * c4 + h] = hfma2(u1, one, off);
+                    sl[s + 1][2 * c4 + h] = hfma2(u1, one, off);
                   }
                 }
               }
