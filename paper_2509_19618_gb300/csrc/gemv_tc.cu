@@ -38,7 +38,11 @@
 // row.  E follows columns that matter to every right-hand side (x_jr within
 // 2^6 of the column's largest for all r); with hardly any such column, and in
 // blocks with a non-finite x or an E at the ends of fp64's range, all products
-// are fp64 FMAs.
+// are fp64 FMAs, taken from the same stages (a second, direct read of A made
+// matrices with zero blocks, whose rows have no E there, and unlike right-hand
+// sides up to 2 times slower than gemv_partial_kernel).  Zero entries are skipped:
+// n = 16384, four right-hand sides, lower triangular 2740 -> 471 us, unlike
+// right-hand sides 2350 -> 1780 (the FMA kernel 1755).
 //
 // Layout: a CTA takes 512 rows, four groups of 128 threads (thread = row, TMEM
 // lane), by 64-column blocks.  A's columns come by TMA (16 columns x 128 rows per
@@ -49,8 +53,8 @@
 // instructions and stores them to TMEM (the MMA's A operand).  Slice s adds to D's
 // columns 8 (s + u) + r of the block's 64.  Bound by the integer pipe (half the
 // issue rate) and the group's barriers; with seven digits 34 instructions per
-// entry, 17 of them integer (56 % busy), and the eighth costs 5 %: 432 -> 456 us at
-// n = 16384 with four right-hand sides, 1.49 -> 1.57 ms at 32768 with one (5.5 TB/s
+// entry, 17 of them integer (56 % busy), and the eighth costs 5 %: 432 -> 458 us at
+// n = 16384 with four right-hand sides, 1.49 -> 1.58 ms at 32768 with one (5.4 TB/s
 // of A), against 1.76 and 1.78 ms of fp64 FMAs.
 #include "tcgen05.h"
 
@@ -233,7 +237,6 @@ __device__ __forceinline__ float abs_est(int hi) {
 
 struct GemvTc {
   int64_t n;
-  const double* A; int64_t lda;
   const double* X; int64_t ldx;
   const uint8_t* dig;
   const int* ex;
@@ -360,16 +363,17 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
     wend = p.split.begin(range + 1);
     a0 = apos;
     b0 = bpos;
-    if (tg == 32 && !plain) {
+    if (tg == 32) {
       for (a_loads = a0; a_loads < a0 + kStages; ++a_loads) load_a(a_loads);
-      if (g == 0)
+      if (g == 0 && !plain)
         for (b_loads = b0; b_loads < b0 + kBBufs - 1; ++b_loads) load_b(b_loads);
     }
     while (w < wend) {
-      const int tile = w / nkb, kb0 = w - tile * nkb, kb1 = min(nkb, kb0 + wend - w);
+      int tile = w / nkb, kb0 = w - tile * nkb;
+      const int kb1 = min(nkb, kb0 + wend - w);
       w += kb1 - kb0;
       const int piece = range - p.split.first_cta(tile);
-      const int64_t row = (int64_t)tile * kTileRows + tid, rowc = min(row, p.n - 1);
+      const int64_t row = (int64_t)tile * kTileRows + tid;
       double facc[K];                 // products taken in fp64, and the folded integers
 #pragma unroll
       for (int r = 0; r < K; ++r) {
@@ -391,26 +395,29 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
           hl[(K + r) * kTileRows + tid] = 0;
         }
       };
-      // block kb in fp64 from A and X, eight columns' loads at a time; the two largest scaled
-      // exponents among the robust columns into m1, m2
-      auto fp64_block = [&](int kb, const int* eg, int& m1, int& m2) {
-        const int64_t j0 = (int64_t)kb * kBlk, j1 = min(j0 + kBlk, p.n);
+      // a stage's columns, from j on, in fp64, for the rows that want it (`mine`).  all: zero entries
+      // count (x may be non-finite).  A row without an E keeps its two largest scaled exponents among
+      // the robust columns in otop, over
+      auto fp64_stage = [&](const double* col, const int* ej, int64_t j, bool all, bool mine) {
+        if (!all) {
+          uint32_t any = 0;
+#pragma unroll
+          for (int c = 0; c < kCols; ++c)
+            any |= ((uint32_t)__double2hiint(col[c * kRowsT]) << 1) | (uint32_t)__double2loint(col[c * kRowsT]);
+          if (any == 0) return;
+        }
+        const int cols = mine ? (int)min((int64_t)kCols, p.n - j) : 0;
 #pragma unroll 1
-        for (int64_t j = j0; j < j1; j += 8) {
-          double av[8];
+        for (int c = 0; c < cols; ++c) {
+          const double a = col[c * kRowsT];
 #pragma unroll
-          for (int c = 0; c < 8; ++c) av[c] = j + c < j1 ? p.A[rowc + (j + c) * p.lda] : 0.0;
-#pragma unroll
-          for (int c = 0; c < 8; ++c) {
-            if (kAbs && plain) rowsum += abs_est(__double2hiint(av[c]));
-            if (eg) {
-              const int t = (__double2hiint(av[c]) & 0x7fffffff) + eg[j + c - j0];
-              m2 = max(m2, min(m1, t));
-              m1 = max(m1, t);
-            }
-#pragma unroll
-            for (int r = 0; r < K; ++r)
-              facc[r] = __fma_rn(av[c], j + c < j1 ? __ldg(p.X + j + c + r * p.ldx) : 0.0, facc[r]);
+          for (int r = 0; r < K; ++r) facc[r] = __fma_rn(a, __ldg(p.X + j + c + r * p.ldx), facc[r]);
+          if (plain) {
+            if (kAbs) rowsum += abs_est(__double2hiint(a));
+          } else if (E < kMinE) {
+            const int t = (__double2hiint(a) & 0x7fffffff) + ej[kBlk + c];
+            over = max(over, min(otop, t));
+            otop = max(otop, t);
           }
         }
       };
@@ -447,153 +454,163 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
       };
 
       if (plain) {
-        int m1 = 0, m2 = 0;
-        for (int kb = kb0; kb < kb1; ++kb) fp64_block(kb, nullptr, m1, m2);
-      } else {
-        for (int kb = kb0; kb < kb1; ++kb, ++bpos) {
-          const int bb = bpos % kBBufs;
-          wait(b_full(bb), (bpos / kBBufs) & 1);
-          const int* e0 = exps + bb * kExpW;
-          if (kb == kb0) {
-            // E from the first 16 columns: one above the largest of the robust ones, unless that
-            // one stands alone (a dominant diagonal)
-            wait(a_full(g, apos % kStages), (apos / kStages) & 1);
-            const double* col = reinterpret_cast<const double*>(ring + (g * kStages + apos % kStages) * kStage) + tg;
-            int m1 = INT_MIN, m2 = INT_MIN;
-#pragma unroll
-            for (int c = 0; c < kCols; ++c) {
-              const int t = (__double2hiint(col[c * kRowsT]) & 0x7fffffff) + e0[kBlk + c];
-              m2 = max(m2, min(m1, t));
-              m1 = max(m1, t);
-            }
-            m1 >>= 20;
-            m2 >>= 20;
-            E = min(m1 - m2 <= 3 ? m1 + 1 : m2 + 2, kMaxE + 1);
-          }
-          const bool bad = E < kMinE || E > kMaxE || e0[2 * kBlk] != 0;   // this block in fp64
-          const int etop = E * (1 << 20) + 0xfffff;
-          int E_next = E;
-          if (bad) {
-            int m1 = INT_MIN, m2 = INT_MIN;
-            fp64_block(kb, e0 + kBlk, m1, m2);
-            if (E < kMinE) E_next = max(E, min((m2 >> 20) + 1, kMaxE + 1));
-          }
-#pragma unroll 1
-          for (int sub = 0; sub < 4; ++sub, ++apos) {
-            const uint32_t st = apos % kStages;
-            wait(a_full(g, st), (apos / kStages) & 1);
-#pragma unroll
-            for (int half = 0; half < 2; ++half) {   // 8 columns at a time: their digits are 32 registers
-              const double* col = reinterpret_cast<const double*>(ring + (g * kStages + st) * kStage) + 8 * half * kRowsT + tg;
-              const int* ej = e0 + 16 * sub + 8 * half;
-              int tmax = INT_MIN;
-              uint32_t sl[kSlices][4];
-#pragma unroll
-              for (int c4 = 0; c4 < 2; ++c4) {
-                const int4 ec4 = *reinterpret_cast<const int4*>(ej + 4 * c4);
-                const int ec[4] = {ec4.x, ec4.y, ec4.z, ec4.w};
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                  uint32_t vh[2], vl[2], hi2[2];
-                  int t2[2];
-#pragma unroll
-                  for (int b = 0; b < 2; ++b) {
-                    const double a = col[(4 * c4 + 2 * h + b) * kRowsT];
-                    const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
-                    hi2[b] = hi;
-                    if (kAbs) rowsum += abs_est((int)hi);
-                    t2[b] = mad((int)(hi & 0x7fffffffu), p.one, ec[2 * h + b]);
-                    // significand with its leading one at bit 63, then down to 2^E's scale; a zero or
-                    // subnormal entry shifts out (E >= kMinE), and so does one above 2^E (a negative
-                    // count, read unsigned)
-                    const uint64_t ml = (uint64_t)lo * p.k2048;
-                    const uint64_t m =
-                        ((uint64_t)((hi | 0x00100000u) * p.k2048 + (uint32_t)(ml >> 32)) << 32) | (uint32_t)ml;
-                    uint64_t v;
-                    asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"((uint32_t)(mad(t2[b], p.minus, etop) >> 20)));
-                    vh[b] = (uint32_t)(v >> 32);
-                    vl[b] = (uint32_t)v;
-                  }
-                  tmax = __vimax3_s32(tmax, t2[0], t2[1]);
-                  // digits as fp16: 0x6400 | u is 1024 + u; times the sign, minus 1024 times the sign
-                  const uint32_t sg = __byte_perm(hi2[0], hi2[1], 0x7030);
-                  const uint32_t one = (sg & 0x80008000u) | 0x3c003c00u, off = hmul2(one, 0xe400e400u);
-#pragma unroll
-                  for (int s = 0; s < kSlices; s += 2) {   // two bytes of both entries, then each with the exponent byte
-                    const uint32_t by = s < 4 ? __byte_perm(vh[0], vh[1], s == 0 ? 0x6723 : 0x4501)
-                                              : __byte_perm(vl[0], vl[1], s == 4 ? 0x6723 : 0x4501);
-                    const uint32_t u0 = __byte_perm(by, 0x64646464u, 0x4240), u1 = __byte_perm(by, 0x64646464u, 0x4341);
-                    sl[s][2 * c4 + h] = hfma2(u0, one, off);
-                    sl[s + 1][2 * c4 + h] = hfma2(u1, one, off);
-                  }
-                }
-              }
-              if (tmax > etop && !bad) {   // entries above 2^E: their products in fp64
-                // every lane its own columns, so that a warp on the diagonal takes one round
-                uint32_t above = 0;
-#pragma unroll
-                for (int c = 0; c < 8; ++c)
-                  above |= (uint32_t)((__double2hiint(col[c * kRowsT]) & 0x7fffffff) + ej[c] > etop) << c;
-                // columns past the last one are zeros, but after a wait that ran out the stage and the
-                // exponents hold anything: x has n entries
-                const int64_t left = p.n - ((int64_t)kb * kBlk + 16 * sub + 8 * half);
-                if (left < 8) above &= left > 0 ? (1u << left) - 1u : 0u;
-                while (above) {
-                  const int c = __ffs((int)above) - 1;
-                  above &= above - 1;
-                  const double a = col[c * kRowsT];
-                  const double* x = p.X + (int64_t)kb * kBlk + 16 * sub + 8 * half + c;
-#pragma unroll
-                  for (int r = 0; r < K; ++r) facc[r] = __fma_rn(a, __ldg(x + r * p.ldx), facc[r]);
-                  if (ej[kBlk + c] == ej[c]) {
-                    ++over;
-                    otop = max(otop, (__double2hiint(a) & 0x7fffffff) + ej[c]);
-                  }
-                }
-              }
-              if (half == 0) {
-                wait_mma();                    // the digits' TMEM is free, and D complete
-                if (sub == 0 && pend) flush();
-              }
-#pragma unroll
-              for (int s = 0; s < kSlices; ++s) tmem_st4(ta + lane_off + 8 * s + 4 * half, sl[s]);
-            }
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            tc_fence_before();
-            group_barrier(g);
-            if (tg == 0) {
-              tc_fence_after();
-              const uint32_t bd = digits_at(bb) + 32 * sub;
-#pragma unroll
-              for (int s = 0; s < kSlices; ++s)
-                // D's columns from 8 s on (an odd s starts a zero group and 8 columns earlier, so
-                // that the column counts are multiples of 16)
-                tc_mma_ts(td + 16 * (s / 2), ta + 8 * s, sdesc_sw128(bd - (s & 1) * 1024),
-                          make_idesc(0, 64 - 16 * (s / 2)), sub > 0 || s > 0);
-              if (sub == 3) tc_commit(b_empty(bb));
-              tc_commit(bar_mma);   // the last one, which the drain below waits for
-            } else if (tg == 32) {   // every thread of the group has read this stage
-              load_a(a_loads++);
-              if (g == 0 && sub == 2) load_b(b_loads++);
-            }
-            ++issued;
-          }
-          pend = true;
-          pend_bad = bad;
-          pend_E = E;
-          if (E != E_next || over >= 3) {
-            fold();
-            E = over >= 3 ? min(otop >> 20, kMaxE + 1) : E_next;
-            over = otop = 0;
-          }
+        for (int q = 4 * kb0; q < 4 * kb1; ++q, ++apos) {
+          const uint32_t st = apos % kStages;
+          wait(a_full(g, st), (apos / kStages) & 1);
+          fp64_stage(reinterpret_cast<const double*>(ring + (g * kStages + st) * kStage) + tg, exps, (int64_t)q * kCols, true,
+                     true);
+          group_barrier(g);
+          if (tg == 32) load_a(a_loads++);
         }
-        if (pend) {
-          wait_mma();
-          flush();
-          tc_fence_before();
-        }
-        fold();
+        kb0 = kb1;
       }
+      for (int kb = kb0; kb < kb1; ++kb, ++bpos) {
+        const int bb = bpos % kBBufs;
+        wait(b_full(bb), (bpos / kBBufs) & 1);
+        const int* e0 = exps + bb * kExpW;
+        if (kb == kb0) {
+          // E from the first 16 columns: one above the largest of the robust ones, unless that
+          // one stands alone (a dominant diagonal)
+          wait(a_full(g, apos % kStages), (apos / kStages) & 1);
+          const double* col = reinterpret_cast<const double*>(ring + (g * kStages + apos % kStages) * kStage) + tg;
+          int m1 = INT_MIN, m2 = INT_MIN;
+#pragma unroll
+          for (int c = 0; c < kCols; ++c) {
+            const int t = (__double2hiint(col[c * kRowsT]) & 0x7fffffff) + e0[kBlk + c];
+            m2 = max(m2, min(m1, t));
+            m1 = max(m1, t);
+          }
+          m1 >>= 20;
+          m2 >>= 20;
+          E = min(m1 - m2 <= 3 ? m1 + 1 : m2 + 2, kMaxE + 1);
+        }
+        const bool odd_x = e0[2 * kBlk] != 0;
+        const bool bad = odd_x || E < kMinE || E > kMaxE;   // this block in fp64
+        const int etop = E * (1 << 20) + 0xfffff;
+        if (E < kMinE) over = otop = INT_MIN;
+        // one branch per warp and behind the digits: a row's own ahead of them cost every block 4 %
+        const bool any_bad = __any_sync(0xffffffffu, bad);
+#pragma unroll 1
+        for (int sub = 0; sub < 4; ++sub, ++apos) {
+          const uint32_t st = apos % kStages;
+          wait(a_full(g, st), (apos / kStages) & 1);
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {   // 8 columns at a time: their digits are 32 registers
+            const double* col = reinterpret_cast<const double*>(ring + (g * kStages + st) * kStage) + 8 * half * kRowsT + tg;
+            const int* ej = e0 + 16 * sub + 8 * half;
+            int tmax = INT_MIN;
+            uint32_t sl[kSlices][4];
+#pragma unroll
+            for (int c4 = 0; c4 < 2; ++c4) {
+              const int4 ec4 = *reinterpret_cast<const int4*>(ej + 4 * c4);
+              const int ec[4] = {ec4.x, ec4.y, ec4.z, ec4.w};
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                uint32_t vh[2], vl[2], hi2[2];
+                int t2[2];
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                  const double a = col[(4 * c4 + 2 * h + b) * kRowsT];
+                  const uint32_t hi = (uint32_t)__double2hiint(a), lo = (uint32_t)__double2loint(a);
+                  hi2[b] = hi;
+                  if (kAbs) rowsum += abs_est((int)hi);
+                  t2[b] = mad((int)(hi & 0x7fffffffu), p.one, ec[2 * h + b]);
+                  // significand with its leading one at bit 63, then down to 2^E's scale; a zero or
+                  // subnormal entry shifts out (E >= kMinE), and so does one above 2^E (a negative
+                  // count, read unsigned)
+                  const uint64_t ml = (uint64_t)lo * p.k2048;
+                  const uint64_t m =
+                      ((uint64_t)((hi | 0x00100000u) * p.k2048 + (uint32_t)(ml >> 32)) << 32) | (uint32_t)ml;
+                  uint64_t v;
+                  asm("shr.u64 %0, %1, %2;" : "=l"(v) : "l"(m), "r"((uint32_t)(mad(t2[b], p.minus, etop) >> 20)));
+                  vh[b] = (uint32_t)(v >> 32);
+                  vl[b] = (uint32_t)v;
+                }
+                tmax = __vimax3_s32(tmax, t2[0], t2[1]);
+                // digits as fp16: 0x6400 | u is 1024 + u; times the sign, minus 1024 times the sign
+                const uint32_t sg = __byte_perm(hi2[0], hi2[1], 0x7030);
+                const uint32_t one = (sg & 0x80008000u) | 0x3c003c00u, off = hmul2(one, 0xe400e400u);
+#pragma unroll
+                for (int s = 0; s < kSlices; s += 2) {   // two bytes of both entries, then each with the exponent byte
+                  const uint32_t by = s < 4 ? __byte_perm(vh[0], vh[1], s == 0 ? 0x6723 : 0x4501)
+                                            : __byte_perm(vl[0], vl[1], s == 4 ? 0x6723 : 0x4501);
+                  const uint32_t u0 = __byte_perm(by, 0x64646464u, 0x4240), u1 = __byte_perm(by, 0x64646464u, 0x4341);
+                  sl[s][2 * c4 + h] = hfma2(u0, one, off);
+                  sl[s + 1][2 * c4 + h] = hfma2(u1, one, off);
+                }
+              }
+            }
+            if (tmax > etop && !bad) {   // entries above 2^E: their products in fp64
+              // every lane its own columns, so that a warp on the diagonal takes one round
+              uint32_t above = 0;
+#pragma unroll
+              for (int c = 0; c < 8; ++c)
+                above |= (uint32_t)((__double2hiint(col[c * kRowsT]) & 0x7fffffff) + ej[c] > etop) << c;
+              // columns past the last one are zeros, but after a wait that ran out the stage and the
+              // exponents hold anything: x has n entries
+              const int64_t left = p.n - ((int64_t)kb * kBlk + 16 * sub + 8 * half);
+              if (left < 8) above &= left > 0 ? (1u << left) - 1u : 0u;
+              while (above) {
+                const int c = __ffs((int)above) - 1;
+                above &= above - 1;
+                const double a = col[c * kRowsT];
+                const double* x = p.X + (int64_t)kb * kBlk + 16 * sub + 8 * half + c;
+#pragma unroll
+                for (int r = 0; r < K; ++r) facc[r] = __fma_rn(a, __ldg(x + r * p.ldx), facc[r]);
+                if (ej[kBlk + c] == ej[c]) {
+                  ++over;
+                  otop = max(otop, (__double2hiint(a) & 0x7fffffff) + ej[c]);
+                }
+              }
+            }
+            if (half == 0) {
+              wait_mma();                    // the digits' TMEM is free, and D complete
+              if (sub == 0 && pend) flush();
+            }
+#pragma unroll
+            for (int s = 0; s < kSlices; ++s) tmem_st4(ta + lane_off + 8 * s + 4 * half, sl[s]);
+          }
+          if (any_bad)
+            fp64_stage(reinterpret_cast<const double*>(ring + (g * kStages + st) * kStage) + tg, e0 + kCols * sub,
+                       (int64_t)kb * kBlk + kCols * sub, odd_x, bad);
+          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+          tc_fence_before();
+          group_barrier(g);
+          if (tg == 0) {
+            tc_fence_after();
+            const uint32_t bd = digits_at(bb) + 32 * sub;
+#pragma unroll
+            for (int s = 0; s < kSlices; ++s)
+              // D's columns from 8 s on (an odd s starts a zero group and 8 columns earlier, so
+              // that the column counts are multiples of 16)
+              tc_mma_ts(td + 16 * (s / 2), ta + 8 * s, sdesc_sw128(bd - (s & 1) * 1024),
+                        make_idesc(0, 64 - 16 * (s / 2)), sub > 0 || s > 0);
+            if (sub == 3) tc_commit(b_empty(bb));
+            tc_commit(bar_mma);   // the last one, which the drain below waits for
+          } else if (tg == 32) {   // every thread of the group has read this stage
+            load_a(a_loads++);
+            if (g == 0 && sub == 2) load_b(b_loads++);
+          }
+          ++issued;
+        }
+        pend = true;
+        pend_bad = bad;
+        pend_E = E;
+        if (E < kMinE) {   // nothing in H, L or D yet
+          E = max(E, min((over >> 20) + 1, kMaxE + 1));
+          over = otop = 0;
+        } else if (over >= 3) {
+          fold();
+          E = min(otop >> 20, kMaxE + 1);
+          over = otop = 0;
+        }
+      }
+      if (pend) {
+        wait_mma();
+        flush();
+        tc_fence_before();
+      }
+      fold();
       if (row < p.n) {
 #pragma unroll
         for (int r = 0; r < K; ++r) p.P[((int64_t)piece * K + r) * p.n + row] = facc[r];
@@ -668,7 +685,7 @@ cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double
                     Gate live) {
   const int nkb = (int)cdiv<int64_t>(n, kBlk);
   GemvTc p{};
-  p.n = n; p.A = A; p.lda = lda; p.X = X; p.ldx = ldx;
+  p.n = n; p.X = X; p.ldx = ldx;
   uint8_t* dig = (uint8_t*)prep;
   int* ex = (int*)(dig + (size_t)nkb * kDig);
   int* fr = ex + (size_t)nkb * kExpW;
