@@ -14,10 +14,12 @@
 // 16-byte, bank-conflict-free accesses.
 //
 // Large products of depth 512 run on pairs of CTAs (kPair): rank 0 issues the
-// MMAs of both, is told by rank 1's MMA warp when that CTA's operands are there
-// (arrivals without a cluster-scope acquire or release: only the tensor cores
-// read them, and those fences took 0.5 us a stage), and commits to both CTAs'
-// barriers; each CTA has its own producer, epilogue and C movers.
+// MMAs of both and commits to both CTAs' barriers; each CTA has its own producer,
+// epilogue and C movers.  Both producers' loads complete on rank 0's barrier, so
+// that the bytes of rank 1's shared memory are ordered before the MMAs that read
+// them as those of its own are (no relay by a thread of rank 1, whose cluster-scope
+// fences took 0.5 us a stage); rank 1's epilogue frees an accumulator, once per
+// tile, by an arrival at cluster scope.
 //
 // Roles: warp 0 TMA producer of the operand ring; warp 1 TMEM owner and MMA
 // issuer; warps 2..9 epilogue in two groups of four (warp w reads TMEM lanes
@@ -76,7 +78,7 @@ struct TileCfg {
   static constexpr int kSegs = TI / 128;                    // 64-row segments of an epilogue group's TI/2 rows
   static constexpr int kSegBoxes = kBoxes / kSegs;          // C boxes of a segment
   static constexpr int kCSlots = kCBufs * kEpiGroups * kSegs;
-  static constexpr int kBars = 2 * kStages + 5 + 2 * kCSlots + (kPair ? kStages : 0);
+  static constexpr int kBars = 2 * kStages + 5 + 2 * kCSlots;
   static constexpr size_t kSmem = 1024 + (size_t)kStages * (kStageA + kStageB) + (size_t)kCBufs * kCTile +
                                   8 * kBars + 16;
 };
@@ -198,9 +200,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   };
   auto c_done = [&](int b, int g, int h) { return c_full(b, g, h) + 8u * (uint32_t)Cfg::kCSlots; };
   const uint32_t mma_drain = bar0 + 8u * (uint32_t)(2 * kStages + 4 + 2 * Cfg::kCSlots);
-  // (pair, rank 0) the other CTA's operands of stage s are there
-  auto peer_full = [&](int s) { return mma_drain + 8u * (uint32_t)(1 + s); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + Cfg::kBars);
+  // (pair) stages loaded by the producers of ranks 0 and 1 and used by the MMAs, when they have ended
+  volatile int* ended = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = kPair ? (int)cluster_rank() : 0;
@@ -258,8 +260,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           mbar_init(c_done(b, g, h), kEpiWarps);
         }
     mbar_init(mma_drain, 1);
-    if (kPair)
-      for (int s = 0; s < kStages; ++s) mbar_init(peer_full(s), 1);
     fence_mbar_init();
     if (items == nullptr) {
       asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tmA) : "memory");
@@ -287,16 +287,38 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   pdl_trigger();
   if (p.span && threadIdx.x == 0) atomicMin(p.span, global_ns());
 
+  // operand ring: stage s holds K bytes [128 kb, +128) of the tile's rows j (A) and rows i (B);
+  // pos: ring position over all tiles of this CTA
+  auto load_stage = [&](const TileLoc& L, int kb, long long pos) {
+    const int s = (int)(pos % kStages);
+    if constexpr (kPair) {
+      if (rank == 0) mbar_expect_tx(full(s), 2 * (kStageA + kStageB));
+      const uint32_t bar = smem_at(full(s), 0);
+      tma_load_2d_pair(sOpA + s * kStageA, L.b, kb * (kRowBytes / 2), L.j0, bar);
+      tma_load_2d_pair(sOpB + s * kStageB, L.a, kb * (kRowBytes / 2), L.i0 + rank * Cfg::kRowsB, bar);
+    } else {
+      mbar_expect_tx(full(s), kStageA + kStageB);
+      tma_load_2d(sOpA + s * kStageA, L.b, kb * (kRowBytes / 2), L.j0, full(s));
+      tma_load_2d(sOpB + s * kStageB, L.a, kb * (kRowBytes / 2), L.i0, full(s));
+    }
+  };
+  // the last load of every stage has landed before the CTA (or its pair) can exit
+  auto drain_loads = [&](long long pos) {
+    for (long long q = (pos > kStages ? pos - kStages : 0); q < pos; ++q)
+      if (!mbar_wait(full((int)(q % kStages)), (uint32_t)((q / kStages) & 1))) atomicOr(p.status, kErrTimeout);
+  };
+  auto report_end = [&](int which, long long pos) {
+    for (int r = 0; r < 2; ++r) store_at(smem_at(smem_u32(tmem_slot + 1 + which), (uint32_t)r), (int)pos);
+  };
+
   if (warp == 0) {
     if (lane == 0) {
-      // operand ring: stage s holds K bytes [128 kb, +128) of the tile's rows j (A) and rows i (B)
-      long long pos = 0;   // ring position over all tiles of this CTA
+      long long pos = 0;
       bool ok = true;
       acquire_maps(0);
       acquire_maps(1);
       for (int t = first(); t < p.ntiles && ok; t += stride()) {
         const TileLoc L = locate(t);
-        const int i0 = L.i0, j0 = L.j0;
         for (int kb = 0; kb < p.nkb; ++kb, ++pos) {
           const int s = (int)(pos % kStages);
           const long long use = pos / kStages;
@@ -304,31 +326,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
             ok = false;
             break;
           }
-          mbar_expect_tx(full(s), kStageA + kStageB);
-          tma_load_2d(sOpA + s * kStageA, L.b, kb * (kRowBytes / 2), j0, full(s));
-          tma_load_2d(sOpB + s * kStageB, L.a, kb * (kRowBytes / 2), i0 + rank * Cfg::kRowsB, full(s));
+          load_stage(L, kb, pos);
         }
       }
       if (!ok) atomicOr(p.status, kErrTimeout);
-      // drain: the last load of every stage has landed before the CTA can exit
-      for (long long q = (pos > kStages ? pos - kStages : 0); q < pos; ++q)
-        if (!mbar_wait(full((int)(q % kStages)), (uint32_t)((q / kStages) & 1))) atomicOr(p.status, kErrTimeout);
+      if constexpr (kPair) report_end(rank, pos);   // drained below, together
+      else drain_loads(pos);
     }
   } else if (kPair && warp == 1 && rank == 1) {
-    // the MMAs are issued by rank 0, which is told when this CTA's operands are there
-    if (lane == 0) {
-      long long pos = 0;
-      bool ok = true;
-      for (int t = first(); t < p.ntiles && ok; t += stride())
-        for (int kb = 0; kb < p.nkb; ++kb, ++pos) {
-          const int s = (int)(pos % kStages);
-          if (!mbar_wait(full(s), (uint32_t)((pos / kStages) & 1), p.wait_polls, p.wait_ns)) { ok = false; break; }
-          mbar_arrive_at(peer_full(s), 0);
-        }
-      if (!ok) atomicOr(p.status, kErrTimeout);
-      // rank 0's MMAs, which read this CTA's shared memory and write its tensor memory, have completed
-      if (!mbar_wait(mma_drain, 0)) atomicOr(p.status, kErrTimeout);
-    }
+    // the MMAs are issued by rank 0
   } else if (warp == 1) {
     if (lane == 0) {
       auto commit = [](uint32_t bar) {
@@ -341,7 +347,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       int local = 0;
       for (int t = first(); t < p.ntiles && ok; t += stride(), ++local) {
         const int ab = local % p.nbuf, ause = local / p.nbuf;
-        if (ause > 0 && !mbar_wait(acc_empty(ab), (uint32_t)((ause - 1) & 1), p.wait_polls, p.wait_ns)) {
+        const uint32_t aph = (uint32_t)((ause - 1) & 1);
+        if (ause > 0 &&
+            !bounded_wait([&] { return kPair ? mbar_try_cluster(acc_empty(ab), aph) : mbar_try(acc_empty(ab), aph); },
+                          p.wait_polls, p.wait_ns)) {
           ok = false;
           break;
         }
@@ -350,8 +359,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         for (int kb = 0; kb < p.nkb; ++kb, ++pos) {
           const int s = (int)(pos % kStages);
           const uint32_t ph = (uint32_t)((pos / kStages) & 1);
-          if (!mbar_wait(full(s), ph, p.wait_polls, p.wait_ns) ||
-              (kPair && !mbar_wait(peer_full(s), ph, p.wait_polls, p.wait_ns))) {
+          if (!mbar_wait(full(s), ph, p.wait_polls, p.wait_ns)) {
             ok = false;
             break;
           }
@@ -377,6 +385,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       // epilogue group gave up before the last accumulator was written
       commit(mma_drain);
       if (!mbar_wait(mma_drain, 0)) atomicOr(p.status, kErrTimeout);
+      if constexpr (kPair) report_end(2, pos);
     }
   } else if (warp >= 2 + kEpiGroups * kEpiWarps) {
     // C mover of group g: a segment's C is loaded ahead of the epilogue, and
@@ -510,7 +519,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
           tc_fence_before();
           __syncwarp();
           if (lane == 0) {
-            if constexpr (kPair) mbar_arrive_at(acc_empty(ab), 0);
+            if (kPair && rank == 1) mbar_arrive_cluster(smem_at(acc_empty(ab), 0));
             else mbar_arrive(acc_empty(ab));
           }
         }
@@ -577,8 +586,25 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
   }
   tc_fence_before();
   __syncthreads();
-  // neither CTA of a pair leaves while the other may still read its shared memory or arrive there
-  if constexpr (kPair) cluster_sync();
+  if constexpr (kPair) {
+    // neither CTA of a pair leaves while the other may still read its shared memory or arrive there
+    cluster_sync();
+    if (ended[0] != ended[1] || ended[0] != ended[2]) {
+      // A wait ran out (the same three values, so the same decision in both CTAs).  A stage loaded by
+      // one rank only would never complete on rank 0's barrier: the other rank loads it too.  The stage
+      // is free there, since the MMAs before it released both CTAs' together.  Then rank 0 waits for all.
+      const int most = max(ended[0], ended[1]);
+      if (threadIdx.x == 0) {
+        for (int pos = ended[rank]; pos < most; ++pos) load_stage(locate(first() + pos / p.nkb * stride()), pos % p.nkb, pos);
+        if (rank == 0) drain_loads(most);
+      }
+      __syncthreads();
+      cluster_sync();
+    }
+    // rank 0's last commit arrives here too
+    if (rank == 1 && threadIdx.x == 32 && !mbar_wait(mma_drain, 0)) atomicOr(p.status, kErrTimeout);
+    __syncwarp();
+  }
   if (warp == 1) {
     tc_fence_after();
     if constexpr (kPair) tmem_dealloc_pair(tmem, p.ncols);

@@ -31,15 +31,19 @@ __device__ inline bool mbar_try(uint32_t bar, uint32_t parity) {
 }
 // Bounded wait for the phase with the given parity to complete: at most
 // `polls` polls and `ns` nanoseconds (the defaults for the drain waits).
-__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, long long polls = kSpinLimit,
-                                 unsigned long long ns = kWaitNs) {
-  if (mbar_try(bar, parity)) return true;
+template <class Try>
+__device__ inline bool bounded_wait(Try&& done, long long polls, unsigned long long ns) {
+  if (done()) return true;
   const unsigned long long t0 = global_ns();
   for (long long i = 1; i < polls; ++i) {
-    if (mbar_try(bar, parity)) return true;
+    if (done()) return true;
     if ((i & 255) == 0 && global_ns() - t0 > ns) return false;
   }
   return false;
+}
+__device__ inline bool mbar_wait(uint32_t bar, uint32_t parity, long long polls = kSpinLimit,
+                                 unsigned long long ns = kWaitNs) {
+  return bounded_wait([&] { return mbar_try(bar, parity); }, polls, ns);
 }
 
 __device__ inline void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
@@ -126,11 +130,40 @@ __device__ inline uint32_t cluster_rank() {
 __device__ inline void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-// Arrive on the barrier at `bar`'s offset in CTA `rank` of the cluster.
-__device__ inline void mbar_arrive_at(uint32_t bar, uint32_t rank) {
+// The shared-memory address `addr` of CTA `rank` of the cluster.
+__device__ inline uint32_t smem_at(uint32_t addr, uint32_t rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(addr), "r"(rank));
+  return a;
+}
+__device__ inline void store_at(uint32_t cluster_addr, int v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+// Arrive on a barrier of the other CTA, and wait for a barrier that the other CTA
+// arrives on, relaxed at cluster scope: the two order the execution, and between
+// tcgen05.fence::before_thread_sync and ::after_thread_sync that orders the tensor
+// memory accesses on both sides.  (Release and acquire would order ordinary
+// accesses too, which nothing here needs: 0.5 us each.)
+__device__ inline void mbar_arrive_cluster(uint32_t cluster_bar) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_bar) : "memory");
+}
+__device__ inline bool mbar_try_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
   asm volatile(
-      "{\n .reg .b32 a;\n mapa.shared::cluster.u32 a, %0, %1;\n"
-      " mbarrier.arrive.shared::cluster.b64 _, [a];\n}\n" ::"r"(bar), "r"(rank)
+      "{\n .reg .pred p;\n mbarrier.try_wait.parity.relaxed.cluster.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// A load into this CTA's shared memory whose bytes complete on a barrier of either
+// CTA of the pair.
+__device__ inline void tma_load_2d_pair(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t cluster_bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+      "[%4];" ::"r"(dst),
+      "l"((uint64_t)tm), "r"(x), "r"(y), "r"(cluster_bar)
       : "memory");
 }
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows of
