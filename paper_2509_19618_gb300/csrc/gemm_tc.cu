@@ -850,11 +850,15 @@ cudaError_t gemm_tc(const GemmArgs& g, cudaStream_t st) {
   if (!g.fp8 && g.M >= 256 && g.K >= 256 && wide_tiles_enabled()) {
     // Pairs of CTAs where the operands' intake is the bound: a depth of 512 and
     // more tiles than SMs.  Pairs / single CTAs, C -= A B, us: order 28672, depth
-    // 512: 728 / 894; 16384: 257 / 284; 8192: 83 / 93; 3072: 29.5 / 30.3; 2048
+    // 512: 710 / 884; 16384: 245 / 284; 8192: 80 / 93; 3072: 28.5 / 30.3; 2048
     // (fewer tiles than SMs): 25.7 / 25.1; depth 384 at 16384: 246 / 241; depth
-    // 256 at 28672: 699 / 687 (the C round trip bounds both).
+    // 256 at 28672: 699 / 687 (the C round trip bounds both).  An odd number of
+    // 128-column tiles leaves half of the last pairs empty, which pays from seven
+    // on: 30000 rows, 128 columns (a panel's) 35.5 / 28.5; 384: 34.3 / 32.5; 512:
+    // 33.4 / 36.0; 640: 38.6 / 37.7; 896: 46.6 / 49.1.
     const int cap = g.max_ctas > 0 ? std::min(g.max_ctas, grid_cap()) : grid_cap();
-    if (g.K >= 512 && cap >= 2 && 2LL * cdiv(g.M, 256) * cdiv(g.N, 2 * kTJ) > num_sms())
+    const int jt = cdiv(g.N, kTJ);
+    if (g.K >= 512 && cap >= 2 && (jt % 2 == 0 || jt >= 7) && (long long)cdiv(g.M, 256) * jt > num_sms())
       return gemm_tc_tiles<256, 2, true>(g, st);
     return gemm_tc_tiles<256>(g, st);
   }
