@@ -644,7 +644,7 @@ struct SolveWs {
 int gemv_chunks(int64_t n, int K = kMaxK) {
   const int64_t rb = cdiv<int64_t>(n, kGemvRows);
   const int64_t spread = std::min<int64_t>(cdiv<int64_t>(8 * 152, rb), cdiv<int64_t>(n, 32));
-  int64_t c = std::max<int64_t>(cdiv<int64_t>(n * K, kGemvChunkElems), spread);
+  int64_t c = std::max<int64_t>(cdiv<int64_t>(n, kGemvChunkElems / K), spread);   // chunk = ceil(n / c) columns
   c = std::max<int64_t>(1, std::min<int64_t>(c, cdiv<int64_t>(n, 8)));
   return (int)c;
 }
@@ -696,7 +696,7 @@ template <int K>
 cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int64_t ldx, int abs_mode,
                    const SolveWs& w, int nchunk, cudaStream_t st, Gate gate) {
   const int64_t chunk = cdiv<int64_t>(n, nchunk);
-  if (chunk * K > kGemvChunkElems) return cudaErrorInvalidValue;
+  if (chunk * K > kGemvChunkElems) return cudaErrorInvalidValue;   // gemv_chunks never gives that
   dim3 grid((unsigned)cdiv<int64_t>(n, kGemvRows), (unsigned)nchunk);
   const int T = kGemvThreads;
   double* P = w.P;
