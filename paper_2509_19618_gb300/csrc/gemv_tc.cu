@@ -656,13 +656,14 @@ int sm_count() {
 }
 
 template <int K, bool kAbs>
-cudaError_t launch_k(const CUtensorMap& tm, const GemvTc& p, cudaStream_t st) {
+cudaError_t launch_k(const CUtensorMap& tm, const GemvTc& p, cudaStream_t st, bool pdl) {
   // one value for every call: concurrent solves on other threads set the same
   cudaError_t e = cudaFuncSetAttribute(gemv_tc_kernel<K, kAbs>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)gemv_smem<K>());
   if (e != cudaSuccess) return e;
   const int budget = sm_budget();
-  return launch_pdl(gemv_tc_kernel<K, kAbs>, dim3(budget > 0 ? std::min(budget, p.split.ctas) : p.split.ctas), dim3(kThr), gemv_smem<K>(), st, tm, p);
+  const int grid = budget > 0 ? std::min(budget, p.split.ctas) : p.split.ctas;
+  return launch_vec(pdl, gemv_tc_kernel<K, kAbs>, dim3(grid), dim3(kThr), gemv_smem<K>(), st, tm, p);
 }
 
 }  // namespace
@@ -681,7 +682,7 @@ bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, Gemv
 }
 
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
-                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate,
+                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, bool pdl, Gate gate,
                     Gate live) {
   const int nkb = (int)cdiv<int64_t>(n, kBlk);
   GemvTc p{};
@@ -701,11 +702,11 @@ cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double
   CUtensorMap tm;
   if (!encode_f64_map(&tm, A, n, n, lda, kRowsT, kCols)) return cudaErrorInvalidValue;
   count_launches(3);
-  cudaError_t e = launch_pdl(xscale_kernel, dim3(K), dim3(1024), 0, st, n, X, ldx, fr, gate, live);
-  if (e == cudaSuccess) e = launch_pdl(digit_kernel, dim3(nkb), dim3(512), 0, st, n, K, X, ldx, fr, dig, ex, gate);
+  cudaError_t e = launch_vec(pdl, xscale_kernel, dim3(K), dim3(1024), 0, st, n, X, ldx, fr, gate, live);
+  if (e == cudaSuccess) e = launch_vec(pdl, digit_kernel, dim3(nkb), dim3(512), 0, st, n, K, X, ldx, fr, dig, ex, gate);
   if (e != cudaSuccess) return e;
 #define HPMXP_GEMV_K(KK) \
-  case KK: return abs_sums ? launch_k<KK, true>(tm, p, st) : launch_k<KK, false>(tm, p, st)
+  case KK: return abs_sums ? launch_k<KK, true>(tm, p, st, pdl) : launch_k<KK, false>(tm, p, st, pdl)
   switch (K) {
     HPMXP_GEMV_K(1);
     HPMXP_GEMV_K(2);

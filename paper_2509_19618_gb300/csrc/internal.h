@@ -232,10 +232,11 @@ bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, Gemv
 // P[c][r][i] = the partial sums of row i in its tile's piece c; with abs_sums
 // also RS[c][i], the fp32 estimates of the |A| row sums.  prep: gemv_tc_bytes(n)
 // of scratch, 16-byte aligned.  live: the right-hand sides whose sums are wanted,
-// by their flags (none given: all).
+// by their flags (none given: all).  pdl: as launch_vec.
 size_t gemv_tc_bytes(int64_t n);
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,
-                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, Gate gate, Gate live);
+                    void* prep, double* P, void* RS, const GemvSplit& split, uint32_t* status, cudaStream_t st, bool pdl, Gate gate,
+                    Gate live);
 
 // precond.cu: z = U^{-1} L^{-1} v (of diag(cs) U^{-1} L^{-1} diag(rs) with rs, cs)
 // for K right-hand sides, in fp32 or fp64.  Once per solve: a plan, the inverted
@@ -325,6 +326,21 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
                        Args&&... args) {
   return launch_pdl_cluster(kernel, 1, grid, block, smem, st, static_cast<Args&&>(args)...);
 }
+#ifdef __CUDACC__
+// launch_pdl, or a plain launch.  For the refinement's kernels: dependents of one
+// another for one system, whose kernels of a few microseconds otherwise start 2 to 3
+// us apart (n = 1024: 575 -> 500 us, 8192 with eight right-hand sides 5.40 -> 5.31
+// ms); plain where other streams share the chip (a batch's systems, an SM budget),
+// since the CTAs that wait take room from their kernels (24 mixed systems 8.55 ms,
+// 8.80 as dependents).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_vec(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                       Args&&... args) {
+  if (pdl) return launch_pdl(kernel, grid, block, smem, st, static_cast<Args&&>(args)...);
+  kernel<<<grid, block, smem, st>>>(static_cast<Args&&>(args)...);
+  return cudaGetLastError();
+}
+#endif
 
 void* prof_begin(cudaStream_t st);
 // work: the kind's unit (flops or bytes, see hpmxp.h); bytes: algorithmic DRAM

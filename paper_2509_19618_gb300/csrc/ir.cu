@@ -621,7 +621,7 @@ struct SolveWs {
   Brief* brief;
   unsigned int* counter;
   size_t control_bytes;   // report .. counter, zeroed at the start of a solve
-  bool pdl = true;        // programmatic launches (launch_vec)
+  bool pdl;               // programmatic launches (launch_vec): not where the call shares the chip
   double* partials;  // kMaxK * kRedBlocks
   double* r;         // n x K
   double* w;         // n x K
@@ -674,19 +674,9 @@ SolveWs carve_solve(void* base, int64_t n, int64_t K, int m) {
   w.pub = take(precond_pub_bytes(n, K));
   w.dinv = take(precond_inverse_bytes(n));
   w.chain = take(precond_chain_bytes(n));
+  w.pdl = sm_budget() <= 0;   // under a budget the call shares the chip, as a batch's systems do
   w.bytes = off;
   return w;
-}
-
-// The refinement's kernels: as programmatic dependents of one another for one
-// system, whose kernels of a few microseconds otherwise start 2 to 3 us apart (n =
-// 1024: 575 -> 500 us, 8192 with eight right-hand sides 5.40 -> 5.31 ms); as plain
-// launches for the systems of a batch, where the CTAs that wait take room from
-// other streams' kernels (24 mixed systems 8.55 ms, 8.80 as dependents).
-template <typename... KArgs, typename... Args>
-void launch_vec(bool pdl, void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args&&... args) {
-  if (pdl) launch_pdl(kernel, grid, block, 0, st, static_cast<Args&&>(args)...);
-  else kernel<<<grid, block, 0, st>>>(static_cast<Args&&>(args)...);
 }
 
 // abs_mode: 0 plain, 1 with the fp32 |A| estimate (the first residual; also
@@ -703,16 +693,16 @@ cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int
   void* RS = w.RS;
   if (abs_mode == 3 && w.a32) {
     dim3 g32((unsigned)cdiv<int64_t>(n, kGemv32Rows), (unsigned)nchunk);
-    launch_vec(w.pdl, gemv32_partial_kernel<K>, g32, dim3(T), st, n, w.a32, w.ld32, X, ldx, chunk, P, gate);
+    launch_vec(w.pdl, gemv32_partial_kernel<K>, g32, dim3(T), 0, st, n, w.a32, w.ld32, X, ldx, chunk, P, gate);
   } else if (abs_mode == 3) {
-    launch_vec(w.pdl, gemv_partial_kernel<K, 0, true>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS,
+    launch_vec(w.pdl, gemv_partial_kernel<K, 0, true>, grid, dim3(T), 0, st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS,
                gate);
   } else if (abs_mode == 0) {
-    launch_vec(w.pdl, gemv_partial_kernel<K, 0>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
+    launch_vec(w.pdl, gemv_partial_kernel<K, 0>, grid, dim3(T), 0, st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
   } else if (abs_mode == 1) {
-    launch_vec(w.pdl, gemv_partial_kernel<K, 1>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, w.a32, w.ld32, P, RS, gate);
+    launch_vec(w.pdl, gemv_partial_kernel<K, 1>, grid, dim3(T), 0, st, n, A, lda, X, ldx, chunk, w.a32, w.ld32, P, RS, gate);
   } else {
-    launch_vec(w.pdl, gemv_partial_kernel<K, 2>, grid, dim3(T), st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
+    launch_vec(w.pdl, gemv_partial_kernel<K, 2>, grid, dim3(T), 0, st, n, A, lda, X, ldx, chunk, nullptr, 0, P, RS, gate);
   }
   return cudaGetLastError();
 }
@@ -750,7 +740,8 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
   if (gemv_on_tensor_cores(n, K, A, lda, abs_mode, w, &split)) {
     // the digits live in the upper half of the row-sum scratch (fp64-sized; mode 1 keeps fp32 sums)
     void* prep = (char*)w.RS + round_up<size_t>(sizeof(float) * (size_t)gemv_chunks(n) * n, 256);
-    e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st, gate, live);
+    e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st, w.pdl, gate,
+                live);
   } else {
     switch (K) {
       case 1: e = gemv_k<1>(n, A, lda, X, ldx, abs_mode, w, nchunk, st, gate); break;
@@ -764,7 +755,7 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
     }
   }
   if (e != cudaSuccess) return e;
-  launch_vec(w.pdl, gemv_finish_kernel, dim3((unsigned)cdiv<int64_t>(n, kFinRows), K), dim3(kFinRows * kFinGroups), st,
+  launch_vec(w.pdl, gemv_finish_kernel, dim3((unsigned)cdiv<int64_t>(n, kFinRows), K), dim3(kFinRows * kFinGroups), 0, st,
              n, K, nchunk, w.P, B, ldb, out, ldo, X, ldx, abs_mode == 3 ? 0 : abs_mode, w.RS, w.st, track, split, gate,
              redo ? (const uint32_t*)w.status : nullptr, A, lda);
   prof_end(tok, abs_mode == 3 ? kProfGemv32 : kProfGemv, 8.0 * (double)n * (double)n, st);
@@ -814,16 +805,16 @@ struct Solver {
   void arnoldi_tail(int j, Gate gate) {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     if (n * K <= kFusedMgsMaxElems) {
-      launch_vec(w.pdl, arnoldi_tail_kernel, dim3(K), dim3(kFusedMgsThreads), st, sp, n, m, j, w.w, n, w.V, n,
+      launch_vec(w.pdl, arnoldi_tail_kernel, dim3(K), dim3(kFusedMgsThreads), 0, st, sp, n, m, j, w.w, n, w.V, n,
                  ldv_rhs(), w.st, w.brief);
       count_launches(1);
       return;
     }
     for (int i = 0; i <= j + 1; ++i)
-      launch_vec(w.pdl, mgs_kernel, dim3(red_blocks()), dim3(256), st, n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st,
+      launch_vec(w.pdl, mgs_kernel, dim3(red_blocks()), dim3(256), 0, st, n, K, m, j, i, w.w, n, w.V, n, ldv_rhs(), w.st,
                  w.partials, w.counter, gate);
-    launch_vec(w.pdl, givens_kernel, dim3(1), dim3(32), st, sp, j, w.st, w.brief);
-    launch_vec(w.pdl, scale_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), st, n, K, w.w, n,
+    launch_vec(w.pdl, givens_kernel, dim3(1), dim3(32), 0, st, sp, j, w.st, w.brief);
+    launch_vec(w.pdl, scale_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), 0, st, n, K, w.w, n,
                w.V + (int64_t)(j + 1) * n, ldv_rhs(), w.st, 1);
     count_launches(j + 4);
   }
@@ -854,9 +845,9 @@ struct Solver {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     const cudaError_t e = precond(w.r, n, w.tmp, n, ahead ? outer_gate() : Gate{});
     if (e != cudaSuccess) return e;
-    launch_vec(w.pdl, norm2_kernel, dim3(red_blocks()), dim3(256), st, n, K, w.tmp, n, w.st, w.partials, w.counter);
-    launch_vec(w.pdl, cycle_start_kernel, dim3(1), dim3(32), st, sp, w.st, w.brief);
-    launch_vec(w.pdl, scale_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), st, n, K, w.tmp, n, w.V,
+    launch_vec(w.pdl, norm2_kernel, dim3(red_blocks()), dim3(256), 0, st, n, K, w.tmp, n, w.st, w.partials, w.counter);
+    launch_vec(w.pdl, cycle_start_kernel, dim3(1), dim3(32), 0, st, sp, w.st, w.brief);
+    launch_vec(w.pdl, scale_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), 0, st, n, K, w.tmp, n, w.V,
                ldv_rhs(), w.st, 0);
     count_launches(3);
     return cudaGetLastError();
@@ -874,8 +865,8 @@ struct Solver {
   // x += V y
   cudaError_t cycle_finish() {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
-    launch_vec(w.pdl, cycle_finish_kernel, dim3(1), dim3(32), st, sp, w.st);
-    launch_vec(w.pdl, update_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), st, n, K, X, ldx, w.V, n,
+    launch_vec(w.pdl, cycle_finish_kernel, dim3(1), dim3(32), 0, st, sp, w.st);
+    launch_vec(w.pdl, update_kernel, dim3((unsigned)cdiv<int64_t>(n, 256)), dim3(256), 0, st, n, K, X, ldx, w.V, n,
                ldv_rhs(), w.st);
     count_launches(2);
     return cudaGetLastError();
@@ -885,7 +876,7 @@ struct Solver {
     const SolveParams sp{K, m, prm.max_iters, prm.inner_tol, prm.theta, prm.accept, n};
     const cudaError_t e = residual(n, K, A, lda, X, ldx, B, ldb, w.r, n, first ? 1 : 0, 1, w, st, {}, outer_gate());
     if (e != cudaSuccess) return e;
-    launch_vec(w.pdl, check_kernel, dim3(1), dim3(32), st, sp, w.st, w.brief, first ? 1 : 0);
+    launch_vec(w.pdl, check_kernel, dim3(1), dim3(32), 0, st, sp, w.st, w.brief, first ? 1 : 0);
     count_launches(1);
     return cudaGetLastError();
   }
@@ -981,7 +972,6 @@ hpmxp_status solve_ir(int64_t n, const double* A, int64_t lda, const void* LU, i
   s.B = b; s.ldb = ldb; s.X = x; s.ldx = ldx;
   s.prm = prm;
   s.w = carve_solve(ws, n, nrhs, prm.restart);
-  s.w.pdl = sm_budget() <= 0;   // under a budget the call shares the chip, as a batch's systems do
   // room for the fp32 copy of A after the workspace proper: the fp32 Arnoldi
   // products then read 4 instead of 8 bytes per entry
   if (prm.matvec_fp32 && ws_bytes >= s.w.bytes + solve_a32_bytes(n)) {

@@ -62,7 +62,10 @@ template <class T>
 __device__ inline T quotient(T s, T d, T r);   // s / d with r = 1 / d
 template <>
 __device__ inline float quotient<float>(float s, float d, float r) { return __fdiv_rn(s, d); }
-// one correction of s * r: the plain fp64 division costs about ten fp64 instructions
+// One correction of s * r: the plain fp64 division costs about ten fp64 instructions.  Correctly
+// rounded like it (while nothing underflows): d has at most 11 significant bits, so no quotient lies
+// within 2^-12 of its last place of a midpoint, r is rounded once, the remainder is exact, and the
+// corrected quotient before its rounding is off by about 2^-52 of that place.
 template <>
 __device__ inline double quotient<double>(double s, double d, double r) {
   const double q = s * r;
@@ -304,7 +307,6 @@ __global__ void __launch_bounds__(2 * kGrp) precond_kernel(PrecondArgs p) {
   constexpr int kR = sizeof(T) == 8 ? 1 : K <= 3 ? 4 : 2, kRB = sizeof(T) == 8 ? 2 : kR;
   constexpr int kQ = K * sizeof(T) <= 16 || (sizeof(T) == 8 && K <= 4) ? 4 : K % 2 == 0 || sizeof(T) == 8 ? 2 : 1;   // columns of a run
   constexpr int kUnroll = K * sizeof(T) <= 8 ? 4 : sizeof(T) == 4 || K == 2 ? 2 : 1;   // runs read ahead, against registers
-  pdl_trigger();   // every CTA is resident: the next kernel's may wait beside them
   if (p.gate.closed()) return;
   extern __shared__ __align__(16) unsigned char sm_raw[];
   __shared__ volatile int ready;   // owned blocks of the sweep whose updates are complete
@@ -382,6 +384,10 @@ __global__ void __launch_bounds__(2 * kGrp) precond_kernel(PrecondArgs p) {
     auto block_at = [&](int pos) { return sweep == 0 ? pos : nb - 1 - pos; };
     auto acc_of = [&](int o) { return acc + (size_t)(sweep == 0 ? o : nown - 1 - o) * TB * K; };
     unsigned long long* pub = p.pub + (size_t)sweep * nb * TB * K * W;
+    // every CTA is resident: the next kernel's may wait beside them, but not for both sweeps, since they
+    // take that long room from other streams' kernels (n = 8192, four right-hand sides, solved by two
+    // threads on their own streams: 2430 us a solve from the start on, 2280 from here; alone 3445 either way)
+    if (sweep == 1) pdl_trigger();
     if (tid == 0) ready = 0;
     __syncthreads();   // acc: the sweep's right-hand sides
     if (chain_group) {
