@@ -24,7 +24,8 @@
 // Roles: warp 0 TMA producer of the operand ring; warp 1 TMEM owner and MMA
 // issuer; warps 2..9 epilogue in two groups of four (warp w reads TMEM lanes
 // 32*(w%4)..+31; group g takes rows TI/2 g .. of the tile); warps 10 and 11
-// move the groups' C: loads ahead, stores behind, by 64-row segments.
+// move the groups' C: loads ahead, stores behind, by 64-row segments (where C has
+// one buffer; with three each group's first thread does).
 // Accumulators are double buffered in TMEM (single buffered for 4-slice FP8),
 // so the epilogue of one tile overlaps the MMAs of the next.  The E4M3
 // variant keeps one accumulator per 128-deep K slice and folds them with the
@@ -54,7 +55,6 @@ constexpr int kCBox = kTJ * 128;              // one C box: 128 bytes of rows x 
 constexpr int kEpiGroups = 2;                 // epilogue groups, one per half of the tile's rows
 constexpr int kEpiThreads = 128;              // threads per epilogue group (one warp per TMEM lane quarter)
 constexpr int kEpiWarps = kEpiThreads / 32;
-constexpr int kThreads = 64 + kEpiGroups * (kEpiThreads + 32);   // and one warp per group that moves its C
 
 // Tile height TI (output rows i per tile = MMA N): 128, or 256 for the large
 // 16-bit products, where every operand byte an SM receives feeds twice the
@@ -75,6 +75,9 @@ struct TileCfg {
   static constexpr int kCTile = kEpiGroups * kBoxes * kCBox;  // 32, 64 KiB (16-bit) or 64 KiB (fp32)
   // C tile buffers; the 256-row and the fp32 tiles have room for one only
   static constexpr int kCBufs = (TI == 128 && CB == 2) ? 3 : 1;
+  // who moves a group's C: a warp of its own, or with three buffers the group's first thread
+  static constexpr bool kMover = kCBufs == 1;
+  static constexpr int kThreads = 64 + kEpiGroups * (kEpiThreads + (kMover ? 32 : 0));
   static constexpr int kSegs = TI / 128;                    // 64-row segments of an epilogue group's TI/2 rows
   static constexpr int kSegBoxes = kBoxes / kSegs;          // C boxes of a segment
   static constexpr int kCSlots = kCBufs * kEpiGroups * kSegs;
@@ -89,6 +92,17 @@ static_assert(TileCfg<128>::kSmem <= 232448 && TileCfg<256>::kSmem <= 232448 && 
 template <int TI>
 constexpr bool tile_fits() { return 2 * TI <= 512 && TI <= 256 && TI % 128 == 0; }
 static_assert(tile_fits<128>() && tile_fits<256>(), "two accumulators in TMEM, one TMA box per stage");
+
+// Barrier of an epilogue group; true for all of its threads when v is true for all.
+__device__ inline bool epi_all(int group, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"((uint32_t)v), "r"(1 + group), "n"(kEpiThreads)
+      : "memory");
+  return r != 0;
+}
 
 // 64 consecutive fp32 columns: two x32 loads in flight, one wait.
 __device__ inline void tmem_ld64(uint32_t taddr, uint32_t (&r)[64]) {
@@ -174,7 +188,7 @@ struct TileLoc {
 };
 
 template <int TI, int CB, bool kPair>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(TileCfg<TI, CB, kPair>::kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                const __grid_constant__ CUtensorMap tmC, TcParams p, const GemmGroupItem* __restrict__ items,
                int nitems, const __grid_constant__ TcSecond second) {
@@ -311,6 +325,21 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     for (int r = 0; r < 2; ++r) store_at(smem_at(smem_u32(tmem_slot + 1 + which), (uint32_t)r), (int)pos);
   };
 
+  // segment h of group g's C of a tile, in buffer b: its boxes, rows, load and store
+  const bool load_c = p.has_c && p.mode == kEpiSub;
+  auto c_box = [&](int b, int g, int h, int k) { return sC + b * kCTile + (g * kBoxes + h * kSegBoxes + k) * kCBox; };
+  auto c_row = [&](int g, int h, int k) { return (TI / 2) * g + 64 * h + kBoxRows * k; };
+  auto load_c_seg = [&](const TileLoc& L, int b, int g, int h) {
+    mbar_expect_tx(c_full(b, g, h), kSegBoxes * kCBox);
+#pragma unroll
+    for (int k = 0; k < kSegBoxes; ++k)
+      tma_load_2d(c_box(b, g, h, k), L.c, L.i0 + c_row(g, h, k), L.j0, c_full(b, g, h));
+  };
+  auto store_c_seg = [&](const TileLoc& L, int b, int g, int h) {
+#pragma unroll
+    for (int k = 0; k < kSegBoxes; ++k) tma_store_2d(L.c, L.i0 + c_row(g, h, k), L.j0, c_box(b, g, h, k));
+  };
+
   if (warp == 0) {
     if (lane == 0) {
       long long pos = 0;
@@ -387,7 +416,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       if (!mbar_wait(mma_drain, 0)) atomicOr(p.status, kErrTimeout);
       if constexpr (kPair) report_end(2, pos);
     }
-  } else if (warp >= 2 + kEpiGroups * kEpiWarps) {
+  } else if (Cfg::kMover && warp >= 2 + kEpiGroups * kEpiWarps) {
     // C mover of group g: a segment's C is loaded ahead of the epilogue, and
     // stored and replaced by that of the buffer's next tile as soon as the
     // epilogue is done with that segment, so that the round trip (store read,
@@ -395,72 +424,48 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // leader moving whole tiles, the one buffer of a 256-row tile was the bound up
     // to a depth of 512: C -= A B of order 16384, depth 256: 324 -> 228 us, depth
     // 512: 316 -> 275 (what is left there is the operands' intake, 48 KB per 64
-    // of depth); order 28672, depth 512: 892 -> 880.
+    // of depth); order 28672, depth 512: 892 -> 880.  (With three buffers the trip
+    // is hidden anyway and the hop to the mover costs: see the epilogue.)
     if (lane == 0 && p.has_c) {
       const int g = warp - 2 - kEpiGroups * kEpiWarps;
-      const bool load_c = p.mode == kEpiSub;
-      int loading[kCBufs][kSegs];   // the phase of a load whose segment the epilogue has not finished, or -1
-      auto box = [&](int b, int h, int k) { return sC + b * kCTile + (g * kBoxes + h * kSegBoxes + k) * kCBox; };
-      auto row = [&](int h, int k) { return (TI / 2) * g + 64 * h + kBoxRows * k; };
-      auto arm = [&](const TileLoc& L, int b, int h, uint32_t phase) {
+      int loading[kSegs];   // the phase of a load whose segment the epilogue has not finished, or -1
+      auto arm = [&](const TileLoc& L, int h, uint32_t phase) {
         if (!load_c) {
-          mbar_arrive(c_full(b, g, h));
+          mbar_arrive(c_full(0, g, h));
           return;
         }
-        loading[b][h] = (int)phase;
-        mbar_expect_tx(c_full(b, g, h), kSegBoxes * kCBox);
-#pragma unroll
-        for (int k = 0; k < kSegBoxes; ++k)
-          tma_load_2d(box(b, h, k), L.c, L.i0 + row(h, k), L.j0, c_full(b, g, h));
+        loading[h] = (int)phase;
+        load_c_seg(L, 0, g, h);
       };
       acquire_maps(2);
 #pragma unroll
-      for (int b = 0; b < kCBufs; ++b) {
-        const int t = first() + b * stride();
-        TileLoc L{};
-        if (t < p.ntiles) L = locate(t);
-#pragma unroll
-        for (int h = 0; h < kSegs; ++h) {
-          loading[b][h] = -1;
-          if (t < p.ntiles) arm(L, b, h, 0);
-        }
+      for (int h = 0; h < kSegs; ++h) {
+        loading[h] = -1;
+        if (first() < p.ntiles) arm(locate(first()), h, 0);
       }
       bool ok = true;
-      int b = 0;
       uint32_t phase = 0;
-      for (int t = first(); t < p.ntiles && ok; t += stride()) {
+      for (int t = first(); t < p.ntiles && ok; t += stride(), phase ^= 1) {
         const TileLoc L = locate(t);
 #pragma unroll 1
         for (int h = 0; h < kSegs; ++h) {
-          if (!mbar_wait(c_done(b, g, h), phase, p.wait_polls, p.wait_ns)) { ok = false; break; }
-          loading[b][h] = -1;
-#pragma unroll
-          for (int k = 0; k < kSegBoxes && (!kPair || L.j0 < L.N); ++k) tma_store_2d(L.c, L.i0 + row(h, k), L.j0, box(b, h, k));
+          if (!mbar_wait(c_done(0, g, h), phase, p.wait_polls, p.wait_ns)) { ok = false; break; }
+          loading[h] = -1;
+          if (!kPair || L.j0 < L.N) store_c_seg(L, 0, g, h);
           bulk_commit();
-          if constexpr (kCBufs == 1) {
-            const int t2 = t + stride();
-            if (t2 < p.ntiles) {
-              asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-              arm(locate(t2), b, h, phase ^ 1);
-            }
-          } else {   // the buffer before this one, whose store has been read by now
-            const int t2 = t + (kCBufs - 1) * stride();
-            if (t != first() && t2 < p.ntiles) {
-              asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kSegs) : "memory");
-              if (b > 0) arm(locate(t2), b - 1, h, phase ^ 1);
-              else arm(locate(t2), kCBufs - 1, h, phase);
-            }
+          const int t2 = t + stride();
+          if (t2 < p.ntiles) {
+            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+            arm(locate(t2), h, phase ^ 1);
           }
         }
-        if (++b == kCBufs) { b = 0; phase ^= 1; }
       }
       bulk_wait0();
       if (!ok) {
         atomicOr(p.status, kErrTimeout);
         // C loads that the epilogue did not reach land before the CTA exits
-        for (int q = 0; q < kCBufs; ++q)
-          for (int h = 0; h < kSegs; ++h)
-            if (loading[q][h] >= 0) mbar_wait(c_full(q, g, h), (uint32_t)loading[q][h]);
+        for (int h = 0; h < kSegs; ++h)
+          if (loading[h] >= 0) mbar_wait(c_full(0, g, h), (uint32_t)loading[h]);
       }
     }
   } else {
@@ -470,6 +475,26 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     const int q = warp & 3;
     const int g = (warp - 2) >> 2;
     const int jl = 32 * q + lane;
+    // Three buffers: the group's first thread moves its C.  The C of the tile after next is loaded into
+    // the buffer of the tile before this one once this one's store has been issued, by when that store
+    // has been read, so that the group never waits for its own.  A warp that moves it instead costs
+    // these short tiles more than the group's barriers do (C = A B of order 16384, depth 128: 216 us
+    // with it, 181 without; C -= A B of order 24000: 517 and 501).
+    const bool leader = !Cfg::kMover && p.has_c && ((warp - 2) & 3) == 0 && lane == 0;
+    int loading[kCBufs];   // (leader) the phase of a load whose tile the group has not reached, or -1
+#pragma unroll
+    for (int b = 0; b < kCBufs; ++b) loading[b] = -1;
+    auto load_ahead = [&](int t, int b, int phase) {
+      if (!load_c || t >= p.ntiles) return;
+#pragma unroll
+      for (int k = 0; k < kCBufs; ++k) loading[k] = k == b ? phase : loading[k];
+      load_c_seg(locate(t), b, g, 0);
+    };
+    if (leader) {
+      acquire_maps(2);
+#pragma unroll
+      for (int b = 0; b < kCBufs - 1; ++b) load_ahead(first() + b * stride(), b, 0);
+    }
     bool ok = true;
     int local = 0;
     for (int t = first(); t < p.ntiles && ok; t += stride(), ++local) {
@@ -477,12 +502,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
       const int i0 = L.i0, j0 = L.j0;
       const int cb = local % kCBufs, ab = local % p.nbuf;
       const uint32_t cphase = (uint32_t)((local / kCBufs) & 1);
-      // a decision per warp (uniform for tcgen05.ld); a warp that gives up leaves its
-      // segment undone, which the mover's and the other waits run out on
-      ok = !p.has_c || mbar_wait(c_full(cb, g, 0), cphase, p.wait_polls, p.wait_ns);
+      // One decision per warp (uniform for tcgen05.ld); a warp that gives up leaves its segment undone,
+      // which the mover's and the other waits run out on.  Without a mover one per group, whose warps
+      // meet at its barriers; this one also says that the buffer's last store has been read.
+      ok = !(Cfg::kMover ? p.has_c : load_c) || mbar_wait(c_full(cb, g, 0), cphase, p.wait_polls, p.wait_ns);
       ok = ok && mbar_wait(acc_full(ab), (uint32_t)((local / p.nbuf) & 1), p.wait_polls, p.wait_ns);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = Cfg::kMover ? __all_sync(0xffffffffu, ok) : epi_all(g, ok);
       if (!ok) break;
+      if (leader) {
+#pragma unroll
+        for (int k = 0; k < kCBufs; ++k) loading[k] = k == cb ? -1 : loading[k];
+      }
       tc_fence_after();
       const uint32_t lane_base = tmem + (uint32_t)ab * p.acc_cols + ((uint32_t)(32 * q) << 16) + (TI / 2) * g;
       float sc[4] = {1.0f, 1.0f, 1.0f, 1.0f};
@@ -577,12 +607,30 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         }
         if (p.has_c) {
           fence_async_smem();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(c_done(cb, g, h));
+          if constexpr (Cfg::kMover) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(c_done(cb, g, h));
+          } else {
+            epi_all(g, true);
+            if (leader) {
+              store_c_seg(L, cb, g, 0);
+              bulk_commit();
+              asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+              const int ahead = local + kCBufs - 1;
+              load_ahead(t + (kCBufs - 1) * stride(), ahead % kCBufs, (ahead / kCBufs) & 1);
+            }
+          }
         }
       }
     }
     if (!ok && lane == 0) atomicOr(p.status, kErrTimeout);
+    if (leader) {
+      bulk_wait0();
+      // C loads that the group did not reach land before the CTA exits
+#pragma unroll
+      for (int b = 0; b < kCBufs; ++b)
+        if (loading[b] >= 0 && !mbar_wait(c_full(b, g, 0), (uint32_t)loading[b])) atomicOr(p.status, kErrTimeout);
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -746,7 +794,7 @@ cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st, const GemmArgs* al
   void* tok = prof_begin(st);
   p.span = prof_device_span(tok);
   const cudaError_t e =
-      launch_pdl_cluster(gemm_tc_kernel<TI, CB, kPair>, kPair ? 2 : 1, dim3(grid), dim3(kThreads), Cfg::kSmem, st, ta, tb, tc, p,
+      launch_pdl_cluster(gemm_tc_kernel<TI, CB, kPair>, kPair ? 2 : 1, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmem, st, ta, tb, tc, p,
                  (const GemmGroupItem*)nullptr, 0, second);
   prof_end(tok, g.mode == kEpiSub ? kProfGemm : kProfGemmStore, flops, st, bytes);
   count_launches(1);
@@ -827,7 +875,7 @@ cudaError_t gemm_tc_grouped(const GemmArgs& g, const GemmGroupItem* dev_items, i
   memset(&none, 0, sizeof(none));   // the items' maps are used instead
   void* tok = prof_begin(st);
   p.span = prof_device_span(tok);
-  const cudaError_t e = launch_pdl(gemm_tc_kernel<128, 2, false>, dim3(grid), dim3(kThreads), Cfg::kSmem, st, none, none,
+  const cudaError_t e = launch_pdl(gemm_tc_kernel<128, 2, false>, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmem, st, none, none,
                                    none, p, dev_items, nitems, TcSecond{});
   prof_end(tok, g.mode == kEpiSub ? kProfGemm : kProfGemmStore, flops, st, bytes);
   count_launches(1);
