@@ -87,8 +87,8 @@ __global__ void __launch_bounds__(kInvThreads) diag_inv_kernel(int64_t n, const 
   const int64_t base = (int64_t)c * TB;
   // the part of the block these columns need: rows and columns j0 .. 127 of L, 0 .. j0 + 31 of U
   const int lo = upper ? 0 : j0, hi = upper ? j0 + kInvCols : TB;
-  // 16-byte loads, all in flight; single values where the columns are not 16-byte aligned (and
-  // padded to 8 rows)
+  // 16-byte loads, all in flight; single values where the columns are not 16-byte aligned and for the
+  // last rows, which need not be padded (the last column's lie at the end of the array)
   uint4 raw[TB * TB / 8 / kInvThreads];
 #pragma unroll
   for (int q = 0; q < TB * TB / 8 / kInvThreads; ++q) {
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kInvThreads) diag_inv_kernel(int64_t n, const 
     raw[q] = make_uint4(0, 0, 0, 0);
     if (i + 8 > lo && i < hi && k >= lo && k < hi && base + k < n && base + i < n) {
       const uint16_t* src = LU + base + i + (base + k) * ld;
-      if (vec) {
+      if (vec && base + i + 8 <= n) {
         raw[q] = *reinterpret_cast<const uint4*>(src);
       } else {
         uint32_t w[8];
