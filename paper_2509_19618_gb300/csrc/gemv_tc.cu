@@ -678,7 +678,8 @@ bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, Gemv
   split->total = tiles * split->blocks;
   split->ctas = std::min(split->total, sm_count());
   // a tile meets at most this many CTAs' ranges
-  return cdiv(split->blocks, split->total / split->ctas) + 1 <= max_pieces;
+  split->most = cdiv(split->blocks, split->total / split->ctas) + 1;
+  return split->most <= max_pieces;
 }
 
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,

@@ -216,6 +216,7 @@ struct Gate {
 constexpr int kGemvTileRows = 512;
 struct GemvSplit {
   int blocks = 0, total = 0, ctas = 0;   // ctas 0: not split this way
+  int most = 0;                          // no tile has more pieces
   __host__ __device__ int begin(int cta) const { return (int)((long long)cta * total / ctas); }
   // the first range that holds part of tile's list [tile * blocks, (tile + 1) * blocks)
   __host__ __device__ int first_cta(int tile) const { return cta_of(tile * blocks); }

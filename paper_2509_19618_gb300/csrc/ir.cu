@@ -707,6 +707,10 @@ cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int
   return cudaGetLastError();
 }
 
+// The digits share the row-sum scratch (fp64, gemv_chunks(n) per row) with the fp32
+// row sums of the product's own pieces, which come first.
+size_t gemv_tc_row_sums(int64_t n, const GemvSplit& s) { return round_up<size_t>(sizeof(float) * (size_t)s.most * n, 256); }
+
 // Which products go to the tensor cores (gemv_tc.cu): fp64 ones that do not
 // also copy A to fp32, from the order at which two launches for X's digits and
 // 226 KB of shared memory per SM pay.  Both kernels timed, microseconds, digit
@@ -718,9 +722,9 @@ bool gemv_on_tensor_cores(int64_t n, int K, const double* A, int64_t lda, int ab
   const int64_t min_n = K == 1 ? 4096 : K < 6 ? 2048 : 1024;
   if (!(abs_mode == 0 || (abs_mode == 1 && !w.a32)) || n < min_n) return false;
   const size_t cap = (size_t)gemv_chunks(n);
-  if (round_up<size_t>(sizeof(float) * cap * n, 256) + gemv_tc_bytes(n) > sizeof(double) * cap * n) return false;
   GemvSplit s;
   if (!gemv_tc_split(n, A, lda, (int)cap, &s)) return false;
+  if (gemv_tc_row_sums(n, s) + gemv_tc_bytes(n) > sizeof(double) * cap * n) return false;
   *split = s;
   return true;
 }
@@ -738,8 +742,7 @@ cudaError_t residual(int64_t n, int K, const double* A, int64_t lda, const doubl
   void* tok = prof_begin(st);
   GemvSplit split;
   if (gemv_on_tensor_cores(n, K, A, lda, abs_mode, w, &split)) {
-    // the digits live in the upper half of the row-sum scratch (fp64-sized; mode 1 keeps fp32 sums)
-    void* prep = (char*)w.RS + round_up<size_t>(sizeof(float) * (size_t)gemv_chunks(n) * n, 256);
+    void* prep = (char*)w.RS + gemv_tc_row_sums(n, split);
     e = gemv_tc(n, K, A, lda, X, ldx, abs_mode == 1, prep, w.P, w.RS, split, w.status, st, w.pdl, gate,
                 live);
   } else {
