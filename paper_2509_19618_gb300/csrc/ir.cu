@@ -713,10 +713,11 @@ size_t gemv_tc_row_sums(int64_t n, const GemvSplit& s) { return round_up<size_t>
 
 // Which products go to the tensor cores (gemv_tc.cu): fp64 ones that do not
 // also copy A to fp32, from the order at which two launches for X's digits and
-// 226 KB of shared memory per SM pay.  Both kernels timed, microseconds, digit
-// products / fp64 FMAs: one right-hand side 30 / 26 at n = 2048, 53 / 57 at 4096,
-// 121 / 131 at 8192, 1570 / 1777 at 32768; two 34 / 25 at 1536, 31 / 35 at 2048,
-// 125 / 239 at 8192; six 35 / 38 at 1024; eight 155 / 885 at 8192, 1860 / 13800 at 32768.
+// up to 223 KB of shared memory per SM pay.  Whole residuals timed, microseconds,
+// digit products / fp64 FMAs: one right-hand side 51 / 50 at n = 4096, 67 / 71 at
+// 5120, 123 / 128 at 8192, 1580 / 1777 at 32768; two 28 / 27 at 2048, 40 / 45 at
+// 3072, 126 / 236 at 8192; four 33 / 43 at 2048; six 32 / 34 at 1024; eight 36 / 43 at
+// 1024, 158 / 885 at 8192, 1910 / 13800 at 32768.
 bool gemv_on_tensor_cores(int64_t n, int K, const double* A, int64_t lda, int abs_mode, const SolveWs& w,
                           GemvSplit* split) {
   const int64_t min_n = K == 1 ? 4096 : K < 6 ? 2048 : 1024;
@@ -891,7 +892,9 @@ struct Solver {
   // it is not.  Issuing the later steps ahead as well gained nothing: the step
   // after a cycle's last one costs 25 us (n = 1024) to 90 us with its gates
   // closed.  628 -> 574 us at n = 1024; 24 mixed systems in one batch 9.30 -> 8.83
-  // ms.  With the kernel timers on, nothing is issued ahead.
+  // ms.  Where x0 is accepted the closed cycle costs what the wait would have and
+  // more: 145 -> 168 us at n = 1024, 802 -> 828 at 4096 in fp64, 803 -> 854 at 8192
+  // with eight right-hand sides.  With the kernel timers on, nothing is issued ahead.
   cudaError_t run() {
     const bool ahead = !prof_on();
     auto report = [&] { return read_to_host(&rep, w.report, report_bytes(), st); };
