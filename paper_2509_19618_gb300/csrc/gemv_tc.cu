@@ -41,8 +41,8 @@
 // are fp64 FMAs, taken from the same stages (a second, direct read of A made
 // matrices with zero blocks, whose rows have no E there, and unlike right-hand
 // sides up to 2 times slower than gemv_partial_kernel).  Zero entries are skipped:
-// n = 16384, four right-hand sides, lower triangular 2740 -> 471 us, unlike
-// right-hand sides 2350 -> 1780 (the FMA kernel 1755).
+// n = 16384, four right-hand sides, lower triangular 2740 -> 440 us, unlike
+// right-hand sides 2350 -> 1800 (the FMA kernel 1755).
 //
 // Layout: a CTA takes 512 rows, four groups of 128 threads (thread = row, TMEM
 // lane), by 64-column blocks.  A's columns come by TMA (16 columns x 128 rows per
@@ -52,10 +52,10 @@
 // buffers that the groups share.  A thread cuts its row's digits with integer
 // instructions and stores them to TMEM (the MMA's A operand).  Slice s adds to D's
 // columns 8 (s + u) + r of the block's 64.  Bound by the integer pipe (half the
-// issue rate) and the group's barriers; with seven digits 34 instructions per
-// entry, 17 of them integer (56 % busy), and the eighth costs 5 %: 432 -> 458 us at
-// n = 16384 with four right-hand sides, 1.49 -> 1.58 ms at 32768 with one (5.4 TB/s
-// of A), against 1.76 and 1.78 ms of fp64 FMAs.
+// issue rate, about 18 of 36 instructions per entry) and the group's barriers: 425 us
+// at n = 16384 with four right-hand sides, 1.46 ms at 32768 with one (5.9 TB/s of A),
+// against 1.76 and 1.78 ms of fp64 FMAs.  (432 and 1.49 with seven digits and all MMAs
+// issued on one scheduler, 458 and 1.58 with eight.)
 #include "tcgen05.h"
 
 #include <cuda_fp16.h>
@@ -271,6 +271,9 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
   volatile uint32_t* dead = slot + 1;   // a wait ran out: no further waits (the results are void, the call reports it)
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = warp >> 2, tg = tid & (kRowsT - 1);
+  // A group's MMAs and its loads are issued by one thread each, in another warp in each group: warps 0 of
+  // all groups share a scheduler, and with their MMAs all issued there the product took 8 % longer
+  const int mma_thread = 32 * g, load_thread = 32 * ((g + 2) & 3);
   const uint32_t bar0 = smem_u32(bars);
   auto b_full = [&](int b) { return bar0 + 8u * (uint32_t)b; };
   auto b_empty = [&](int b) { return bar0 + 8u * (uint32_t)(kBBufs + b); };
@@ -322,7 +325,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
     const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
     const uint32_t ta = tmem + kTmA * g, td = tmem + kTmD + 64 * g;
     uint32_t apos = 0, bpos = 0, issued = 0;   // stages and digit buffers used, commits
-    uint32_t a_loads = 0, b_loads = 0;         // next uses to load (thread tg == 32)
+    uint32_t a_loads = 0, b_loads = 0;         // next uses to load (load_thread)
     uint32_t fills_a[kStages] = {}, fills_b[kBBufs] = {};   // loads issued into each
     // A is read once: its lines leave L2 first, and the factors and inverses that the
     // preconditioner reads next stay
@@ -332,7 +335,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
 #pragma unroll
       for (int i = 0; i < (int)(sizeof(f) / sizeof(f[0])); ++i) f[i] += i == k;
     };
-    // columns of stage use q (of thread tg == 32) and digits of block use q (of group 0's)
+    // columns of stage use q (of load_thread) and digits of block use q (of group 0's)
     auto load_a = [&](uint32_t q) {
       const int lw = w0 + (int)((q - a0) / (kBlk / kCols));
       if (lw >= wend || *dead) return;
@@ -363,7 +366,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
     wend = p.split.begin(range + 1);
     a0 = apos;
     b0 = bpos;
-    if (tg == 32) {
+    if (tg == load_thread) {
       for (a_loads = a0; a_loads < a0 + kStages; ++a_loads) load_a(a_loads);
       if (g == 0 && !plain)
         for (b_loads = b0; b_loads < b0 + kBBufs - 1; ++b_loads) load_b(b_loads);
@@ -460,7 +463,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
           fp64_stage(reinterpret_cast<const double*>(ring + (g * kStages + st) * kStage) + tg, exps, (int64_t)q * kCols, true,
                      true);
           group_barrier(g);
-          if (tg == 32) load_a(a_loads++);
+          if (tg == load_thread) load_a(a_loads++);
         }
         kb0 = kb1;
       }
@@ -576,7 +579,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
           asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           tc_fence_before();
           group_barrier(g);
-          if (tg == 0) {
+          if (tg == mma_thread) {
             tc_fence_after();
             const uint32_t bd = digits_at(bb) + 32 * sub;
 #pragma unroll
@@ -587,7 +590,7 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
                         make_idesc(0, 64 - 16 * (s / 2)), sub > 0 || s > 0);
             if (sub == 3) tc_commit(b_empty(bb));
             tc_commit(bar_mma);   // the last one, which the drain below waits for
-          } else if (tg == 32) {   // every thread of the group has read this stage
+          } else if (tg == load_thread) {   // every thread of the group has read this stage
             load_a(a_loads++);
             if (g == 0 && sub == 2) load_b(b_loads++);
           }
@@ -624,11 +627,11 @@ __global__ void __launch_bounds__(kThr, 1) gemv_tc_kernel(const __grid_constant_
     // Where a wait ran out, several commits can be open, and bar_mma's parity is that of the one before
     // the last as well: the issuing thread commits once more, to a barrier used for nothing else.  (If it
     // does not see the flag, each of its own waits ended before its next MMAs, and one commit at most was open.)
-    if (tg == 0 && issued && *dead) {
+    if (tg == mma_thread && issued && *dead) {
       tc_commit(bar_drain);
       if (!mbar_wait(bar_drain, 0)) atomicOr(p.status, kErrTimeout);
     }
-    if (tg == 32 && *dead) {
+    if (tg == load_thread && *dead) {
       for (int s = 0; s < kStages; ++s)
         if (fills_a[s] && !mbar_wait(a_full(g, s), (fills_a[s] - 1) & 1)) atomicOr(p.status, kErrTimeout);
       for (int b = 0; b < kBBufs; ++b)
@@ -678,8 +681,7 @@ bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, Gemv
   split->total = tiles * split->blocks;
   split->ctas = std::min(split->total, sm_count());
   // a tile meets at most this many CTAs' ranges
-  split->most = cdiv(split->blocks, split->total / split->ctas) + 1;
-  return split->most <= max_pieces;
+  return most_of(*split) <= max_pieces;
 }
 
 cudaError_t gemv_tc(int64_t n, int K, const double* A, int64_t lda, const double* X, int64_t ldx, bool abs_sums,

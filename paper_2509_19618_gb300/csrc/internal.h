@@ -216,7 +216,6 @@ struct Gate {
 constexpr int kGemvTileRows = 512;
 struct GemvSplit {
   int blocks = 0, total = 0, ctas = 0;   // ctas 0: not split this way
-  int most = 0;                          // no tile has more pieces
   __host__ __device__ int begin(int cta) const { return (int)((long long)cta * total / ctas); }
   // the first range that holds part of tile's list [tile * blocks, (tile + 1) * blocks)
   __host__ __device__ int first_cta(int tile) const { return cta_of(tile * blocks); }
@@ -230,6 +229,7 @@ struct GemvSplit {
 // The split for order n; false where a tile could meet more than max_pieces
 // ranges, or A's columns are not 16-byte aligned.
 bool gemv_tc_split(int64_t n, const double* A, int64_t lda, int max_pieces, GemvSplit* split);
+inline int most_of(const GemvSplit& s) { return cdiv(s.blocks, s.total / s.ctas) + 1; }
 // P[c][r][i] = the partial sums of row i in its tile's piece c; with abs_sums
 // also RS[c][i], the fp32 estimates of the |A| row sums.  prep: gemv_tc_bytes(n)
 // of scratch, 16-byte aligned.  live: the right-hand sides whose sums are wanted,

@@ -709,15 +709,15 @@ cudaError_t gemv_k(int64_t n, const double* A, int64_t lda, const double* X, int
 
 // The digits share the row-sum scratch (fp64, gemv_chunks(n) per row) with the fp32
 // row sums of the product's own pieces, which come first.
-size_t gemv_tc_row_sums(int64_t n, const GemvSplit& s) { return round_up<size_t>(sizeof(float) * (size_t)s.most * n, 256); }
+size_t gemv_tc_row_sums(int64_t n, const GemvSplit& s) { return round_up<size_t>(sizeof(float) * (size_t)most_of(s) * n, 256); }
 
 // Which products go to the tensor cores (gemv_tc.cu): fp64 ones that do not
 // also copy A to fp32, from the order at which two launches for X's digits and
 // up to 223 KB of shared memory per SM pay.  Whole residuals timed, microseconds,
-// digit products / fp64 FMAs: one right-hand side 51 / 50 at n = 4096, 67 / 71 at
-// 5120, 123 / 128 at 8192, 1580 / 1777 at 32768; two 28 / 27 at 2048, 40 / 45 at
-// 3072, 126 / 236 at 8192; four 33 / 43 at 2048; six 32 / 34 at 1024; eight 36 / 43 at
-// 1024, 158 / 885 at 8192, 1910 / 13800 at 32768.
+// digit products / fp64 FMAs: one right-hand side 47 / 50 at n = 4096, 61 / 70 at
+// 5120, 112 / 127 at 8192, 1460 / 1787 at 32768; two 27.5 / 26.4 at 2048, 38 / 45 at
+// 3072, 116 / 236 at 8192; four 32 / 43 at 2048; six 32 / 34 at 1024; eight 36 / 43 at
+// 1024, 150 / 890 at 8192, 1820 / 13800 at 32768.
 bool gemv_on_tensor_cores(int64_t n, int K, const double* A, int64_t lda, int abs_mode, const SolveWs& w,
                           GemvSplit* split) {
   const int64_t min_n = K == 1 ? 4096 : K < 6 ? 2048 : 1024;
