@@ -233,7 +233,10 @@ void hpmxp_ir_params_default(hpmxp_ir_params* p);
  *   b        in, n x nrhs fp64, ldb >= n
  *   x        out, n x nrhs fp64, ldx >= n; holds the last iterate even on failure
  *   nrhs     1..8 right-hand sides, refined together (one pass over A and LU per
- *            iteration serves all of them)
+ *            iteration serves all of them).  Each decides its own cycles; the fp64
+ *            products of larger orders round at a common exponent per column of A, so
+ *            that the last bits of one x can depend on the others of the call, with
+ *            errors below those of fp64 FMAs; zero and finished ones have no part
  *   prm      host, NULL for the defaults
  *   info     host, nrhs entries (may be NULL)
  *   ws       scratch of hpmxp_solve_workspace(n, nrhs, restart) bytes
@@ -266,10 +269,10 @@ hpmxp_status hpmxp_solve_ir_scaled(int64_t n, const double* A, int64_t lda, cons
  * Each hpmxp_problem names one system's caller-owned device buffers.  The
  * batched calls run all systems in lockstep with Schur-update depth 128: one
  * grouped launch per stage serves every system that is still active (one CTA
- * per system's diagonal block; one tensor-core launch walking all systems'
- * tiles for each of the row-panel, column-panel and Schur products), so a
- * batch of B systems of order up to N takes about 5 N / 128 launches instead
- * of 5 sum_b n_b / 128.  Each system's factors are bit-for-bit those of
+ * per system's diagonal block's LU, 40 for its inverses; one tensor-core launch
+ * walking all systems' tiles for both panels' products, one for the Schur
+ * updates), so a batch of B systems of order up to N takes about 5 N / 128
+ * launches instead of 5 sum_b n_b / 128.  Each system's factors are bit-for-bit those of
  * hpmxp_factor(n_b, ..., nb = 128) of it alone (the same kernels compute every
  * tile).  Formats: HPMXP_BF16 and HPMXP_FP16. */
 typedef struct {

@@ -63,8 +63,8 @@ constexpr int kEpiWarps = kEpiThreads / 32;
 // trailing matrix: C = fl32(C - acc), 128-row tiles only).
 // kPair: a cluster of two CTAs makes a tile of 256 rows and 256 columns, each
 // its own 128 columns of the accumulator; each stages 128 of the rows i, so that
-// an SM receives 32 instead of 48 KB per 64 of depth (942 -> 1157 TFLOP/s at
-// order 28672, depth 512; the n = 32768 factorization 36.7 -> 32.8 ms).
+// an SM receives 32 instead of 48 KB per 64 of depth (953 -> 1182 TFLOP/s at
+// order 28672, depth 512; the n = 32768 factorization 36.7 -> 32.1 ms).
 template <int TI, int CB = 2, bool kPair = false>
 struct TileCfg {
   static constexpr int kStages = kPair ? 5 : TI == 128 ? 4 : 3;
@@ -794,8 +794,8 @@ cudaError_t gemm_tc_tiles(const GemmArgs& g, cudaStream_t st, const GemmArgs* al
   void* tok = prof_begin(st);
   p.span = prof_device_span(tok);
   const cudaError_t e =
-      launch_pdl_cluster(gemm_tc_kernel<TI, CB, kPair>, kPair ? 2 : 1, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmem, st, ta, tb, tc, p,
-                 (const GemmGroupItem*)nullptr, 0, second);
+      launch_pdl_cluster(gemm_tc_kernel<TI, CB, kPair>, kPair ? 2 : 1, dim3(grid), dim3(Cfg::kThreads), Cfg::kSmem,
+                         st, ta, tb, tc, p, (const GemmGroupItem*)nullptr, 0, second);
   prof_end(tok, g.mode == kEpiSub ? kProfGemm : kProfGemmStore, flops, st, bytes);
   count_launches(1);
   return e;

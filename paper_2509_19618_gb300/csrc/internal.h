@@ -153,7 +153,7 @@ bool encode_f64_map(CUtensorMap* tm, const double* base, int64_t rows, int64_t c
                     int box_cols);
 // Grouped launches of the tensor-core engine: several independent products of
 // the same kind (same mode, sign, format and K, 16-bit operands, K < 256 so
-// all take 128-row tiles, R given for all or none) in ONE launch, the
+// all take 128-row tiles; with or without R each) in ONE launch, the
 // persistent CTAs walking the concatenated tile lists.  One item per product,
 // in device memory (its tensor maps are read from there by the TMA unit).
 struct alignas(128) GemmGroupItem {
