@@ -27,10 +27,10 @@
 // row's largest product for one right-hand side and, since E follows columns whose
 // x_jr differ by 2^6 at most, 2^-50 of a side's own largest for several; the signs
 // differ from column to column.  The plain kernel rounds every partial sum at
-// 2^-53.  With seven digits on both sides a
-// Gaussian A with a dominant diagonal was 1.5 to 2.3 times less accurate than the
-// plain kernel (rms, n = 2048, two right-hand sides), rows whose largest products
-// cancel 16 to 21 times; with eight 0.006 and 0.08.
+// 2^-53.  With seven digits on both sides a Gaussian A with a dominant diagonal was
+// 1.5 to 2.3 times less accurate than the plain kernel (rms, n = 2048, two
+// right-hand sides), rows whose largest products cancel 16 to 21 times; with eight
+// digits the errors are 0.006 and 0.08 of the plain kernel's.
 //
 // An entry above 2^E (a diagonally dominant row's diagonal; a non-finite
 // entry, whose exponent exceeds every E in use) has no digits: its product is
